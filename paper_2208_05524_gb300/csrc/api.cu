@@ -17,6 +17,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "tree.cuh"
 #include "vesis.h"
 #include "vesis_internal.cuh"
 
@@ -230,6 +231,10 @@ struct vesis_system_t {
     int nb_terms = 0;
     ForcePlan fplan{}, fplan_far{};
     int pe_pts = 8;             // cells per thread of the energy kernel (4 or 8)
+    bool tree = false;          // hierarchical fields, and gradient (rules on the sizes,
+    bool tree_force = false;    // decided at set-up)
+    TreePlan tplan{};
+    uint8_t *d_tree = nullptr;  // their workspace
     SweepGate *gate = nullptr;  // set while a batched relaxation runs
     double *d_fpart = nullptr;
     double *d_grad_solv = nullptr, *d_grad_ss = nullptr, *d_grad = nullptr;
@@ -401,6 +406,31 @@ void enq_pack(vesis_system s, const double *d_pos)
                       s->d_oob, s->d_geo + 3, s->d_geo + 6, s->st);
 }
 
+// U and E on the grid at the packed positions.  Large solutes take the
+// hierarchical sums; the direct kernel's pencil length is a choice of the
+// others.
+void enq_pair_energy(vesis_system s, float *U, float *E, int pts)
+{
+    if (s->tree)
+        launch_tree_fields(s->g, s->tplan, s->d_tree, atoms_view(s), (float)s->p.rho_w,
+                           (float)s->cfa, s->rmin2, U, E, E + s->G, E + 2 * s->G, s->st);
+    else
+        launch_pair_energy_grid(s->g, atoms_view(s), (float)s->p.rho_w, (float)s->cfa, s->rmin2,
+                                U, E, E + s->G, E + 2 * s->G, pts, s->st);
+}
+
+// Grid part of the atom gradient into d_grad_solv.
+void enq_pair_force(vesis_system s, const ForcePlan &fp, const uint8_t *chi, const float *E)
+{
+    if (s->tree_force)
+        launch_tree_force(s->g, s->tplan, s->d_tree, atoms_view(s), fp.cg, chi, E, E + s->G,
+                          E + 2 * s->G, s->rmin2, s->d_fpart, s->h3, s->d_grad_solv, s->d_fcount,
+                          s->st);
+    else
+        launch_pair_force_grid(s->g, fp, chi, E, E + s->G, E + 2 * s->G, atoms_view(s), s->rmin2,
+                               s->d_fpart, s->d_fcount, s->st);
+}
+
 // Far-field energy and node fields at the packed positions.
 void enq_far(vesis_system s, double *bk)
 {
@@ -417,9 +447,7 @@ void enq_far(vesis_system s, double *bk)
 void enq_fields(vesis_system s, float *U, float *E, double *bk)
 {
     const int sp = span_begin(s);
-    launch_pair_energy_grid(s->g, atoms_view(s), (float)s->p.rho_w,
-                            (float)s->cfa, s->rmin2, U, E, E + s->G,
-                            E + 2 * s->G, s->pe_pts, s->st);
+    enq_pair_energy(s, U, E, s->pe_pts);
     span_end(s, sp, 0, s->G * (long long)s->n, 0);
     enq_far(s, bk);
 }
@@ -536,12 +564,10 @@ void enq_gradient(vesis_system s, const uint8_t *chi, const float *E,
                   const double *d_pos, double *bk, bool ss_current = false)
 {
     const int sp = span_begin(s);
-    launch_pair_force_grid(s->g, s->fplan, chi, E, E + s->G, E + 2 * s->G,
-                           atoms_view(s), s->rmin2, s->d_fpart, s->d_fcount,
-                           s->st);
+    enq_pair_force(s, s->fplan, chi, E);
     span_end(s, sp, 1, 0, 0);
-    launch_force_reduce(s->d_fpart, s->fplan.nchunk, s->n, s->h3,
-                        s->d_grad_solv, 0, s->st);
+    if (!s->tree_force)
+        launch_force_reduce(s->d_fpart, s->fplan.nchunk, s->n, s->h3, s->d_grad_solv, 0, s->st);
     if (s->nfar > 0) {
         launch_point_force(s->d_far_pts, s->d_far_wf, s->nfar, s->d_far_UE,
                            s->fplan_far, atoms_view(s), s->rmin2, s->d_fpart,
@@ -926,7 +952,19 @@ static int init_impl(vesis_system s, const vesis_params *p, int n,
     // gradient partials
     s->fplan = plan_pair_force(G, n, s->nsm, 4);
     s->fplan_far = plan_point_force(std::max(1, s->nfar), n, s->nsm);
-    const long long nch = std::max(s->fplan.nchunk, s->fplan_far.nchunk);
+    long long nch = std::max(s->fplan.nchunk, s->fplan_far.nchunk);
+    const double max_sigma = *std::max_element(sigma_sw, sigma_sw + n);
+    s->tree = tree_fields_pay(s->g, n, p->h, p->r_min, max_sigma);
+    s->tree_force = tree_force_pays(s->g, n, p->h, p->r_min, max_sigma);
+    if (s->tree) {
+        s->tplan = plan_tree(s->g, n, s->nsm);
+        VTRY(dalloc(s, &s->d_tree, s->tplan.bytes));
+        std::vector<uint8_t> tab(tree_tab_bytes());
+        tree_fill_tab(tab.data());
+        VCK(cudaMemcpy(s->d_tree + s->tplan.o_tab, tab.data(), tab.size(),
+                       cudaMemcpyHostToDevice));
+        if (s->tree_force) nch = std::max<long long>(nch, s->tplan.part_slots);
+    }
     VTRY(dalloc(s, &s->d_fpart, (size_t)nch * n * 3));
     VTRY(dalloc(s, &s->d_grad_solv, 3 * n));
     VTRY(dalloc(s, &s->d_grad_ss, 3 * n));
@@ -1687,15 +1725,13 @@ int vesis_autotune(vesis_system s, const uint8_t *chi_dev, int reps, double *tim
     for (int v = 0; v < 3; ++v) {
         const int P = kPencil[v];
         VTRY(timed([&] {
-            launch_pair_energy_grid(s->g, atoms_view(s), (float)s->p.rho_w, (float)s->cfa,
-                                    s->rmin2, U, E, E + s->G, E + 2 * s->G, P, s->st);
+            enq_pair_energy(s, U, E, P);
         }, &ms[v]));
     }
     for (int v = 0; v < 2; ++v) {
         const ForcePlan fp = plan_pair_force(s->G, s->n, s->nsm, kAtoms[v]);
         VTRY(timed([&] {
-            launch_pair_force_grid(s->g, fp, chi_dev, E, E + s->G, E + 2 * s->G,
-                                   atoms_view(s), s->rmin2, s->d_fpart, s->d_fcount, s->st);
+            enq_pair_force(s, fp, chi_dev, E);
         }, &ms[3 + v]));
     }
     VTRY(last_launch("autotune"));
