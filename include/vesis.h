@@ -263,8 +263,8 @@ int vesis_blsm_relax(vesis_system s, uint8_t *chi_dev, const float *U_dev,
  * flips, flipped cells and FP64 sum of their dE.  Every system's stream is
  * waited for; the work runs on systems[0]'s stream, and the call returns
  * when it is done.  Returns VESIS_W_MAX_ROUNDS if the cap stopped any
- * system.  Device scratch for the launch (about 300 bytes per system) is
- * allocated and freed by the call. */
+ * system.  Device scratch for the launch (about 500 bytes per system and half
+ * a byte per 8^3 tile) is allocated and freed by the call. */
 int vesis_blsm_relax_batch(int nsys, vesis_system *systems, uint8_t *const *chi_dev,
                            const float *const *U_dev, int max_rounds, int *rounds_out,
                            long long *flips_out, double *dE_sum_out);
@@ -312,10 +312,10 @@ int vesis_relax(vesis_system s, uint8_t *chi_dev, double *xyz_inout,
  * vesis_blsm_relax and of the interface relaxations inside vesis_relax)
  * runs as one cooperative launch whose blocks meet at a grid barrier twice
  * per round.  A block that has polled the barrier `polls` times without
- * seeing it complete (each poll an L2 load plus a 32 ns sleep) raises the
- * sweep's error flag and returns, and so does every other block at its
- * next barrier; the call then returns VESIS_E_CUDA with the message "flip
- * sweep grid barrier timed out".  The labels passed in are then partly
+ * seeing it complete (each poll one L2 load) raises the sweep's error flag
+ * and returns, and so does every other block at its next barrier; the call
+ * then returns VESIS_E_CUDA with the message "flip sweep grid barrier timed
+ * out".  The labels passed in are then partly
  * relaxed and must be reset by the caller; the system stays usable, and
  * the next call starts its sweep state afresh.  Default 2^24 polls (seconds
  * of waiting: only a hung block reaches it).  polls >= 0; 0 gives up at the
@@ -329,8 +329,8 @@ int vesis_set_wait_limit(vesis_system s, long long polls);
  * leader word in the previous round keeps its previous verdict (it lost)
  * and need not be decided again; the updates stamp the tiles whose
  * neighbourhood changed.  mode -1 (the default): stamps are written while
- * the tiles holding a leader outnumber the sweep's warps, and read by a
- * block whose own leader tiles outnumber its warps; 0: never (every tile
+ * the half tiles holding a leader outnumber the sweep's warps, and read by a
+ * block whose own leader halves outnumber its warps; 0: never (every tile
  * holding a leader is decided every round); 1: always.  The rounds,
  * flips, labels and energies are identical in every mode; only the time
  * differs.  Applies to later vesis_blsm_relax, vesis_relax and (through

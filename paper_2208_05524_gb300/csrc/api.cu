@@ -266,7 +266,7 @@ struct vesis_system_t {
     unsigned long long *d_part_flips = nullptr;
     double *d_part_dE = nullptr;
     unsigned long long *d_part_tiles = nullptr;
-    double *d_tile_dE = nullptr;      // multi-system sweep: per-tile dE sums
+    double *d_tile_dE = nullptr;      // multi-system sweep: dE sums per half tile
     unsigned *d_tile_nf = nullptr;    // and flip counts
 
     double *d_scal = nullptr;   // two banks of S_BANK doubles
@@ -993,8 +993,8 @@ static int init_impl(vesis_system s, const vesis_params *p, int n,
     VTRY(dalloc(s, &s->d_part_flips, s->sweep_blocks));
     VTRY(dalloc(s, &s->d_part_dE, s->sweep_blocks));
     VTRY(dalloc(s, &s->d_part_tiles, 2 * (size_t)s->sweep_blocks));
-    VTRY(dalloc(s, &s->d_tile_dE, (size_t)s->ntiles));
-    VTRY(dalloc(s, &s->d_tile_nf, (size_t)s->ntiles));
+    VTRY(dalloc(s, &s->d_tile_dE, (size_t)2 * s->ntiles));
+    VTRY(dalloc(s, &s->d_tile_nf, (size_t)2 * s->ntiles));
 
     VTRY(dalloc(s, &s->d_scal, 2 * S_BANK));
     VTRY(dalloc(s, &s->d_rs, 1));
@@ -1238,7 +1238,9 @@ int vesis_blsm_relax_batch(int nsys, vesis_system *systems, uint8_t *const *chi_
         y.st = s->st;
     }
     void *scratch = nullptr;
-    VCK(cudaMalloc(&scratch, sweep_multi_scratch_bytes(nsys)));
+    long long tiles = 0;
+    for (int i = 0; i < nsys; ++i) tiles += systems[i]->ntiles;
+    VCK(cudaMalloc(&scratch, sweep_multi_scratch_bytes(nsys, tiles)));
     struct Free {
         void *p;
         ~Free() { cudaFree(p); }

@@ -22,35 +22,51 @@
 // zero for a brick without one (PL, one word per brick).
 //
 // Round k:
-//   decide (one warp per tile holding a leader): the words of the 6^3
-//     bricks around the tile arrive together; each of the tile's leaders is
-//     tested against every other leader within r.  A winner flips its label
-//     and adds its dE, and posts itself to every tile within r of it: a
-//     16-bit entry (cell within its brick, old label) in the slot of its
-//     brick among the 6^3 bricks that tile can see, plus the slot's bit.
+//   decide (a team of two warps per tile holding a leader): the words of the
+//     6^3 bricks around the tile arrive together, four per thread; the
+//     non-zero ones go to shared memory, and each warp tests its half of the
+//     tile's leaders against them.  A winner flips its label and adds its dE,
+//     and posts itself to every tile within r of it: a 16-bit entry (cell
+//     within its brick, old label) in the slot of its brick among the 6^3
+//     bricks that tile can see, the slot's bit, and the tile's bit in its
+//     owner's update bitmap.
 //   grid barrier
-//   update (one warp per tile that received a winner): W of the tile's own
-//     cells gets +-q_a q_b q_c from each posted winner whose window covers
-//     them (W stays the exact convolution, and only the warp visiting the
-//     tile writes its cells), then the tile's candidates, their dE and its
-//     leaders are recomputed.  Tiles no winner reached keep their leaders.
+//   update (a team per tile that received a winner, a warp per half of 4 x 8
+//     rows of 8 cells, a row per thread): W of the tile's own cells gets +-q_a
+//     q_b q_c from each posted winner whose window covers them (W stays the
+//     exact convolution, and only the team visiting the tile writes its
+//     cells), then the half's candidates, their dE and its leaders are
+//     recomputed.  Tiles no winner reached keep their leaders.
 //   grid barrier
 // The sweep stops when no tile holds a leader or after max_rounds rounds.
 // An opening pass computes every tile's leaders from the starting labels.
+//
+// A round is bound by latency: two grid barriers (1.6 us each) and, in each
+// phase, the chain from a tile's loads to its stores, which teams sharing an
+// SM stretch for one another through the instructions they issue.  A half
+// tile per warp keeps a tile's two warps apart but for one barrier: the
+// bricks, their leaders and the verdicts on them are a warp's own.  Measured
+// with eight teams per block, one block per SM (us per round, before = one
+// warp per tile, 32 per block; two atoms in 128^3, 112^3 small solute, 256^3
+// protein, 384^3 complex): 12.5, 12.4, 14.3, 29.8 before; 7.4, 8.0, 11.0, 22.4
+// now; teams of four warps 9.4, 9.4, 12.0, 26.4; four teams per block 7.4,
+// 8.8, 12.5, 29.5; twelve (80 registers a thread, spilling) 9.5, 9.9, 11.5,
+// 23.7; 76 blocks instead of 152 11.1 for the 112^3 solute; one cluster of 16
+// blocks with its barriers in shared memory 16.4 there.
 //
 // Only tiles whose verdict can change are decided: a leader's verdict is a
 // function of the leader words within r of it, all inside the 27 tiles
 // around its own, so a tile none of whose 27 neighbours (itself included)
 // changed a leader word in the last update keeps its last verdict - it
 // lost (a winner changes its own tile's words) - and is skipped.  Every
-// update that changes one of the tile's words stamps its 27 neighbours with
-// the next round; round 0 decides every tile.  The winners, and so the
-// rounds and labels, are those of deciding every tile every round.  The
-// stamps only pay where warps have several tiles: the updates write them
-// while the tiles holding a leader outnumber the grid's warps (a count all
-// blocks read alike), and a block reads them only after such an update and
-// when its own leader tiles outnumber its warps (deciding an unstamped tile
-// is harmless).
+// update that changes one of the tile's words stamps its 27 neighbours (a
+// bit in the owner's stamp bitmap, read and cleared by the next decide);
+// round 0 decides every tile.  The winners, and so the rounds and labels,
+// are those of deciding every tile every round.  The stamps only pay where
+// teams have several tiles: the updates write them while the half tiles
+// holding a leader outnumber the grid's warps (a count all blocks read alike),
+// and a block reads them only after such an update and when its own leader
+// halves outnumber its warps (deciding an unstamped tile is harmless).
 //
 // The grid barrier spins with a bound; on timeout it raises an error flag
 // and every block returns.
@@ -61,12 +77,12 @@
 namespace vesis {
 
 constexpr int TS = 8;             // tile edge
-#ifndef VESIS_SWEEP_THREADS
-#define VESIS_SWEEP_THREADS 512
-#endif
-constexpr int SW_THREADS = VESIS_SWEEP_THREADS;
-constexpr int NWARP = SW_THREADS / 32;
+constexpr int TEAM = 64;          // threads of a team: two warps, a half tile each
+constexpr int NTEAM = 8;          // teams of a block (named barriers 1 .. 8)
+constexpr int SW_THREADS = TEAM * NTEAM;
 constexpr int kLine = 32;         // words per 128-byte line of the control block
+// control block: the count of leader half tiles, then the barrier's counter
+constexpr int kCtlWords = 2 * kLine;
 constexpr int kMaxBricksPerTile = 64;         // (8 / 2)^3 for bricks of edge 2
 constexpr int kHaloRows = (TS + 2) * (TS + 2);
 // Bricks per axis a tile can see: the tile's own (8 / B) and ceil(r / B) on
@@ -74,31 +90,26 @@ constexpr int kHaloRows = (TS + 2) * (TS + 2);
 // within r of a tile, and the rivals of a tile's own leaders, all lie there.
 constexpr int kNbh = 6;
 constexpr int kNbh3 = kNbh * kNbh * kNbh;
-// Winners within r of a tile are more than r apart inside a box of edge
-// 8 + 2r: at most ceil((8 + 2r) / (r + 1))^3 <= 125 of them.
-constexpr int kMaxWin = 128;
-// Tiles a thread examines per pass when a block lists its tiles: one pass
-// lists up to SW_THREADS * kGatherPer of them.
-constexpr int kGatherPer = 4;
-constexpr int kListCap = SW_THREADS * kGatherPer;
+constexpr int kSlots = (kNbh3 + TEAM - 1) / TEAM;     // of those, per thread
 // Posting area of a tile: 216 16-bit slots and an 8-word slot bitmap.
 constexpr int kPostBytes = 512;
 constexpr int kPostMaskOff = 448;
-
-// Blocks per SM of the cooperative grid (upper bound; shared memory and
-// registers may allow fewer).
-#ifndef VESIS_SWEEP_BPS
-#define VESIS_SWEEP_BPS 1
-#endif
 // A block keeps one bit per own tile (holds a leader) in shared memory:
 // up to 32768 own tiles, more than a grid of 2^31 cells gives any block.
 constexpr int kOwnWords = 1024;
+// 1-D weights padded with zeros: entry a + kQ0 holds q_a, |a| <= 15
+constexpr int kQ0 = 16;
+// a row of the full stencil in shared memory: offsets -15 .. 15, zeros past r
+constexpr int kKtRow = 31;
+
+__host__ __device__ constexpr int sweep_edge(int r) { return r >= 3 ? 4 : 2; }
 
 struct SweepArgs {
     GridDesc g;
     KernelW kw;
     double cD;          // c_N: dE = c_N N - s h^3 U
     double h3;
+    float cDf, h3f;     // the same in FP32
     int qc3;            // k0, the kernel's centre weight
     int ksum;           // S, the sum of all kernel weights
     const int *k3;      // full stencil (device) or NULL for the product kernel
@@ -112,14 +123,24 @@ struct SweepArgs {
                               // at (w nx + i) ny + j (a tile's halo words adjoin)
     int nzw;
     uint8_t *post;            // posting area per tile (kPostBytes)
-    uint8_t *upd;             // tile received a winner this round
-    int *dirty;               // per tile: the round whose decide must visit it
+    // bitmaps over the launch's tiles, block by block: bit j of block b is bit
+    // j % 32 of word b * bwords + j / 32 (see set_tile_bit); two of each, for
+    // even and odd rounds, so that a block clears one while the other is used
+    unsigned *upd;            // tile received a winner this round
+    unsigned *stamp;          // tile must be decided next round
+    int bwords;
+    unsigned mapw;            // words of one bitmap
+    unsigned tile0;           // the system's first tile among the launch's (multi)
+    unsigned nblk, nblk_inv;  // gridDim and ceil(2^32 / gridDim)
     int ntx, nty, ntz;
+    unsigned nty_inv, ntz_inv;    // ceil(2^32 / .)
     int bs, bsh;        // brick edge and its log2
     int reach;          // ceil(r / B)
     int nbx, nby, nbz;  // bricks per axis
-    int vec;            // rows of 8 W and U values may be loaded as vectors
-    unsigned *nlead;    // tiles holding a leader (kept current by the updates)
+    int vec;            // a tile's rows of W and U are loaded as two vectors each (2), as the
+                        // three that cover them (1: rows at odd offsets) or cell by cell (0)
+    unsigned ncell;
+    unsigned *nlead;    // half tiles holding a leader (kept current by the updates)
     unsigned *bar;      // monotonic arrival counter (own 128-byte line)
     int *err;
     unsigned long long *part_flips;   // [gridDim.x]
@@ -131,41 +152,26 @@ struct SweepArgs {
     long long spin_limit;     // polls before a barrier wait gives up
     int stamps;               // decide stamps: -1 by the leader count, 0 never, 1 always
     RoundState *rs;           // this system's totals (multi-system sweep)
-    double *tile_dE;          // per tile: its winners' dE, summed over rounds (multi)
-    unsigned *tile_nf;        // per tile: its flips (multi)
+    double *tile_dE;          // per half tile: its winners' dE, summed over rounds (multi)
+    unsigned *tile_nf;        // per half tile: its flips (multi)
 };
 
-// Per-warp shared memory; the decide and update phases use it in turn.
-struct WarpMem {
-    union {
-        struct {
-            unsigned long long w[kNbh3];   // leader words of the 6^3 bricks
-            unsigned c[kNbh3];             // their cells, 5 bits per axis
-            unsigned long long cw[kNbh3];  // the non-zero words, compacted
-            unsigned cc[kNbh3];            // and their cells
-        } d;
-        struct {
-            unsigned cW[512];              // candidates: W
-            float cU[512];                 //             U
-            unsigned short cP[512];        //             tile cell | label << 9
-            unsigned hr[kHaloRows];        // label bits of the halo rows (bit 0: z = -1)
-            unsigned win[kMaxWin];         // winners: tile coords + 8 (5 bits each) | label << 15
-            unsigned long long bmax[kMaxBricksPerTile];   // new leader per brick
-        } u;
-    };
+// A team's shared memory.  Every area has two copies, taken in turn: between
+// the one barrier of a tile and that of the next, a warp may still read the
+// copy the other warp wrote before the first.
+struct TeamMem {
+    unsigned long long lw[2][kMaxBricksPerTile];  // decide: the tile's leader words
+    unsigned lc[2][kMaxBricksPerTile];            //   and their cells, 5 bits per axis
+    unsigned long long cw[2][2][kSlots * 32];     //   the non-zero words each warp saw
+    unsigned cc[2][2][kSlots * 32];               //   and their cells
+    int ncw[2][2];                                //   their number
+    unsigned long long bmax[kMaxBricksPerTile];   // update: new leader per brick
+    unsigned hr[2][kHaloRows];   //   label bits of the halo rows (bit 0: z = -1)
+    unsigned win[2][2][kSlots * 32];   // winners each warp found: tile coords + 8
+                                       //   (5 bits each) | label << 15
+    int nw[2][2];                      //   their number
 };
 
-// Grid barrier on a monotonic arrival counter: barrier number e (1, 2, ...)
-// completes when the counter reaches e * gridDim.x.  Arrival is one release
-// reduction (it orders the block's earlier writes, which bar.sync has made
-// visible to thread 0), the wait a relaxed poll (an acquire load per poll
-// would discard the SM's L1 under the blocks still working) closed by one
-// acquire load of the counter, which reads the completed count and so
-// synchronises with every arrival's release (a barrier alone measured 1.16
-// us against 1.26 with a closing acquire fence); no reset is needed.  The poll is bounded (A.spin_limit
-// polls; 0 gives up at the first poll that finds the barrier open) and
-// watches the error flag every 256 polls; a timeout raises the flag and the
-// caller returns.
 __device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned *p)
 {
     unsigned v;
@@ -180,65 +186,49 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p)
     return v;
 }
 
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, int *err, long long spin_limit,
-                                             unsigned &target, int *abort_flag)
+// Where a block of the sweep stands at the barrier between phases.
+struct Barrier {
+    unsigned *bar;            // monotonic arrival counter
+    unsigned target;          // thread 0: arrivals the next barrier waits for
+    int *err;
+    long long spin_limit;
+};
+
+// Barrier of all blocks: number e (1, 2, ...) completes when the counter
+// reaches e * gridDim.x.  Arrival is one release reduction (it orders the
+// block's earlier writes, which bar.sync has made visible to thread 0); the
+// wait polls with acquire loads, back to back (this block alone uses its SM,
+// so nothing is lost to the L1 they invalidate, and no closing acquire is
+// needed).  The poll is bounded (spin_limit polls; 0 gives up at the first
+// poll that finds the barrier open) and watches the error flag every 256
+// polls; a timeout raises the flag and the caller returns.  (Spreading the
+// arrivals over 4 or 8 counters, polled by as many lanes, cost 0.1 us a
+// barrier more than one.)
+__device__ __forceinline__ bool all_blocks(Barrier &B, int *abort_flag)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
-        target += gridDim.x;
-        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" :: "l"(bar), "r"(1u)
+        B.target += gridDim.x;
+        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" :: "l"(B.bar), "r"(1u)
                      : "memory");
         long long spins = 0;
-        while ((int)(ld_relaxed_u32(bar) - target) < 0) {
-            if (++spins > spin_limit ||
-                ((spins & 255) == 0 && *(volatile int *)err)) {
-                atomicExch(err, 1);
+        while ((int)(ld_acquire_u32(B.bar) - B.target) < 0) {
+            if (++spins > B.spin_limit ||
+                ((spins & 255) == 0 && *(volatile int *)B.err)) {
+                atomicExch(B.err, 1);
                 *abort_flag = 1;
                 break;
             }
-            __nanosleep(32);
         }
-        (void)ld_acquire_u32(bar);
     }
     __syncthreads();
     return *abort_flag == 0;
 }
 
-__device__ __forceinline__ void tile_origin(const SweepArgs &A, int t, int &i0,
-                                            int &j0, int &k0)
+// Barrier of one team (hardware barriers 1 .. NTEAM; 0 is the block's).
+__device__ __forceinline__ void team_sync(int team)
 {
-    const int tk = t % A.ntz;
-    const int tj = (t / A.ntz) % A.nty;
-    const int ti = t / (A.ntz * A.nty);
-    i0 = ti * TS;
-    j0 = tj * TS;
-    k0 = tk * TS;
-}
-
-// Cell (ci, cj, ck) of the leader word w of brick (bx, by, bz), found from
-// its linear index without a division: the offset from the brick's first
-// cell is di * nyz + dj * nz + dk with 0 <= di, dj, dk < B.
-__device__ __forceinline__ void leader_cell(const SweepArgs &A, unsigned long long w,
-                                            int bx, int by, int bz, int &ci, int &cj,
-                                            int &ck)
-{
-    const long long nyz = (long long)A.g.ny * A.g.nz;
-    const long long p = (long long)(0xffffffffull - ((w >> 1) & 0xffffffffull));
-    ci = bx << A.bsh;
-    cj = by << A.bsh;
-    ck = bz << A.bsh;
-    long long d = p - ((long long)ci * nyz + (long long)cj * A.g.nz + ck);
-    for (int s = 1; s < A.bs; ++s)
-        if (d >= nyz) {
-            d -= nyz;
-            ++ci;
-        }
-    for (int s = 1; s < A.bs; ++s)
-        if (d >= A.g.nz) {
-            d -= A.g.nz;
-            ++cj;
-        }
-    ck += (int)d;
+    asm volatile("bar.sync %0, %1;" :: "r"(team + 1), "n"(TEAM) : "memory");
 }
 
 __device__ __forceinline__ void red_or(unsigned *p, unsigned v)
@@ -251,605 +241,606 @@ __device__ __forceinline__ void red_add(unsigned *p, unsigned v)
     asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
 }
 
-// 16-byte asynchronous global -> shared copy through L2 (zero fill when
-// !valid), and the wait for this thread's copies.
-__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool valid)
+// Tiles are dealt to the blocks in groups of gridDim consecutive ones, each
+// group rotated by a hash of its number: tile t is number j = t / gridDim of
+// block (t + turn(j)) % gridDim.  (Unrotated, the tiles of one z layer share a
+// block whenever gridDim and the tiles per axis have a common factor.)
+__device__ __forceinline__ unsigned turn_of(unsigned j, unsigned nblk)
 {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                 :: "r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+    return __umulhi(j * 0x9E3779B1u, nblk);
 }
 
-__device__ __forceinline__ void cp_async_wait_all()
+// Sets the bit of the system's tile t in a bitmap over the launch's tiles.
+// The quotient by gridDim is exact: at most 2^15 tiles per block and 256 blocks.
+__device__ __forceinline__ void set_tile_bit(const SweepArgs &A, unsigned *map, unsigned t)
 {
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    const unsigned tg = A.tile0 + t;
+    const unsigned j = A.nblk == 1u ? tg : __umulhi(tg, A.nblk_inv);
+    unsigned b = tg - j * A.nblk + turn_of(j, A.nblk);
+    if (b >= A.nblk) b -= A.nblk;
+    red_or(map + (size_t)b * A.bwords + (j >> 5), 1u << (j & 31));
 }
 
-// Labels, W, dE, leader words, postings and tile flags change under other
-// warps and blocks between phases: every read of them goes to L2
+// Tile number j of this block (may lie past the last tile).
+__device__ __forceinline__ long long own_tile_no(int j)
+{
+    int r = (int)blockIdx.x - (int)turn_of((unsigned)j, gridDim.x);
+    if (r < 0) r += (int)gridDim.x;
+    return (long long)j * gridDim.x + r;
+}
+
+// A tile's number and coordinates.
+struct Tile {
+    int t, i, j, k;
+};
+
+// (Quotients exact: t < 2^22 and at most 512 tiles per axis.)
+__device__ __forceinline__ Tile make_tile(const SweepArgs &A, int t)
+{
+    const int q = A.ntz == 1 ? t : (int)__umulhi((unsigned)t, A.ntz_inv);
+    const int i = A.nty == 1 ? q : (int)__umulhi((unsigned)q, A.nty_inv);
+    return {t, i, q - i * A.nty, t - q * A.ntz};
+}
+
+// What a thread of a team does in every tile: its slots of the 6^3 bricks,
+// as a | b << 4 | c << 8 (brick relative to the first) | n << 12, n - 1 the
+// brick's number among the tile's own if it is one (n = 0: it is not); bit
+// 31: no slot.
+struct Lane {
+    int u, w, lane;            // thread of the team, warp, lane
+    unsigned slot[kSlots];
+};
+
+__device__ __forceinline__ Lane make_lane(int bpt, int reach)
+{
+    Lane L;
+    L.u = threadIdx.x % TEAM;
+    L.w = L.u >> 5;
+    L.lane = L.u & 31;
+#pragma unroll
+    for (int m = 0; m < kSlots; ++m) {
+        const int q = L.u + TEAM * m;
+        const int a = q / (kNbh * kNbh), b = (q / kNbh) % kNbh, c = q % kNbh;
+        const int x = a - reach, y = b - reach, z = c - reach;
+        const bool own = x >= 0 && y >= 0 && z >= 0 && x < bpt && y < bpt && z < bpt;
+        L.slot[m] = q < kNbh3 ? (unsigned)(a | b << 4 | c << 8 |
+                                           (own ? (x * bpt + y) * bpt + z + 1 : 0) << 12)
+                              : 0x80000000u;
+    }
+    return L;
+}
+
+// Labels, W, dE, leader words, postings and tile bits change under other
+// teams and blocks between phases: every read of them goes to L2
 // (ld.global.cg), never to a stale L1 line.
 
-// Decide phase for tile t (one warp).
-__device__ __forceinline__ void tile_decide(const SweepArgs &A, WarpMem &M, int t,
-                                            double &e_lane, unsigned &n_lane)
+// Decide phase for one tile; each warp settles half of its leaders (bricks of
+// edge 4: x half w, eight lanes per leader; of edge 2: leaders 32 w .. 32 w +
+// 31, one per lane).  e_lane, n_lane: dE and count of the winners; turn: which
+// copy of the shared areas the tile uses.
+__device__ __forceinline__ void tile_decide(const SweepArgs &A, TeamMem &M, const Lane &L,
+                                            int team, const Tile &tile, int &turn,
+                                            unsigned *upd, double &e_lane, unsigned &n_lane)
 {
-    const int lane = threadIdx.x & 31;
     const GridDesc &g = A.g;
     const int r = A.kw.r, bsh = A.bsh, reach = A.reach;
     const int bpt = TS >> bsh;
-    const int nbt = bpt * bpt * bpt;
-    int i0, j0, k0;
-    tile_origin(A, t, i0, j0, k0);
-    const int nbx0 = (i0 >> bsh) - reach, nby0 = (j0 >> bsh) - reach, nbz0 = (k0 >> bsh) - reach;
-    constexpr int PER = (kNbh3 + 31) / 32;
-    unsigned long long v[PER];
-    unsigned off[PER];
+    const int nbx0 = tile.i * bpt - reach, nby0 = tile.j * bpt - reach, nbz0 = tile.k * bpt - reach;
+    unsigned long long v[kSlots];
+    unsigned off[kSlots];
 #pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int q = lane + 32 * u;
-        v[u] = 0ull;
-        off[u] = 0u;
-        if (q < kNbh3) {
-            const int bx = nbx0 + q / (kNbh * kNbh), by = nby0 + (q / kNbh) % kNbh,
-                      bz = nbz0 + q % kNbh;
-            if (bx >= 0 && by >= 0 && bz >= 0 && bx < A.nbx && by < A.nby && bz < A.nbz) {
-                const long long o = ((long long)bx * A.nby + by) * A.nbz + bz;
-                v[u] = __ldcg(A.PL + o);
-                off[u] = __ldcg(A.PO + o);
-            }
+    for (int m = 0; m < kSlots; ++m) {
+        const int bx = nbx0 + (int)(L.slot[m] & 15u), by = nby0 + (int)((L.slot[m] >> 4) & 15u),
+                  bz = nbz0 + (int)((L.slot[m] >> 8) & 15u);
+        v[m] = 0ull;
+        off[m] = 0u;
+        if ((int)L.slot[m] >= 0 && (unsigned)bx < (unsigned)A.nbx &&
+            (unsigned)by < (unsigned)A.nby && (unsigned)bz < (unsigned)A.nbz) {
+            const int q = (bx * A.nby + by) * A.nbz + bz;
+            v[m] = __ldcg(A.PL + q);
+            off[m] = __ldcg(A.PO + q);
         }
     }
-    // leader cells relative to the neighbourhood's first cell; the non-zero
-    // words compacted for the scans below
-    int m = 0;
+    // the tile's own words and all non-zero ones to shared memory, with their
+    // cells relative to the neighbourhood's first cell
+    const unsigned below = (1u << L.lane) - 1u;
+    int at = 0;
 #pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int q = lane + 32 * u;
-        unsigned c = 0u;
-        if (v[u] != 0ull) {
-            const int bx = q / (kNbh * kNbh), by = (q / kNbh) % kNbh, bz = q % kNbh;
-            c = (unsigned)(bx * A.bs + (int)(off[u] & 3u)) |
-                ((unsigned)(by * A.bs + (int)((off[u] >> 2) & 3u)) << 5) |
-                ((unsigned)(bz * A.bs + (int)((off[u] >> 4) & 3u)) << 10);
+    for (int m = 0; m < kSlots; ++m) {
+        const unsigned c = ((L.slot[m] & 15u) << bsh) + (off[m] & 3u) +
+                           (((((L.slot[m] >> 4) & 15u) << bsh) + ((off[m] >> 2) & 3u)) << 5) +
+                           (((((L.slot[m] >> 8) & 15u) << bsh) + ((off[m] >> 4) & 3u)) << 10);
+        const int own = (int)((L.slot[m] >> 12) & 127u) - 1;
+        if (own >= 0) {
+            M.lw[turn][own] = v[m];
+            M.lc[turn][own] = c;
         }
-        if (q < kNbh3) {
-            M.d.w[q] = v[u];
-            M.d.c[q] = c;
+        const unsigned bm = __ballot_sync(0xffffffffu, v[m] != 0ull);
+        if (v[m] != 0ull) {
+            const int to = at + __popc(bm & below);
+            M.cw[turn][L.w][to] = v[m];
+            M.cc[turn][L.w][to] = c;
         }
-        const unsigned bm = __ballot_sync(0xffffffffu, v[u] != 0ull);
-        if (v[u] != 0ull) {
-            const int pos = m + __popc(bm & ((1u << lane) - 1u));
-            M.d.cw[pos] = v[u];
-            M.d.cc[pos] = c;
-        }
-        m += __popc(bm);
+        at += __popc(bm);
     }
-    __syncwarp();
-    // verdicts: a leader of the tile wins unless another within r is better.
-    // G lanes share one of the tile's bricks and split the scan of the
-    // compacted words between them.
-    unsigned long long wmask = 0ull;
-    {
-        const int G = nbt >= 32 ? 1 : 32 / nbt;      // 4 for 8 bricks
-        const int P = 32 / G;                         // bricks per pass
-        const int gl = lane / G, sub = lane - gl * G;
-        for (int b0 = 0; b0 < nbt; b0 += P) {
-            const int b = b0 + gl;
-            unsigned long long L = 0ull;
-            int lx = 0, ly = 0, lz = 0;
-            if (b < nbt) {
-                const int bx = b / (bpt * bpt), by = (b / bpt) % bpt, bz = b % bpt;
-                const int o = ((reach + bx) * kNbh + (reach + by)) * kNbh + (reach + bz);
-                L = M.d.w[o];
-                const unsigned lc = M.d.c[o];
-                lx = lc & 31;
-                ly = (lc >> 5) & 31;
-                lz = (lc >> 10) & 31;
-            }
-            bool lose = false;
-            if (L != 0ull) {
-                // branch-free and unrolled, so that several shared-memory
-                // loads are in flight at once
-#pragma unroll 4
-                for (int q = sub; q < m; q += G) {
-                    const unsigned long long w = M.d.cw[q];
-                    const unsigned c = M.d.cc[q];
-                    const int ox = c & 31, oy = (c >> 5) & 31, oz = (c >> 10) & 31;
-                    lose |= (w > L) & (abs(ox - lx) <= r) & (abs(oy - ly) <= r) &
-                            (abs(oz - lz) <= r);
-                }
-            }
-            const unsigned lb = __ballot_sync(0xffffffffu, lose);
-            const unsigned gm = (G == 32) ? 0xffffffffu : ((1u << G) - 1u);
-            const bool win = L != 0ull && sub == 0 && ((lb >> (gl * G)) & gm) == 0u;
-            const unsigned wb = __ballot_sync(0xffffffffu, win);
-            for (int q = 0; q < P && b0 + q < nbt; ++q)
-                if ((wb >> (q * G)) & 1u) wmask |= 1ull << (b0 + q);
+    if (L.lane == 0) M.ncw[turn][L.w] = at;
+    team_sync(team);
+    // a leader of the tile loses to any better word within r
+    const int n0 = M.ncw[turn][0], ncw = n0 + M.ncw[turn][1];
+    const int per = bpt == 2 ? 4 : 32;                 // leaders of a warp
+    const int mine = per * L.w + (L.lane & (per - 1)), step = 32 / per;
+    const unsigned long long lead = M.lw[turn][mine];
+    bool beat = false;
+    if (lead != 0ull) {
+        const unsigned lc = M.lc[turn][mine];
+        const int lx = (int)(lc & 31u) - r, ly = (int)((lc >> 5) & 31u) - r,
+                  lz = (int)((lc >> 10) & 31u) - r;
+        const unsigned long long *cw = M.cw[turn][0];
+        const unsigned *cc = M.cc[turn][0];
+#pragma unroll 2
+        for (int q = bpt == 2 ? L.lane >> 2 : 0; q < ncw; q += step) {
+            const int k = q < n0 ? q : q - n0 + kSlots * 32;
+            const unsigned long long o = cw[k];
+            const unsigned c = cc[k];
+            beat |= (o > lead) & ((unsigned)((int)(c & 31u) - lx) <= 2u * r) &
+                    ((unsigned)((int)((c >> 5) & 31u) - ly) <= 2u * r) &
+                    ((unsigned)((int)((c >> 10) & 31u) - lz) <= 2u * r);
         }
     }
-    if (wmask == 0ull) return;
-    // winners: flip and fetch dE (added at the end), post to every tile
-    // within r
-    double dv[2] = {0.0, 0.0};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int b = lane + 32 * h;
-        if (b >= nbt || !((wmask >> b) & 1ull)) continue;
-        const int bx = b / (bpt * bpt), by = (b / bpt) % bpt, bz = b % bpt;
-        const int o = ((reach + bx) * kNbh + (reach + by)) * kNbh + (reach + bz);
-        const unsigned long long L = M.d.w[o];
-        const unsigned lc = M.d.c[o];
-        const int ci = nbx0 * A.bs + (int)(lc & 31), cj = nby0 * A.bs + (int)((lc >> 5) & 31),
-                  ck = nbz0 * A.bs + (int)((lc >> 10) & 31);
-        const long long p = (long long)(0xffffffffull - ((L >> 1) & 0xffffffffull));
-        A.chi[p] = (uint8_t)(1u - (unsigned)(L & 1ull));
+    // winners among the warp's leaders: bit l is leader per * w + l
+    unsigned wm = __ballot_sync(0xffffffffu, beat);
+    if (bpt == 2) {
+        wm |= wm >> 16;
+        wm |= wm >> 8;
+        wm |= wm >> 4;
+    }
+    wm = __ballot_sync(0xffffffffu, lead != 0ull) & ~wm & (bpt == 2 ? 15u : 0xffffffffu);
+    const int my = turn;
+    turn ^= 1;
+    // they flip and fetch dE (added at the end) ...
+    double dv = 0.0;
+    if ((wm >> L.lane) & 1u) {
+        const unsigned long long won = M.lw[my][per * L.w + L.lane];
+        const unsigned lc = M.lc[my][per * L.w + L.lane];
+        const int ci = (nbx0 << bsh) + (int)(lc & 31u), cj = (nby0 << bsh) + (int)((lc >> 5) & 31u),
+                  ck = (nbz0 << bsh) + (int)((lc >> 10) & 31u);
+        const unsigned p = ~(unsigned)(won >> 1);
+        A.chi[p] = (uint8_t)(1u - (unsigned)(won & 1ull));
         asm volatile("red.relaxed.gpu.global.xor.b32 [%0], %1;"
-                     :: "l"(A.CB + ((long long)(ck >> 5) * g.nx + ci) * g.ny + cj),
+                     :: "l"(A.CB + (((ck >> 5) * g.nx + ci) * g.ny + cj)),
                         "r"(1u << (ck & 31)) : "memory");
-        dv[h] = __ldcg(A.dE + p);
+        dv = __ldcg(A.dE + p);
         n_lane += 1u;
     }
-    unsigned long long rest = wmask;
-    while (rest) {
-        const int b = __ffsll((long long)rest) - 1;
-        rest &= rest - 1;
-        const int bx = b / (bpt * bpt), by = (b / bpt) % bpt, bz = b % bpt;
-        const int o = ((reach + bx) * kNbh + (reach + by)) * kNbh + (reach + bz);
-        const unsigned long long L = M.d.w[o];
-        const unsigned lc = M.d.c[o];
-        const int ci = (nbx0 * A.bs) + (int)(lc & 31), cj = (nby0 * A.bs) + (int)((lc >> 5) & 31),
-                  ck = (nbz0 * A.bs) + (int)((lc >> 10) & 31);
-        const unsigned entry = (unsigned)(ci & (A.bs - 1)) | ((unsigned)(cj & (A.bs - 1)) << 2) |
-                               ((unsigned)(ck & (A.bs - 1)) << 4) | ((unsigned)(L & 1ull) << 6);
-        const int ti0 = max(ci - r, 0) / TS, ti1 = min(ci + r, g.nx - 1) / TS;
-        const int tj0 = max(cj - r, 0) / TS, tj1 = min(cj + r, g.ny - 1) / TS;
-        const int tk0 = max(ck - r, 0) / TS, tk1 = min(ck + r, g.nz - 1) / TS;
-        if (lane < 27) {
-            const int ta = ti0 + lane / 9, tb = tj0 + (lane / 3) % 3, tc = tk0 + lane % 3;
-            if (ta <= ti1 && tb <= tj1 && tc <= tk1) {
-                const int tt = (ta * A.nty + tb) * A.ntz + tc;
-                // the winner's brick among the 6^3 bricks tile tt sees
-                const int sx = (ci >> bsh) - ((ta * TS) >> bsh) + reach;
-                const int sy = (cj >> bsh) - ((tb * TS) >> bsh) + reach;
-                const int sz = (ck >> bsh) - ((tc * TS) >> bsh) + reach;
-                const int slot = (sx * kNbh + sy) * kNbh + sz;
-                uint8_t *pa = A.post + (size_t)tt * kPostBytes;
-                reinterpret_cast<unsigned short *>(pa)[slot] = (unsigned short)entry;
-                red_or(reinterpret_cast<unsigned *>(pa + kPostMaskOff) + (slot >> 5),
-                       1u << (slot & 31));
-                A.upd[tt] = 1;
-            }
+    // ... and post themselves to every tile within r, a lane per tile
+    for (unsigned todo = wm; todo; todo &= todo - 1) {
+        const int b = per * L.w + __ffs(todo) - 1;
+        const unsigned long long won = M.lw[my][b];
+        const unsigned lc = M.lc[my][b];
+        const int ci = (nbx0 << bsh) + (int)(lc & 31u), cj = (nby0 << bsh) + (int)((lc >> 5) & 31u),
+                  ck = (nbz0 << bsh) + (int)((lc >> 10) & 31u);
+        const int ta = (max(ci - r, 0) / TS) + L.lane / 9, tb = (max(cj - r, 0) / TS) + (L.lane / 3) % 3,
+                  tc = (max(ck - r, 0) / TS) + L.lane % 3;
+        if (L.lane < 27 && ta <= min(ci + r, g.nx - 1) / TS && tb <= min(cj + r, g.ny - 1) / TS &&
+            tc <= min(ck + r, g.nz - 1) / TS) {
+            const unsigned entry = (unsigned)(ci & (A.bs - 1)) | ((unsigned)(cj & (A.bs - 1)) << 2) |
+                                   ((unsigned)(ck & (A.bs - 1)) << 4) |
+                                   ((unsigned)(won & 1ull) << 6);
+            const int tt = (ta * A.nty + tb) * A.ntz + tc;
+            // the winner's brick among the 6^3 bricks tile tt sees
+            const int sx = (ci >> bsh) - ((ta * TS) >> bsh) + reach;
+            const int sy = (cj >> bsh) - ((tb * TS) >> bsh) + reach;
+            const int sz = (ck >> bsh) - ((tc * TS) >> bsh) + reach;
+            const int slot = (sx * kNbh + sy) * kNbh + sz;
+            uint8_t *pa = A.post + (size_t)tt * kPostBytes;
+            reinterpret_cast<unsigned short *>(pa)[slot] = (unsigned short)entry;
+            red_or(reinterpret_cast<unsigned *>(pa + kPostMaskOff) + (slot >> 5),
+                   1u << (slot & 31));
+            set_tile_bit(A, upd, (unsigned)tt);
         }
     }
-    e_lane += dv[0];
-    e_lane += dv[1];
+    e_lane += dv;
 }
 
-// Update phase for tile t (one warp).  first: the opening pass (no
-// winners; every tile computes its leaders).  mark >= 0: if a leader word
-// of the tile changes, the 27 tiles around it (itself included) are
-// stamped with mark, the round whose decide must visit them.
+// Update phase for one tile, the half with 0 <= x - 4 w < 4 by warp w (bricks
+// never straddle the halves).  first: the opening pass (no winners; every tile
+// computes its leaders).  stamp: the bitmap (or NULL) in which the 27 tiles
+// around it (itself included) are marked for the next decide if a leader word
+// of the half changes.
+// Returns whether the warp's half holds a leader.
 template <bool STENCIL>
-__device__ __forceinline__ bool tile_update(const SweepArgs &A, WarpMem &M, const int *qw,
-                                            const int *kt,
-                                            int t, bool first, int mark)
+__device__ __forceinline__ bool tile_update(const SweepArgs &A, TeamMem &M, const int *qw,
+                                            const int *kt, const Lane &L, int team,
+                                            const Tile &tile, bool first, unsigned *stamp, int &turn)
 {
-    const int lane = threadIdx.x & 31;
     const GridDesc &g = A.g;
-    const long long nyz = (long long)g.ny * g.nz;
+    const int nyz = g.ny * g.nz;
     const int r = A.kw.r, bsh = A.bsh, reach = A.reach;
     const int bpt = TS >> bsh;
-    const int nbt = bpt * bpt * bpt;
-    int i0, j0, k0;
-    tile_origin(A, t, i0, j0, k0);
-    const int zlim = min(TS, g.nz - k0);
-    const unsigned zmask = (1u << zlim) - 1u;
+    const int ti = tile.i, tj = tile.j, tk = tile.k;
+    const int i0 = ti * TS, j0 = tj * TS, k0 = tk * TS;
+    const int u = L.u;
 
     // ---------------------------------------------------------- loads
-    // All of a lane's loads are issued before the first use.  W and U of the
-    // tile's own cells: rows rho = lane + 32 m, (x, y) = (rho >> 3, rho & 7).
-    // With 8-cell rows in 16-byte pieces (vec) they pass through the warp's
-    // candidate area in shared memory, consecutive lanes on consecutive
-    // pieces (two lanes per 32-byte row), so that each copy instruction
-    // reads whole sectors; otherwise each lane loads its rows itself.
-    unsigned Wr[2][TS];
-    float Ur[2][TS];
-    bool rowok[2];
+    // All of a thread's loads are issued before the first use.  Its cells:
+    // row (cx, cy).
+    const int cx = u >> 3, cy = u & 7;
+    const bool rowok = i0 + cx < g.nx && j0 + cy < g.ny;
+    const int zc = rowok ? min(TS, g.nz - k0) : 0;        // cells inside the grid
+    const unsigned o = (unsigned)(i0 + cx) * (unsigned)nyz + (unsigned)((j0 + cy) * g.nz + k0);
+    unsigned Wr[TS];
+    float Ur[TS];
 #pragma unroll
-    for (int m = 0; m < 2; ++m) {
-        const int rho = lane + 32 * m;
-        rowok[m] = (i0 + (rho >> 3) < g.nx) && (j0 + (rho & 7) < g.ny);
-#pragma unroll
-        for (int z = 0; z < TS; ++z) {
-            Wr[m][z] = 0u;
-            Ur[m][z] = 0.f;
-        }
+    for (int z = 0; z < TS; ++z) {
+        Wr[z] = 0u;
+        Ur[z] = 0.f;
     }
-    const unsigned sW = (unsigned)__cvta_generic_to_shared(M.u.cW);
-    const unsigned sU = (unsigned)__cvta_generic_to_shared(M.u.cU);
-    if (A.vec) {
+    if (A.vec == 2) {
+        if (zc) {
 #pragma unroll
-        for (int c4 = 0; c4 < 4; ++c4) {
-            const int c = lane + 32 * c4;            // piece c: row c >> 1, half c & 1
-            const int rho = c >> 1;
-            const bool ok = (i0 + (rho >> 3) < g.nx) && (j0 + (rho & 7) < g.ny);
-            const long long o = ok ? (long long)(i0 + (rho >> 3)) * nyz +
-                                         (long long)(j0 + (rho & 7)) * g.nz + k0 + 4 * (c & 1)
-                                   : 0;
-            cp_async16(sW + 16u * (unsigned)c, A.W + o, ok);
-            cp_async16(sU + 16u * (unsigned)c, A.U + o, ok);
+            for (int h = 0; h < TS; h += 4) {
+                const uint4 wv = __ldcg(reinterpret_cast<const uint4 *>(A.W + o + h));
+                const float4 uv = __ldg(reinterpret_cast<const float4 *>(A.U + o + h));
+                Wr[h] = wv.x; Wr[h + 1] = wv.y; Wr[h + 2] = wv.z; Wr[h + 3] = wv.w;
+                Ur[h] = uv.x; Ur[h + 1] = uv.y; Ur[h + 2] = uv.z; Ur[h + 3] = uv.w;
+            }
+        }
+    } else if (A.vec == 1 && (o & ~3u) + 12u <= A.ncell) {
+        if (zc) {
+            unsigned wv[12], uv[12];
+#pragma unroll
+            for (int h = 0; h < 12; h += 4) {
+                const uint4 a = __ldcg(reinterpret_cast<const uint4 *>(A.W + ((o & ~3u) + h)));
+                const uint4 b = __ldg(reinterpret_cast<const uint4 *>(A.U + ((o & ~3u) + h)));
+                wv[h] = a.x; wv[h + 1] = a.y; wv[h + 2] = a.z; wv[h + 3] = a.w;
+                uv[h] = b.x; uv[h + 1] = b.y; uv[h + 2] = b.z; uv[h + 3] = b.w;
+            }
+#pragma unroll
+            for (int z = 0; z < 11; ++z) {
+                wv[z] = o & 1u ? wv[z + 1] : wv[z];
+                uv[z] = o & 1u ? uv[z + 1] : uv[z];
+            }
+#pragma unroll
+            for (int z = 0; z < TS; ++z) {
+                Wr[z] = o & 2u ? wv[z + 2] : wv[z];
+                Ur[z] = __uint_as_float(o & 2u ? uv[z + 2] : uv[z]);
+            }
         }
     } else {
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            const int rho = lane + 32 * m;
-            if (!rowok[m]) continue;
-            const long long o = (long long)(i0 + (rho >> 3)) * nyz +
-                                (long long)(j0 + (rho & 7)) * g.nz + k0;
-#pragma unroll
-            for (int z = 0; z < TS; ++z)
-                if (z < zlim) {
-                    Wr[m][z] = __ldcg(A.W + o + z);
-                    Ur[m][z] = __ldg(A.U + o + z);
-                }
-        }
+        for (int z = 0; z < TS; ++z)
+            if (z < zc) {
+                Wr[z] = __ldcg(A.W + o + z);
+                Ur[z] = __ldg(A.U + o + z);
+            }
     }
     // halo label rows from the bit copy: row h = hx * 10 + hy is the cell
     // column (i0 - 1 + hx, j0 - 1 + hy); bit z + 1 is cell k0 + z, z = -1..8.
     // Cells k0..k0 + 7 share word k0 / 32 (k0 is a multiple of 8); cell k0 - 1
     // or k0 + 8 sits in the word before or after when k0 % 32 is 0 or 24.
     // Bits past the end of a row are zero (solvent, as outside the box).
-    unsigned hb[4];
+    unsigned hm[2], hn[2];     // the word, and the word before or after
+    const int sh = k0 & 31;
+    const int pl = g.nx * g.ny;                           // words per plane
+    const int side = sh == 0 ? (k0 > 0 ? -pl : 0) : sh == 24 ? (k0 + TS < g.nz ? pl : 0) : 0;
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+        const int q = u + TEAM * m, hx = q / 10;
+        const int i = i0 - 1 + hx, j = j0 - 1 + q - 10 * hx;
+        hm[m] = hn[m] = 0u;
+        if (q < kHaloRows && i >= 0 && j >= 0 && i < g.nx && j < g.ny) {
+            const unsigned *col = A.CB + ((k0 >> 5) * pl + i * g.ny + j);
+            hm[m] = __ldcg(col);
+            if (side) hn[m] = __ldcg(col + side);
+        }
+    }
+    // posted winners: thread q < 54 holds slots 4 q .. 4 q + 3 and their bits
+    uint8_t *pa = A.post + (size_t)tile.t * kPostBytes;
+    unsigned *pmask = reinterpret_cast<unsigned *>(pa + kPostMaskOff);
+    unsigned long long ps = 0ull;
+    unsigned pm = 0u;
+    if (!first && u < kNbh3 / 4) {
+        ps = __ldcg(reinterpret_cast<const unsigned long long *>(pa) + u);
+        pm = __ldcg(pmask + (u >> 3));
+    }
+    // the leader word of the lane's brick before this update
+    const int per = bpt == 2 ? 4 : 32;                 // bricks of a warp
+    const int brick = per * L.w + (L.lane & (per - 1));
+    int bq = -1;
     {
-        const int sh = k0 & 31, wm = k0 >> 5;
-        const bool need_lo = sh == 0 && k0 > 0, need_hi = sh == 24 && k0 + TS < g.nz;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int h = lane + 32 * u;
-            hb[u] = 0u;
-            if (h < kHaloRows) {
-                const int i = i0 - 1 + h / 10, j = j0 - 1 + h % 10;
-                if (i >= 0 && j >= 0 && i < g.nx && j < g.ny) {
-                    const unsigned *col = A.CB + (long long)i * g.ny + j;
-                    const long long pl = (long long)g.nx * g.ny;     // words per plane
-                    const unsigned vm = __ldcg(col + wm * pl);
-                    const unsigned vl = need_lo ? __ldcg(col + (wm - 1) * pl) : 0u;
-                    const unsigned vh = need_hi ? __ldcg(col + (wm + 1) * pl) : 0u;
-                    const unsigned lo = sh == 0 ? (vl >> 31) : ((vm >> (sh - 1)) & 1u);
-                    const unsigned hi = sh == 24 ? (vh & 1u) : ((vm >> (sh + 8)) & 1u);
-                    hb[u] = lo | (((vm >> sh) & 0xffu) << 1) | (hi << 9);
-                }
-            }
-        }
+        const int gx = ti * bpt + brick / (bpt * bpt), gy = tj * bpt + (brick / bpt) % bpt,
+                  gz = tk * bpt + brick % bpt;
+        if (L.lane < per && gx < A.nbx && gy < A.nby && gz < A.nbz)
+            bq = (gx * A.nby + gy) * A.nbz + gz;
     }
-    // the tile's leader words before this update (brick b = lane + 32 h)
-    unsigned long long oldw[2] = {0ull, 0ull};
-    if (mark >= 0) {
+    unsigned long long oldw = 0ull;
+    if (stamp && bq >= 0) oldw = __ldcg(A.PL + bq);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int b = lane + 32 * h;
-            if (b >= nbt) continue;
-            const int gx = (i0 >> bsh) + b / (bpt * bpt), gy = (j0 >> bsh) + (b / bpt) % bpt,
-                      gz = (k0 >> bsh) + b % bpt;
-            if (gx < A.nbx && gy < A.nby && gz < A.nbz)
-                oldw[h] = __ldcg(A.PL + ((long long)gx * A.nby + gy) * A.nbz + gz);
-        }
+    for (int m = 0; m < 2; ++m) {
+        const unsigned lo = sh == 0 ? hn[m] >> 31 : (hm[m] >> (sh - 1)) & 1u;
+        const unsigned hi = sh == 24 ? hn[m] & 1u : (hm[m] >> (sh + 8)) & 1u;
+        if (u + TEAM * m < kHaloRows)
+            M.hr[turn][u + TEAM * m] = lo | (((hm[m] >> sh) & 0xffu) << 1) | (hi << 9);
     }
-    // posted winners: slot bitmap (lanes 0..7) and the 216 slots (lanes x 4 per u64)
-    uint8_t *pa = A.post + (size_t)t * kPostBytes;
-    unsigned pmask = 0u;
-    unsigned long long pslot[2] = {0ull, 0ull};
     if (!first) {
-        if (lane < 8) pmask = __ldcg(reinterpret_cast<const unsigned *>(pa + kPostMaskOff) + lane);
+        const unsigned set = (pm >> ((4 * u) & 31)) & 15u;
+        int at = 0;      // the order of the winners is free: W is an integer sum
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            const int q = lane + 32 * m;            // u64 q holds slots 4q .. 4q + 3
-            if (q < kNbh3 / 4) pslot[m] = __ldcg(reinterpret_cast<const unsigned long long *>(pa) + q);
+        for (int m = 0; m < 4; ++m) {
+            const bool have = (set >> m) & 1u;
+            const unsigned bm = __ballot_sync(0xffffffffu, have);
+            if (have) {
+                const int slot = 4 * u + m;
+                const unsigned e = (unsigned)(ps >> (16 * m)) & 0xffffu;
+                const int sx = slot / (kNbh * kNbh), sy = (slot / kNbh) % kNbh, sz = slot % kNbh;
+                // winner cell relative to the tile origin
+                const int wx = (sx - reach) * A.bs + (int)(e & 3u);
+                const int wy = (sy - reach) * A.bs + (int)((e >> 2) & 3u);
+                const int wz = (sz - reach) * A.bs + (int)((e >> 4) & 3u);
+                M.win[turn][L.w][at + __popc(bm & ((1u << L.lane) - 1u))] =
+                    (unsigned)(wx + 8) | ((unsigned)(wy + 8) << 5) | ((unsigned)(wz + 8) << 10) |
+                    (((e >> 6) & 1u) << 15);
+            }
+            at += __popc(bm);
         }
+        if (L.lane == 0) M.nw[turn][L.w] = at;
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int h = lane + 32 * u;
-        if (h < kHaloRows) M.u.hr[h] = hb[u];
-    }
-    if (A.vec) {      // the staged rows into registers before the area is reused
-        cp_async_wait_all();
-        __syncwarp();
-#pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            const int rho = lane + 32 * m;
-            const uint4 w0 = reinterpret_cast<const uint4 *>(M.u.cW)[2 * rho];
-            const uint4 w1 = reinterpret_cast<const uint4 *>(M.u.cW)[2 * rho + 1];
-            const float4 u0 = reinterpret_cast<const float4 *>(M.u.cU)[2 * rho];
-            const float4 u1 = reinterpret_cast<const float4 *>(M.u.cU)[2 * rho + 1];
-            Wr[m][0] = w0.x; Wr[m][1] = w0.y; Wr[m][2] = w0.z; Wr[m][3] = w0.w;
-            Wr[m][4] = w1.x; Wr[m][5] = w1.y; Wr[m][6] = w1.z; Wr[m][7] = w1.w;
-            Ur[m][0] = u0.x; Ur[m][1] = u0.y; Ur[m][2] = u0.z; Ur[m][3] = u0.w;
-            Ur[m][4] = u1.x; Ur[m][5] = u1.y; Ur[m][6] = u1.z; Ur[m][7] = u1.w;
-        }
-        __syncwarp();
-    }
+    team_sync(team);
 
-    // ------------------------------------------------- posted winners
-    int nw = 0;
+    // ------------------------------------------------- W of the own cells
     if (!first) {
         // the bitmap is consumed: clear it for the next round's postings
-        if (lane < 8 && pmask) reinterpret_cast<unsigned *>(pa + kPostMaskOff)[lane] = 0u;
-        // slot values to shared memory (reuse the candidate W list as scratch)
-        unsigned short *ps = reinterpret_cast<unsigned short *>(M.u.cW);
-#pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            const int q = lane + 32 * m;
-            if (q < kNbh3 / 4) reinterpret_cast<unsigned long long *>(ps)[q] = pslot[m];
-        }
-        __syncwarp();
-        // decode the set slots of each bitmap word (lane l < 7 owns word l)
-        const int cnt = __popc(pmask);
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        nw = __shfl_sync(0xffffffffu, incl, 7);
-        int pos = incl - cnt;
-        unsigned mm = pmask;
-        while (mm) {
-            const int bit = __ffs(mm) - 1;
-            mm &= mm - 1;
-            const int slot = lane * 32 + bit;
-            const unsigned e = ps[slot];
-            const int sx = slot / (kNbh * kNbh), sy = (slot / kNbh) % kNbh, sz = slot % kNbh;
-            // winner cell relative to the tile origin
-            const int wx = (sx - reach) * A.bs + (int)(e & 3u);
-            const int wy = (sy - reach) * A.bs + (int)((e >> 2) & 3u);
-            const int wz = (sz - reach) * A.bs + (int)((e >> 4) & 3u);
-            if (pos < kMaxWin)
-                M.u.win[pos] = (unsigned)(wx + 8) | ((unsigned)(wy + 8) << 5) |
-                               ((unsigned)(wz + 8) << 10) | (((e >> 6) & 1u) << 15);
-            ++pos;
-        }
-        nw = min(nw, kMaxWin);
-        __syncwarp();
-        // W of the tile's own cells
-        bool changed[2] = {false, false};
+        if (u < kNbh3 / 4 && (u & 7) == 0 && pm) pmask[u >> 3] = 0u;
+        const int n0 = M.nw[turn][0], nw = n0 + M.nw[turn][1];
+        const unsigned *win = M.win[turn][0];
+        bool changed = false;
         for (int e = 0; e < nw; ++e) {
-            const unsigned wv = M.u.win[e];
-            const int wx = (int)(wv & 31) - 8, wy = (int)((wv >> 5) & 31) - 8,
-                      wz = (int)((wv >> 10) & 31) - 8;
+            const unsigned wv = win[e < n0 ? e : e - n0 + kSlots * 32];
+            const int ax = cx + 8 - (int)(wv & 31u), ay = cy + 8 - (int)((wv >> 5) & 31u),
+                      az = 8 - (int)((wv >> 10) & 31u);
             const int sgn = ((wv >> 15) & 1u) ? -1 : 1;   // solute -> solvent lowers W
-#pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                const int rho = lane + 32 * m;
-                const int ax = (rho >> 3) - wx, ay = (rho & 7) - wy;
+            if (STENCIL) {      // full stencil: the row of weights at (ax, ay)
                 if (abs(ax) > r || abs(ay) > r) continue;
-                changed[m] = true;
-                if (STENCIL) {      // full stencil: the row of weights at (ax, ay)
-                    const int *wr = kt + ((ax + r) * (2 * r + 1) + (ay + r)) * (2 * r + 1) + r;
+                const int *wr = kt + ((ax + r) * (2 * r + 1) + (ay + r)) * kKtRow + (kKtRow >> 1) + az;
 #pragma unroll
-                    for (int z = 0; z < TS; ++z) {
-                        const int az = z - wz;
-                        if (abs(az) <= r) Wr[m][z] += (unsigned)(sgn * wr[az]);
-                    }
-                } else {
-                    const int qxy = sgn * qw[ax + r] * qw[ay + r];
+                for (int z = 0; z < TS; ++z) Wr[z] += (unsigned)(sgn * wr[z]);
+                changed = true;
+            } else {
+                const int qxy = sgn * qw[ax + kQ0] * qw[ay + kQ0];
+                if (qxy == 0) continue;
 #pragma unroll
-                    for (int z = 0; z < TS; ++z) {
-                        const int az = z - wz;
-                        if (abs(az) <= r) Wr[m][z] += (unsigned)(qxy * qw[az + r]);
-                    }
-                }
+                for (int z = 0; z < TS; ++z) Wr[z] += (unsigned)(qxy * qw[az + z + kQ0]);
+                changed = true;
             }
         }
+        if (changed && zc) {
+            if (A.vec == 2) {
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            if (!changed[m] || !rowok[m]) continue;
-            const int rho = lane + 32 * m;
-            const long long o = (long long)(i0 + (rho >> 3)) * nyz +
-                                (long long)(j0 + (rho & 7)) * g.nz + k0;
-            if (A.vec) {
-                uint4 *wp = reinterpret_cast<uint4 *>(A.W + o);
-                wp[0] = make_uint4(Wr[m][0], Wr[m][1], Wr[m][2], Wr[m][3]);
-                wp[1] = make_uint4(Wr[m][4], Wr[m][5], Wr[m][6], Wr[m][7]);
+                for (int h = 0; h < TS; h += 4)
+                    *reinterpret_cast<uint4 *>(A.W + o + h) =
+                        make_uint4(Wr[h], Wr[h + 1], Wr[h + 2], Wr[h + 3]);
             } else {
 #pragma unroll
                 for (int z = 0; z < TS; ++z)
-                    if (z < zlim) A.W[o + z] = Wr[m][z];
+                    if (z < zc) A.W[o + z] = Wr[z];
             }
         }
-        __syncwarp();
     }
 
     // ------------------------------------ candidates, dE, new leaders
-    for (int b = lane; b < nbt; b += 32) M.u.bmax[b] = 0ull;
-    int ncand = 0;
+    // dE = c [s (1 - 2w) - g0] - s h^3 U with s = 1 - 2 chi, w = W / S and
+    // g0 = k0 / S (S the sum of the kernel's weights, k0 its centre weight):
+    // the bracket is the integer N = s (S - 2W) - k0 over S, so
+    // c * bracket = c_N N with c_N = c / S and one rounding.  FP32 estimates
+    // come first and leave the FP64 unit (2 results a clock per SM) the cells
+    // that may lead their brick: an estimate is off by at most 4 ulp of
+    // |c_N N| + |h^3 U| (2.4e-7 of it), so with bounds of 1e-6 of that sum a
+    // cell whose lower bound is positive does not lower the energy, and one
+    // whose lower bound lies above another's upper bound comes after it, also
+    // in the rounded keys.  What is not finite is settled in FP64.
     {
-        unsigned cm[2], lab[2];
-        int cnt = 0;
+        const int h = (cx + 1) * 10 + cy + 1;
+        const unsigned *hr = M.hr[turn];
+        const unsigned c = hr[h];
+        const unsigned d = (c ^ hr[h - 10]) | (c ^ hr[h + 10]) | (c ^ hr[h - 1]) |
+                           (c ^ hr[h + 1]) | (c ^ (c << 1)) | (c ^ (c >> 1));
+        const unsigned cm = (d >> 1) & ((1u << zc) - 1u);
+        const unsigned lab = c >> 1;
+        unsigned open = 0u;
+        float lo[TS], best[2] = {INFINITY, INFINITY};
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            const int rho = lane + 32 * m;
-            const int x = rho >> 3, y = rho & 7;
-            const unsigned c = M.u.hr[(x + 1) * 10 + (y + 1)];
-            const unsigned d = (c ^ M.u.hr[x * 10 + (y + 1)]) |
-                               (c ^ M.u.hr[(x + 2) * 10 + (y + 1)]) |
-                               (c ^ M.u.hr[(x + 1) * 10 + y]) |
-                               (c ^ M.u.hr[(x + 1) * 10 + (y + 2)]) |
-                               (c ^ (c << 1)) | (c ^ (c >> 1));
-            cm[m] = rowok[m] ? (d >> 1) & zmask : 0u;
-            lab[m] = (c >> 1) & 0xffu;
-            cnt += __popc(cm[m]);
+        for (int z = 0; z < TS; ++z) {
+            const bool solute = (lab >> z) & 1u;
+            const int base = A.ksum - 2 * (int)Wr[z];
+            const float t1 = A.cDf * (float)((solute ? -base : base) - A.qc3), t2 = A.h3f * Ur[z];
+            const float est = solute ? t1 + t2 : t1 - t2;
+            const float err = 1e-6f * (fabsf(t1) + fabsf(t2)) + 1e-30f;
+            lo[z] = est - err;
+            if (((cm >> z) & 1u) && !(lo[z] > 0.f)) {
+                open |= 1u << z;
+                best[z >> 2] = fminf(best[z >> 2], est + err);
+            }
         }
-        int incl = cnt;   // inclusive warp scan of the counts
+        // bricks of edge 4: 16 lanes, lane bits 0, 1, 3, 4
+        if (bsh == 2) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
+            for (int m = 1; m <= 16; m = m == 2 ? 8 : 2 * m) {
+                best[0] = fminf(best[0], __shfl_xor_sync(0xffffffffu, best[0], m));
+                best[1] = fminf(best[1], __shfl_xor_sync(0xffffffffu, best[1], m));
+            }
+#pragma unroll
+            for (int z = 0; z < TS; ++z)
+                if (lo[z] > best[z >> 2]) open &= ~(1u << z);
         }
-        ncand = __shfl_sync(0xffffffffu, incl, 31);
-        int pos = incl - cnt;
-        __syncwarp();     // the slot scratch in cW is no longer read
+        while (open) {
+            const int z = __ffs(open) - 1;
+            open &= open - 1;
+            unsigned Wv = Wr[0];
+            float Uv = Ur[0];
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            const int rho = lane + 32 * m;
-#pragma unroll
-            for (int z = 0; z < TS; ++z) {
-                if ((cm[m] >> z) & 1u) {
-                    M.u.cW[pos] = Wr[m][z];
-                    M.u.cU[pos] = Ur[m][z];
-                    M.u.cP[pos] = (unsigned short)((rho << 3) | z | (((lab[m] >> z) & 1u) << 9));
-                    ++pos;
+            for (int y = 1; y < TS; ++y)
+                if (z == y) {
+                    Wv = Wr[y];
+                    Uv = Ur[y];
                 }
+            const bool solute = (lab >> z) & 1u;
+            const int base = A.ksum - 2 * (int)Wv;
+            const int N = (solute ? -base : base) - A.qc3;
+            const double t1 = __dmul_rn(A.cD, (double)N);
+            const double t2 = __dmul_rn(A.h3, (double)Uv);
+            const double e = __dadd_rn(t1, solute ? t2 : -t2);
+            if (e < 0.0) {
+                const unsigned p = o + (unsigned)z;
+                A.dE[p] = e;
+                const unsigned key = __float_as_uint(__double2float_rn(e)) & 0x7fffffffu;
+                const unsigned long long w = ((unsigned long long)key << 33) |
+                                             ((unsigned long long)~p << 1) |
+                                             (unsigned long long)solute;
+                atomicMax(&M.bmax[((cx >> bsh) * bpt + (cy >> bsh)) * bpt + (z >> bsh)], w);
             }
         }
     }
     __syncwarp();
-    // dE = c [s (1 - 2w) - g0] - s h^3 U with s = 1 - 2 chi, w = W / S and
-    // g0 = k0 / S (S the sum of the kernel's weights, k0 its centre weight):
-    // the bracket is the integer N = s (S - 2W) - k0 over S, so
-    // c * bracket = c_N N with c_N = c / S and one rounding.
-    for (int q0 = 0; q0 < ncand; q0 += 32) {
-        const int q = q0 + lane;
-        if (q >= ncand) continue;
-        const unsigned Wv = M.u.cW[q];
-        const float Uv = M.u.cU[q];
-        const unsigned cp = M.u.cP[q];
-        const int x = (cp >> 6) & 7, y = (cp >> 3) & 7, z = cp & 7;
-        const bool solute = (cp >> 9) & 1u;
-        const int base = A.ksum - 2 * (int)Wv;
-        const int N = (solute ? -base : base) - A.qc3;
-        const double t1 = __dmul_rn(A.cD, (double)N);
-        const double t2 = __dmul_rn(A.h3, (double)Uv);
-        const double e = __dadd_rn(t1, solute ? t2 : -t2);
-        if (e < 0.0) {
-            const long long p =
-                (long long)(i0 + x) * nyz + (long long)(j0 + y) * g.nz + (k0 + z);
-            A.dE[p] = e;
-            const unsigned key = __float_as_uint(__double2float_rn(e)) & 0x7fffffffu;
-            const unsigned long long w = ((unsigned long long)key << 33) |
-                                         ((0xffffffffull - (unsigned long long)p) << 1) |
-                                         (unsigned long long)solute;
-            atomicMax(&M.u.bmax[((x >> bsh) * bpt + (y >> bsh)) * bpt + (z >> bsh)], w);
-        }
-    }
-    __syncwarp();
+    turn ^= 1;
     bool any = false, changed = false;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int b = lane + 32 * h;
-        if (b >= nbt) continue;
-        const int bx = b / (bpt * bpt), by = (b / bpt) % bpt, bz = b % bpt;
-        const int gx = (i0 >> bsh) + bx, gy = (j0 >> bsh) + by, gz = (k0 >> bsh) + bz;
-        if (gx >= A.nbx || gy >= A.nby || gz >= A.nbz) continue;
-        const unsigned long long w = M.u.bmax[b];
-        const long long o = ((long long)gx * A.nby + gy) * A.nbz + gz;
-        changed |= w != oldw[h];
-        A.PL[o] = w;
-        if (w != 0ull) {
-            int ci, cj, ck;
-            leader_cell(A, w, gx, gy, gz, ci, cj, ck);
-            A.PO[o] = (uint8_t)((ci & (A.bs - 1)) | ((cj & (A.bs - 1)) << 2) |
-                                ((ck & (A.bs - 1)) << 4));
+    if (L.lane < per) {
+        const unsigned long long w = M.bmax[brick];
+        M.bmax[brick] = 0ull;
+        if (bq >= 0) {
+            changed = w != oldw;
+            any = w != 0ull;
+            A.PL[bq] = w;
+            if (any) {
+                // the leader's cell from its linear index, without a division: the
+                // offset from the brick's first cell is di nyz + dj nz + dk
+                const int gx = ti * bpt + brick / (bpt * bpt), gy = tj * bpt + (brick / bpt) % bpt,
+                          gz = tk * bpt + brick % bpt;
+                int d = (int)~(unsigned)(w >> 1) -
+                        ((gx << bsh) * nyz + (gy << bsh) * g.nz + (gz << bsh));
+                unsigned di = 0, dj = 0;
+                for (int s = 1; s < A.bs; ++s)
+                    if (d >= nyz) {
+                        d -= nyz;
+                        ++di;
+                    }
+                for (int s = 1; s < A.bs; ++s)
+                    if (d >= g.nz) {
+                        d -= g.nz;
+                        ++dj;
+                    }
+                A.PO[bq] = (uint8_t)(di | (dj << 2) | ((unsigned)d << 4));
+            }
         }
-        any |= w != 0ull;
     }
-    if (mark >= 0 && __any_sync(0xffffffffu, changed) && lane < 27) {
-        const int tk = t % A.ntz, tj = (t / A.ntz) % A.nty, ti = t / (A.ntz * A.nty);
-        const int a = ti + lane / 9 - 1, b = tj + (lane / 3) % 3 - 1, c = tk + lane % 3 - 1;
+    if (stamp && __any_sync(0xffffffffu, changed) && L.lane < 27) {
+        const int a = ti + L.lane / 9 - 1, b = tj + (L.lane / 3) % 3 - 1, c = tk + L.lane % 3 - 1;
         if (a >= 0 && b >= 0 && c >= 0 && a < A.ntx && b < A.nty && c < A.ntz)
-            A.dirty[(a * A.nty + b) * A.ntz + c] = mark;
+            set_tile_bit(A, stamp, (unsigned)((a * A.nty + b) * A.ntz + c));
     }
     return __any_sync(0xffffffffu, any);
 }
 
 struct SweepShared {
-    unsigned own[kOwnWords];   // own tile j = (t - blockIdx.x) / gridDim.x holds a leader
-    int list[kListCap];
-    int wc[NWARP];
-    int qw[2 * kMaxR + 1];
-    double e[NWARP];
-    unsigned nf[NWARP];
+    unsigned own[2][kOwnWords];    // half w of own tile j holds a leader
+    int qw[2 * kQ0];
+    double e[2 * NTEAM];
+    unsigned nf[2 * NTEAM];
     unsigned ncnt;
-    int nown;                  // own tiles holding a leader
+    int nown;                  // own half tiles holding a leader
     int abort_flag;
 };
 
-// Lists this block's tiles t = blockIdx.x + j * gridDim.x, j in [base,
-// base + kListCap), for which pick(j, t) holds, in a fixed order (thread i
-// examines j = base + i + c * SW_THREADS, c < kGatherPer, and its picks
-// follow those of threads i' < i); returns the count (list in S.list).
-// pick is called once per j < limit with t < ntiles; it may clear a flag.
-template <class Pick>
-__device__ int list_tiles(SweepShared &S, int base, int limit, long long ntiles, Pick pick)
+// Visits this team's share of the block's tiles whose bit is set in word(k),
+// k < words (bit b of word k is own tile 32 k + b): of the set bits in order,
+// team q takes numbers q, q + NTEAM, ...  Every warp holds 32 words, one per
+// lane, with a running count, and finds its next bit by rank (twelve
+// instructions a visit; walking all the bits cost every warp eight per bit).
+// Returns the number of set bits.
+template <class Word, class Visit>
+__device__ __forceinline__ int each_tile(int words, int team, Word word, Visit visit)
 {
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    if (limit - base <= SW_THREADS) {    // one tile per thread: a ballot orders them
-        const int j = base + threadIdx.x;
-        const long long t = (long long)blockIdx.x + (long long)j * gridDim.x;
-        const bool fl = j < limit && t < ntiles && pick(j, (int)t);
-        const unsigned b = __ballot_sync(0xffffffffu, fl);
-        __syncthreads();      // the previous list is no longer read
-        if (lane == 0) S.wc[wp] = __popc(b);
-        __syncthreads();
-        int off = 0, tot = 0;
-#pragma unroll
-        for (int q = 0; q < NWARP; ++q) {
-            if (q < wp) off += S.wc[q];
-            tot += S.wc[q];
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    int n = 0, next = team;
+    for (int base = 0; base < words; base += 32) {
+        const unsigned mine = base + lane < words ? word(base + lane) : 0u;
+        const int cnt = __popc(mine);
+        int upto = cnt;           // set bits of this and the lower lanes' words
+        const int held = min(words - base, 32);
+        for (int s = 1; s < held; s <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, upto, s);
+            if (lane >= s) upto += v;
         }
-        if (fl) S.list[off + __popc(b & ((1u << lane) - 1u))] = (int)t;
-        __syncthreads();
-        return tot;
+        const int total = __shfl_sync(0xffffffffu, upto, held - 1);
+        for (; next - n < total; next += NTEAM) {
+            const int want = next - n;
+            // the word holding it, then the bit of that rank in the word
+            const int l = __ffs(__ballot_sync(0xffffffffu, upto > want)) - 1;
+            const unsigned m = __shfl_sync(0xffffffffu, mine, l);
+            const int rank = want - __shfl_sync(0xffffffffu, upto - cnt, l);
+            const int bit = __ffs(__ballot_sync(0xffffffffu, ((m >> lane) & 1u) != 0u &&
+                                                                 __popc(m & below) == rank)) - 1;
+            visit(32 * (base + l) + bit);
+        }
+        n += total;
     }
+    return n;
+}
+
+// Clears a block's words of a bitmap.
+__device__ __forceinline__ void clear_words(unsigned *map, int words)
+{
+    for (int k = threadIdx.x; k < words; k += SW_THREADS) map[k] = 0u;
+}
+
+// Mask of the own tiles 32 k .. 32 k + 31 that exist among ntiles.
+__device__ __forceinline__ unsigned tile_mask(int k, int nown, long long ntiles)
+{
     unsigned m = 0u;
-#pragma unroll
-    for (int c = 0; c < kGatherPer; ++c) {
-        const int j = base + threadIdx.x + c * SW_THREADS;
-        const long long t = (long long)blockIdx.x + (long long)j * gridDim.x;
-        if (j < limit && t < ntiles && pick(j, (int)t)) m |= 1u << c;
-    }
-    const int cnt = __popc(m);
-    int incl = cnt;   // inclusive warp scan of the counts
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    __syncthreads();          // the previous list is no longer read
-    if (lane == 31) S.wc[wp] = incl;
-    __syncthreads();
-    int off = 0, tot = 0;
-#pragma unroll
-    for (int q = 0; q < NWARP; ++q) {
-        if (q < wp) off += S.wc[q];
-        tot += S.wc[q];
-    }
-    int pos = off + incl - cnt;
-#pragma unroll
-    for (int c = 0; c < kGatherPer; ++c)
-        if ((m >> c) & 1u)
-            S.list[pos++] = (int)(blockIdx.x + (long long)(base + threadIdx.x + c * SW_THREADS) *
-                                                   gridDim.x);
-    __syncthreads();
-    return tot;
+    for (int b = 0; b < 32; ++b)
+        if (32 * k + b < nown && own_tile_no(32 * k + b) < ntiles) m |= 1u << b;
+    return m;
 }
 
-// Whether own tile j holds a leader.
-__device__ __forceinline__ bool own_bit(const SweepShared &S, int j)
+// Records whether half w of own tile j holds a leader, keeping the counts.
+__device__ __forceinline__ void set_own(SweepShared &S, int w, int j, bool now, unsigned *nlead,
+                                        unsigned *nlead_sys)
 {
-    return (S.own[j >> 5] >> (j & 31)) & 1u;
-}
-
-// Records whether own tile t holds a leader, keeping the global count.
-__device__ __forceinline__ void set_own(const SweepArgs &A, SweepShared &S, int t, bool now)
-{
-    const int j = (int)((t - (int)blockIdx.x) / (int)gridDim.x);
     const unsigned bit = 1u << (j & 31);
-    const bool old = (S.own[j >> 5] & bit) != 0u;
-    if (now == old) return;
-    if (now) atomicOr(&S.own[j >> 5], bit);
-    else atomicAnd(&S.own[j >> 5], ~bit);
+    unsigned *word = &S.own[w][j >> 5];
+    if (now == ((*word & bit) != 0u)) return;
+    if (now) atomicOr(word, bit);
+    else atomicAnd(word, ~bit);
     atomicAdd(&S.nown, now ? 1 : -1);
-    red_add(A.nlead, now ? 1u : 0xffffffffu);
+    red_add(nlead, now ? 1u : 0xffffffffu);
+    if (nlead_sys) red_add(nlead_sys, now ? 1u : 0xffffffffu);
+}
+
+// Shared set-up of a sweep block: weights, stencil, counters, team areas.
+__device__ __forceinline__ void sweep_init(SweepShared &S, TeamMem *TM, int *kt,
+                                           const KernelW &kw, const int *k3)
+{
+    if (kt) {
+        const int w = 2 * kw.r + 1;
+        for (int a = threadIdx.x; a < w * w * kKtRow; a += SW_THREADS) {
+            const int row = a / kKtRow, z = a - row * kKtRow - (kKtRow >> 1);
+            kt[a] = abs(z) <= kw.r ? k3[row * w + z + kw.r] : 0;
+        }
+    }
+    for (int a = threadIdx.x; a < 2 * kQ0; a += SW_THREADS) {
+        const int d = a - kQ0;
+        S.qw[a] = abs(d) <= kw.r ? kw.q[d + kw.r] : 0;
+    }
+    for (int a = threadIdx.x; a < 2 * kOwnWords; a += SW_THREADS)
+        S.own[a / kOwnWords][a % kOwnWords] = 0u;
+    for (int a = threadIdx.x; a < NTEAM * kMaxBricksPerTile; a += SW_THREADS)
+        TM[a / kMaxBricksPerTile].bmax[a % kMaxBricksPerTile] = 0ull;
+    if (threadIdx.x == 0) {
+        S.abort_flag = 0;
+        S.ncnt = 1u;
+        S.nown = 0;
+    }
+    __syncthreads();
 }
 
 template <bool STENCIL>
@@ -858,42 +849,35 @@ k_sweep(SweepArgs A)
 {
     __shared__ SweepShared S;
     extern __shared__ __align__(16) unsigned char dyn[];
-    WarpMem *WM = reinterpret_cast<WarpMem *>(dyn);
+    TeamMem *TM = reinterpret_cast<TeamMem *>(dyn);
+    // the full stencil, if any, follows the teams' areas
+    int *kt = STENCIL ? reinterpret_cast<int *>(dyn + NTEAM * sizeof(TeamMem)) : nullptr;
     const int ntiles = A.ntx * A.nty * A.ntz;
-    const int per_block = (ntiles + gridDim.x - 1) / gridDim.x;
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    WarpMem &M = WM[wp];
-    // the full stencil, if any, follows the warps' areas
-    int *kt = STENCIL ? reinterpret_cast<int *>(dyn + NWARP * sizeof(WarpMem)) : nullptr;
-    if (STENCIL) {
-        const int w = 2 * A.kw.r + 1;
-        for (int a = threadIdx.x; a < w * w * w; a += SW_THREADS) kt[a] = A.k3[a];
-    }
-    for (int a = threadIdx.x; a <= 2 * A.kw.r; a += SW_THREADS) S.qw[a] = A.kw.q[a];
-    for (int a = threadIdx.x; a < kOwnWords; a += SW_THREADS) S.own[a] = 0u;
-    if (threadIdx.x == 0) {
-        S.abort_flag = 0;
-        S.ncnt = 1u;
-        S.nown = 0;
-    }
-    __syncthreads();
-    unsigned target = 0;      // thread 0: arrivals the next barrier waits for
+    const int nown = (ntiles + (int)gridDim.x - 1) / (int)gridDim.x;    // or one fewer
+    const int words = (nown + 31) / 32;
+    const int team = threadIdx.x / TEAM;
+    TeamMem &M = TM[team];
+    const Lane L = make_lane(TS >> A.bsh, A.reach);
+    unsigned *upd = A.upd + (size_t)blockIdx.x * A.bwords;
+    unsigned *stamp = A.stamp + (size_t)blockIdx.x * A.bwords;
+    sweep_init(S, TM, kt, A.kw, A.k3);
+    Barrier B{A.bar, 0u, A.err, A.spin_limit};
+    auto own_tile = [&](int j) { return make_tile(A, (int)own_tile_no(j)); };
+    int turn = 0, uturn = 0;
     double e_lane = 0.0;
     unsigned n_lane = 0;
-    unsigned long long t_dec = 0, t_upd = 0;   // thread 0: tiles visited per phase
+    unsigned long long t_dec = 0, t_upd = 0;   // tiles visited per phase
     int round = 0, capped = 0;
     bool marked = false;      // the last update stamped the tiles to decide
     // opening pass: leaders of the starting labels
-    for (int base = 0; base < per_block; base += kListCap) {
-        const int n = list_tiles(S, base, per_block, ntiles, [](int, int) { return true; });
-        for (int q = wp; q < n; q += NWARP) {
-            const int t = S.list[q];
-            const bool now = tile_update<STENCIL>(A, M, S.qw, kt, t, true, -1);
-            if (lane == 0) set_own(A, S, t, now);
-        }
-    }
-    if (!grid_barrier(A.bar, A.err, A.spin_limit, target, &S.abort_flag)) return;
-    for (int k = 0;; ++k) {
+    each_tile(words, team, [&](int k) { return tile_mask(k, nown, ntiles); }, [&](int j) {
+        const bool now =
+            tile_update<STENCIL>(A, M, S.qw, kt, L, team, own_tile(j), true, nullptr, uturn);
+        if (L.lane == 0) set_own(S, L.w, j, now, A.nlead, nullptr);
+    });
+    bool ok = all_blocks(B, &S.abort_flag);
+    for (int k = 0; ok; ++k) {
+        const unsigned here = (k & 1) * A.mapw, last = A.mapw - here;
         if (k >= A.max_rounds) {     // cap reached: capped if leaders are left
             round = k;
             capped = -1;
@@ -903,55 +887,53 @@ k_sweep(SweepArgs A)
         // changes in the update phases)
         unsigned nl = 1u;
         if (threadIdx.x == 0) nl = ld_relaxed_u32(A.nlead);
-        const bool stamped = marked && (A.stamps > 0 || S.nown > NWARP);
-        for (int base = 0; base < per_block; base += kListCap) {
-            const int n = list_tiles(S, base, per_block, ntiles, [&](int j, int t) {
-                return own_bit(S, j) && (!stamped || __ldcg(A.dirty + t) == k);
+        const bool stamped = marked && (A.stamps > 0 || S.nown > 2 * NTEAM);
+        t_dec += (unsigned long long)each_tile(
+            words, team,
+            [&](int w) {
+                const unsigned own = S.own[0][w] | S.own[1][w];
+                return stamped ? own & __ldcg(stamp + last + w) : own;
+            },
+            [&](int j) {
+                tile_decide(A, M, L, team, own_tile(j), turn, A.upd + here, e_lane, n_lane);
             });
-            t_dec += (unsigned long long)n;
-            for (int q = wp; q < n; q += NWARP) tile_decide(A, M, S.list[q], e_lane, n_lane);
-        }
+        clear_words(upd + last, words);
         if (threadIdx.x == 0) S.ncnt = nl;
-        __syncthreads();
+        ok = all_blocks(B, &S.abort_flag);
+        if (!ok) break;
+        // (S.ncnt: the leader half tiles of this round, alike in every block)
         if (S.ncnt == 0u) {          // no leader was left: converged
             round = k;
             break;
         }
-        if (!grid_barrier(A.bar, A.err, A.spin_limit, target, &S.abort_flag)) return;
-        // update (S.ncnt: the leader tiles of this round, alike in every block)
-        marked = A.stamps > 0 || (A.stamps < 0 && S.ncnt > (unsigned)(NWARP * gridDim.x));
-        const int mark = marked ? k + 1 : -1;
-        for (int base = 0; base < per_block; base += kListCap) {
-            const int n = list_tiles(S, base, per_block, ntiles, [&](int, int t) {
-                const bool f = __ldcg(A.upd + t) != 0;
-                if (f) A.upd[t] = 0;
-                return f;
+        if (marked) clear_words(stamp + last, words);
+        marked = A.stamps > 0 || (A.stamps < 0 && S.ncnt > (unsigned)(2 * NTEAM * gridDim.x));
+        unsigned *mark = marked ? A.stamp + here : nullptr;
+        t_upd += (unsigned long long)each_tile(
+            words, team, [&](int w) { return __ldcg(upd + here + w); }, [&](int j) {
+                const bool now =
+                    tile_update<STENCIL>(A, M, S.qw, kt, L, team, own_tile(j), false, mark, uturn);
+                if (L.lane == 0) set_own(S, L.w, j, now, A.nlead, nullptr);
             });
-            t_upd += (unsigned long long)n;
-            for (int q = wp; q < n; q += NWARP) {
-                const int t = S.list[q];
-                const bool now = tile_update<STENCIL>(A, M, S.qw, kt, t, false, mark);
-                if (lane == 0) set_own(A, S, t, now);
-            }
-        }
-        if (!grid_barrier(A.bar, A.err, A.spin_limit, target, &S.abort_flag)) return;
+        ok = all_blocks(B, &S.abort_flag);
     }
-    // FP64 sums of the flipped cells' dE and their counts: lanes, then warps
-    // in order
+    if (!ok) return;
+    // FP64 sums of the flipped cells' dE and their counts: the lanes of the
+    // warps, then the warps in order
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         e_lane += __shfl_down_sync(0xffffffffu, e_lane, o);
         n_lane += __shfl_down_sync(0xffffffffu, n_lane, o);
     }
-    if (lane == 0) {
-        S.e[wp] = e_lane;
-        S.nf[wp] = n_lane;
+    if (L.lane == 0) {
+        S.e[threadIdx.x >> 5] = e_lane;
+        S.nf[threadIdx.x >> 5] = n_lane;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         double te = 0.0;
         unsigned long long tf = 0;
-        for (int q = 0; q < NWARP; ++q) {
+        for (int q = 0; q < 2 * NTEAM; ++q) {
             te += S.e[q];
             tf += S.nf[q];
         }
@@ -966,18 +948,29 @@ k_sweep(SweepArgs A)
     }
 }
 
-__global__ void k_sweep_final(const unsigned long long *part_flips,
-                              const double *part_dE, const unsigned long long *part_tiles,
-                              int nb, const int *rounds, const int *capped, RoundState *rs)
+// Totals over the blocks, one warp: lane l adds blocks l, l + 32, ... in
+// order, then a fixed tree (one thread adding 152 blocks took 26 us).
+__global__ void __launch_bounds__(32)
+k_sweep_final(const unsigned long long *part_flips, const double *part_dE,
+              const unsigned long long *part_tiles, int nb, const int *rounds, const int *capped,
+              RoundState *rs)
 {
     unsigned long long f = 0, td = 0, tu = 0;
     double e = 0.0;
-    for (int b = 0; b < nb; ++b) {
+    for (int b = threadIdx.x; b < nb; b += 32) {
         f += part_flips[b];
         e += part_dE[b];
         td += part_tiles[b];
         tu += part_tiles[nb + b];
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        f += __shfl_down_sync(0xffffffffu, f, o);
+        e += __shfl_down_sync(0xffffffffu, e, o);
+        td += __shfl_down_sync(0xffffffffu, td, o);
+        tu += __shfl_down_sync(0xffffffffu, tu, o);
+    }
+    if (threadIdx.x) return;
     rs->tiles_decide = td;
     rs->tiles_update = tu;
     rs->done = 1;
@@ -994,7 +987,7 @@ int sweep_tiles(const GridDesc &g)
     return ((g.nx + TS - 1) / TS) * ((g.ny + TS - 1) / TS) * ((g.nz + TS - 1) / TS);
 }
 
-int sweep_brick_edge(int r) { return r >= 3 ? 4 : 2; }
+int sweep_brick_edge(int r) { return sweep_edge(r); }
 
 long long sweep_bricks(const GridDesc &g, int r)
 {
@@ -1004,14 +997,20 @@ long long sweep_bricks(const GridDesc &g, int r)
 
 static size_t pad256(size_t x) { return (x + 255) / 256 * 256; }
 
-// Sweep state: leader words, leader offsets, the per-tile posting areas,
-// the update flags, the decide stamps and the label bits.
+// Words per block of a bitmap over nt tiles, and bytes of the bitmap, for a
+// grid of `blocks` blocks (at most kMaxSweepBlocks).
+constexpr int kMaxSweepBlocks = 256;
+static int bitmap_words(size_t nt, int blocks) { return (int)((nt + 32ull * blocks - 1) / (32ull * blocks)); }
+static size_t bitmap_bytes_max(size_t nt) { return pad256((nt / 32 + 2 * kMaxSweepBlocks) * 4); }
+
+// Sweep state: leader words, leader offsets, the per-tile posting areas, the
+// update and stamp bitmaps and the label bits.
 size_t sweep_state_bytes(const GridDesc &g, int r)
 {
     const size_t nt = (size_t)sweep_tiles(g);
     const size_t nb = (size_t)sweep_bricks(g, r);
     const size_t nzw = ((size_t)g.nz + 31) / 32;
-    return nb * 8 + pad256(nb) + nt * kPostBytes + pad256(nt) + pad256(nt * 4) +
+    return nb * 8 + pad256(nb) + nt * kPostBytes + 4 * bitmap_bytes_max(nt) +
            (size_t)g.nx * g.ny * nzw * 4;
 }
 
@@ -1041,48 +1040,45 @@ __global__ void k_pack_labels(const uint8_t *__restrict__ chi, int nz, long long
     CB[w] = b;
 }
 
-// warps' areas plus room for the largest full stencil ((2 * 8 + 1)^3 ints)
+// teams' areas plus room for the largest full stencil (17^2 rows)
 constexpr size_t kSweepSmem =
-    NWARP * sizeof(WarpMem) + sizeof(int) * (2 * kMaxR + 1) * (2 * kMaxR + 1) * (2 * kMaxR + 1);
+    NTEAM * sizeof(TeamMem) + sizeof(int) * (2 * kMaxR + 1) * (2 * kMaxR + 1) * kKtRow;
 
 cudaError_t sweep_grid_size(int nsm, int r, int *blocks)
 {
     (void)r;
-    cudaError_t e = cudaFuncSetAttribute(k_sweep<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSweepSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_sweep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kSweepSmem);
-    if (e != cudaSuccess) return e;
-    int per = 0, per2 = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sweep<false>, SW_THREADS,
-                                                      kSweepSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per2, k_sweep<true>, SW_THREADS,
-                                                      kSweepSmem);
-    if (e != cudaSuccess) return e;
-    per = per2 < per ? per2 : per;
-    per = per > VESIS_SWEEP_BPS ? VESIS_SWEEP_BPS : per;
-    *blocks = per * nsm;
+    cudaError_t e = cudaSuccess;
+    int per = 1;          // one block per SM: a barrier of few blocks
+    for (int q = 0; q < 2; ++q) {
+        void *fn = q ? (void *)k_sweep<true> : (void *)k_sweep<false>;
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmem);
+        if (e != cudaSuccess) return e;
+        int n = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, SW_THREADS, kSweepSmem);
+        if (e != cudaSuccess) return e;
+        per = n < per ? n : per;
+    }
+    *blocks = per * nsm < kMaxSweepBlocks ? per * nsm : kMaxSweepBlocks;
     return *blocks > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
-int sweep_ctl_words() { return 3 * kLine; }
+int sweep_ctl_words() { return kCtlWords; }
 
 // Arguments of one system's sweep, with its set-up enqueued on st: the
-// posting bitmaps, update flags and control words cleared and the label
-// bits packed (leader words are all rewritten by the opening pass).
+// posting bitmaps and control words cleared and the label bits packed (leader
+// words are all rewritten by the opening pass).
 static SweepArgs sweep_setup(const GridDesc &g, const KernelW &kw, const int *k3,
                              const FlipConst &fc, uint8_t *chi, uint32_t *W, const float *U,
                              double *dE, void *state, unsigned *ctl, int *err, int max_rounds,
-                             long long spin_limit, cudaStream_t st)
+                             int blocks, long long spin_limit, cudaStream_t st)
 {
     SweepArgs A;
     A.g = g;
     A.kw = kw;
     A.cD = fc.cN;
     A.h3 = fc.h3;
+    A.cDf = (float)fc.cN;
+    A.h3f = (float)fc.h3;
     A.qc3 = fc.k0;
     A.ksum = fc.S;
     A.k3 = k3;
@@ -1099,16 +1095,26 @@ static SweepArgs sweep_setup(const GridDesc &g, const KernelW &kw, const int *k3
     A.nbx = (g.nx + A.bs - 1) / A.bs;
     A.nby = (g.ny + A.bs - 1) / A.bs;
     A.nbz = (g.nz + A.bs - 1) / A.bs;
-    A.vec = (g.nz % TS == 0) && ((uintptr_t)W % 16 == 0) && ((uintptr_t)U % 16 == 0);
+    A.vec = (uintptr_t)W % 16 || (uintptr_t)U % 16 ? 0 : g.nz % TS == 0 ? 2 : 1;
+    A.ncell = (unsigned)g.nx * (unsigned)(g.ny * g.nz);
     const size_t nb = (size_t)A.nbx * A.nby * A.nbz;
     const size_t nt = (size_t)A.ntx * A.nty * A.ntz;
     uint8_t *base = static_cast<uint8_t *>(state);
     A.PL = reinterpret_cast<unsigned long long *>(base);
     A.PO = base + nb * 8;
     A.post = A.PO + pad256(nb);
-    A.upd = A.post + nt * kPostBytes;
-    A.dirty = reinterpret_cast<int *>(A.upd + pad256(nt));
-    A.CB = reinterpret_cast<unsigned *>(A.upd + pad256(nt) + pad256(nt * 4));
+    uint8_t *maps = A.post + nt * kPostBytes;
+    A.upd = reinterpret_cast<unsigned *>(maps);
+    A.stamp = reinterpret_cast<unsigned *>(maps + 2 * bitmap_bytes_max(nt));
+    A.CB = reinterpret_cast<unsigned *>(maps + 4 * bitmap_bytes_max(nt));
+    A.mapw = (unsigned)(bitmap_bytes_max(nt) / 4);
+    A.bwords = bitmap_words(nt, blocks);
+    A.tile0 = 0;
+    A.nblk = (unsigned)blocks;
+    auto inv = [](int d) { return (unsigned)(((1ull << 32) + d - 1) / d); };
+    A.nblk_inv = inv(blocks);
+    A.nty_inv = inv(A.nty);
+    A.ntz_inv = inv(A.ntz);
     A.nzw = (g.nz + 31) / 32;
     A.nlead = ctl;
     A.bar = ctl + kLine;
@@ -1126,8 +1132,7 @@ static SweepArgs sweep_setup(const GridDesc &g, const KernelW &kw, const int *k3
     A.tile_nf = nullptr;
     // postings start empty (a slot is only read under its bitmap bit)
     cudaMemset2DAsync(A.post + kPostMaskOff, kPostBytes, 0, 32, nt, st);
-    cudaMemsetAsync(A.upd, 0, nt, st);
-    cudaMemsetAsync(A.dirty, 0, nt * 4, st);
+    cudaMemsetAsync(maps, 0, 4 * bitmap_bytes_max(nt), st);
     cudaMemsetAsync(ctl, 0, sweep_ctl_words() * sizeof(unsigned), st);
     cudaMemsetAsync(err, 0, sizeof(int), st);
     {
@@ -1152,7 +1157,7 @@ cudaError_t launch_sweep(const GridDesc &g, const KernelW &kw, const int *k3,
         const size_t nt = (size_t)sweep_tiles(g);
         if ((nt + blocks - 1) / blocks > (size_t)kOwnWords * 32) return cudaErrorInvalidValue;
     }
-    SweepArgs A = sweep_setup(g, kw, k3, fc, chi, W, U, dE, state, ctl, err, max_rounds,
+    SweepArgs A = sweep_setup(g, kw, k3, fc, chi, W, U, dE, state, ctl, err, max_rounds, blocks,
                               spin_limit, st);
     A.part_flips = part_flips;
     A.part_dE = part_dE;
@@ -1162,12 +1167,12 @@ cudaError_t launch_sweep(const GridDesc &g, const KernelW &kw, const int *k3,
     A.stamps = stamps;
     void *args[] = {&A};
     count_launch();
-    cudaError_t e = cudaLaunchCooperativeKernel(k3 ? (void *)k_sweep<true> : (void *)k_sweep<false>,
-                                                dim3(blocks),
-                                                dim3(SW_THREADS), args, kSweepSmem, st);
+    void *fn = k3 ? (void *)k_sweep<true> : (void *)k_sweep<false>;
+    const cudaError_t e =
+        cudaLaunchCooperativeKernel(fn, dim3(blocks), dim3(SW_THREADS), args, kSweepSmem, st);
     if (e != cudaSuccess) return e;
     count_launch();
-    k_sweep_final<<<1, 1, 0, st>>>(part_flips, part_dE, part_tiles, blocks, rounds, capped, rs);
+    k_sweep_final<<<1, 32, 0, st>>>(part_flips, part_dE, part_tiles, blocks, rounds, capped, rs);
     return cudaGetLastError();
 }
 
@@ -1181,8 +1186,8 @@ cudaError_t launch_sweep(const GridDesc &g, const KernelW &kw, const int *k3,
 // exactly as in the single-system sweep, so each system goes through the
 // same rounds as alone.  A system whose leaders are gone contributes no
 // tiles; the launch ends when no system has any.  The FP64 sum of a tile's
-// flipped dE is kept per tile (the tile's warp adds it, round after round)
-// and summed over the system's tiles in tile order at the end.
+// flipped dE is kept per half tile (its warp adds it, round after round) and
+// summed over the system's half tiles in order at the end.
 
 // dynamic shared memory offset of the systems' arguments (16-byte aligned)
 constexpr size_t kSweepSysOff = (kSweepSmem + 15) / 16 * 16;
@@ -1192,11 +1197,14 @@ struct MultiArgs {
     const long long *toff;    // [nsys + 1]: first global tile of each system
     int nsys;
     int ntiles;
-    unsigned *nlead;          // tiles holding a leader, all systems (own line)
+    unsigned *nlead;          // half tiles holding a leader, all systems (own line)
     unsigned *bar;            // grid barrier arrivals (own line)
     int *err;
     int *rounds;              // [nsys]
     int *capped;              // [nsys]
+    unsigned *upd, *stamp;    // bitmaps over all systems' tiles, two of each
+    int bwords;
+    unsigned mapw;
     int max_rounds;
     long long spin_limit;
     int stamps;               // as SweepArgs::stamps, for all systems
@@ -1215,34 +1223,6 @@ __device__ __forceinline__ int sys_of(const long long *toff, int nsys, long long
     return lo;
 }
 
-// The block's tiles that received a winner, over the global tile numbers,
-// each flag read (and cleared) in its own system's update flags.
-__device__ int gather_tiles_multi(SweepShared &S, const SweepArgs *sys, const long long *toff,
-                                  int nsys, int base, int per_block, int ntiles)
-{
-    return list_tiles(S, base, per_block, ntiles, [&](int, int t) {
-        const int q = sys_of(toff, nsys, t);
-        uint8_t *f = sys[q].upd + (t - toff[q]);
-        const bool fl = __ldcg(f) != 0;
-        if (fl) *f = 0;
-        return fl;
-    });
-}
-
-__device__ __forceinline__ void set_own_multi(SweepShared &S, long long tg, bool now,
-                                              unsigned *nlead_all, unsigned *nlead_sys)
-{
-    const int j = (int)((tg - (long long)blockIdx.x) / (long long)gridDim.x);
-    const unsigned bit = 1u << (j & 31);
-    const bool old = (S.own[j >> 5] & bit) != 0u;
-    if (now == old) return;
-    if (now) atomicOr(&S.own[j >> 5], bit);
-    else atomicAnd(&S.own[j >> 5], ~bit);
-    atomicAdd(&S.nown, now ? 1 : -1);
-    red_add(nlead_all, now ? 1u : 0xffffffffu);
-    red_add(nlead_sys, now ? 1u : 0xffffffffu);
-}
-
 template <bool STENCIL>
 __global__ void __launch_bounds__(SW_THREADS, 1)
 k_sweep_multi(MultiArgs P)
@@ -1251,51 +1231,51 @@ k_sweep_multi(MultiArgs P)
     __shared__ long long s_toff[kMaxSweepSys + 1];
     __shared__ int s_rounds[kMaxSweepSys];
     extern __shared__ __align__(16) unsigned char dyn[];
-    WarpMem *WM = reinterpret_cast<WarpMem *>(dyn);
-    // after the warps' areas and the stencil: the systems' arguments
+    TeamMem *TM = reinterpret_cast<TeamMem *>(dyn);
+    int *kt = STENCIL ? reinterpret_cast<int *>(dyn + NTEAM * sizeof(TeamMem)) : nullptr;
+    // after the teams' areas and the stencil: the systems' arguments
     SweepArgs *s_sys = reinterpret_cast<SweepArgs *>(dyn + kSweepSysOff);
-    const int ntiles = P.ntiles, nsys = P.nsys;
-    const int per_block = (ntiles + gridDim.x - 1) / gridDim.x;
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    WarpMem &M = WM[wp];
-    int *kt = STENCIL ? reinterpret_cast<int *>(dyn + NWARP * sizeof(WarpMem)) : nullptr;
-    if (STENCIL) {
-        const int w = 2 * P.kw.r + 1;
-        for (int a = threadIdx.x; a < w * w * w; a += SW_THREADS) kt[a] = P.k3[a];
-    }
+    const int nsys = P.nsys;
+    const int nown = (P.ntiles + (int)gridDim.x - 1) / (int)gridDim.x;      // or one fewer
+    const int words = (nown + 31) / 32;
+    const int team = threadIdx.x / TEAM;
+    TeamMem &M = TM[team];
     {
-        const int words = nsys * (int)(sizeof(SweepArgs) / 4);
+        const int nwords = nsys * (int)(sizeof(SweepArgs) / 4);
         const unsigned *src = reinterpret_cast<const unsigned *>(P.sys);
         unsigned *dst = reinterpret_cast<unsigned *>(s_sys);
-        for (int a = threadIdx.x; a < words; a += SW_THREADS) dst[a] = src[a];
+        for (int a = threadIdx.x; a < nwords; a += SW_THREADS) dst[a] = src[a];
     }
-    for (int a = threadIdx.x; a <= 2 * P.kw.r; a += SW_THREADS) S.qw[a] = P.kw.q[a];
-    for (int a = threadIdx.x; a < kOwnWords; a += SW_THREADS) S.own[a] = 0u;
     for (int a = threadIdx.x; a <= nsys; a += SW_THREADS) s_toff[a] = P.toff[a];
     for (int a = threadIdx.x; a < nsys; a += SW_THREADS) s_rounds[a] = 0;
-    if (threadIdx.x == 0) {
-        S.abort_flag = 0;
-        S.ncnt = 1u;
-        S.nown = 0;
-    }
-    __syncthreads();
-    unsigned target = 0;
-    int capped = 0;
+    sweep_init(S, TM, kt, P.kw, P.k3);
+    unsigned *upd = P.upd + (size_t)blockIdx.x * P.bwords;
+    unsigned *stamp = P.stamp + (size_t)blockIdx.x * P.bwords;
+    const Lane L = make_lane(TS / sweep_edge(P.kw.r), (P.kw.r + sweep_edge(P.kw.r) - 1) / sweep_edge(P.kw.r));
+    Barrier B{P.bar, 0u, P.err, P.spin_limit};
+    // own tile j: its system, and its number there
+    auto own_sys = [&](int j, int &t) {
+        const long long tg = own_tile_no(j);
+        const int q = sys_of(s_toff, nsys, tg);
+        t = (int)(tg - s_toff[q]);
+        return q;
+    };
+    int uturn = 0;
+    auto update = [&](int j, bool first, unsigned *mark) {
+        int t;
+        const SweepArgs &A = s_sys[own_sys(j, t)];
+        const bool now =
+            tile_update<STENCIL>(A, M, S.qw, kt, L, team, make_tile(A, t), first, mark, uturn);
+        if (L.lane == 0) set_own(S, L.w, j, now, P.nlead, A.nlead);
+    };
+    int capped = 0, turn = 0;
     bool marked = false;
     // opening pass: leaders of every system's starting labels
-    for (int base = 0; base < per_block; base += kListCap) {
-        const int n = list_tiles(S, base, per_block, ntiles, [](int, int) { return true; });
-        for (int q = wp; q < n; q += NWARP) {
-            const int tg = S.list[q];
-            const int sq = sys_of(s_toff, nsys, tg);
-            const SweepArgs &A = s_sys[sq];
-            const bool now =
-                tile_update<STENCIL>(A, M, S.qw, kt, (int)(tg - s_toff[sq]), true, -1);
-            if (lane == 0) set_own_multi(S, tg, now, P.nlead, A.nlead);
-        }
-    }
-    if (!grid_barrier(P.bar, P.err, P.spin_limit, target, &S.abort_flag)) return;
+    each_tile(words, team, [&](int k) { return tile_mask(k, nown, P.ntiles); },
+              [&](int j) { update(j, true, nullptr); });
+    if (!all_blocks(B, &S.abort_flag)) return;
     for (int k = 0;; ++k) {
+        const unsigned here = (k & 1) * P.mapw, last = P.mapw - here;
         if (k >= P.max_rounds) {
             capped = 1;
             break;
@@ -1305,51 +1285,41 @@ k_sweep_multi(MultiArgs P)
         if (blockIdx.x == 0)         // rounds of each system that still had leaders
             for (int q = threadIdx.x; q < nsys; q += SW_THREADS)
                 if (ld_relaxed_u32(s_sys[q].nlead) != 0u) s_rounds[q] = k + 1;
-        const bool stamped = marked && (P.stamps > 0 || S.nown > NWARP);
-        for (int base = 0; base < per_block; base += kListCap) {
-            const int n = list_tiles(S, base, per_block, ntiles, [&](int j, int tg) {
-                if (!own_bit(S, j)) return false;
-                if (!stamped) return true;
-                const int sq = sys_of(s_toff, nsys, tg);
-                return __ldcg(s_sys[sq].dirty + (tg - s_toff[sq])) == k;
-            });
-            for (int q = wp; q < n; q += NWARP) {
-                const int tg = S.list[q];
-                const int sq = sys_of(s_toff, nsys, tg);
-                const SweepArgs &A = s_sys[sq];
-                const int t = (int)(tg - s_toff[sq]);
+        const bool stamped = marked && (P.stamps > 0 || S.nown > 2 * NTEAM);
+        each_tile(
+            words, team,
+            [&](int w) {
+                const unsigned own = S.own[0][w] | S.own[1][w];
+                return stamped ? own & __ldcg(stamp + last + w) : own;
+            },
+            [&](int j) {
+                int t;
+                const SweepArgs &A = s_sys[own_sys(j, t)];
                 double e = 0.0;
                 unsigned nf = 0;
-                tile_decide(A, M, t, e, nf);
+                tile_decide(A, M, L, team, make_tile(A, t), turn, P.upd + here, e, nf);
+                if (__any_sync(0xffffffffu, nf != 0u)) {
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    e += __shfl_down_sync(0xffffffffu, e, o);
-                    nf += __shfl_down_sync(0xffffffffu, nf, o);
+                    for (int o = 16; o > 0; o >>= 1) {
+                        e += __shfl_down_sync(0xffffffffu, e, o);
+                        nf += __shfl_down_sync(0xffffffffu, nf, o);
+                    }
+                    if (L.lane == 0) {
+                        A.tile_dE[2 * t + L.w] += e;
+                        A.tile_nf[2 * t + L.w] += nf;
+                    }
                 }
-                if (lane == 0 && nf) {
-                    A.tile_dE[t] += e;
-                    A.tile_nf[t] += nf;
-                }
-            }
-        }
+            });
+        clear_words(upd + last, words);
         if (threadIdx.x == 0) S.ncnt = nl;
-        __syncthreads();
+        if (!all_blocks(B, &S.abort_flag)) return;
         if (S.ncnt == 0u) break;
-        if (!grid_barrier(P.bar, P.err, P.spin_limit, target, &S.abort_flag)) return;
-        marked = P.stamps > 0 || (P.stamps < 0 && S.ncnt > (unsigned)(NWARP * gridDim.x));
-        const int mark = marked ? k + 1 : -1;
-        for (int base = 0; base < per_block; base += kListCap) {
-            const int n = gather_tiles_multi(S, s_sys, s_toff, nsys, base, per_block, ntiles);
-            for (int q = wp; q < n; q += NWARP) {
-                const int tg = S.list[q];
-                const int sq = sys_of(s_toff, nsys, tg);
-                const SweepArgs &A = s_sys[sq];
-                const bool now =
-                    tile_update<STENCIL>(A, M, S.qw, kt, (int)(tg - s_toff[sq]), false, mark);
-                if (lane == 0) set_own_multi(S, tg, now, P.nlead, A.nlead);
-            }
-        }
-        if (!grid_barrier(P.bar, P.err, P.spin_limit, target, &S.abort_flag)) return;
+        if (marked) clear_words(stamp + last, words);
+        marked = P.stamps > 0 || (P.stamps < 0 && S.ncnt > (unsigned)(2 * NTEAM * gridDim.x));
+        unsigned *mark = marked ? P.stamp + here : nullptr;
+        each_tile(words, team, [&](int w) { return __ldcg(upd + here + w); },
+                  [&](int j) { update(j, false, mark); });
+        if (!all_blocks(B, &S.abort_flag)) return;
     }
     if (blockIdx.x == 0) {
         __syncthreads();
@@ -1368,7 +1338,7 @@ __global__ void __launch_bounds__(256) k_sweep_multi_final(const SweepArgs *sys,
     __shared__ double se[256];
     __shared__ unsigned long long sf[256];
     const SweepArgs &A = sys[blockIdx.x];
-    const int nt = A.ntx * A.nty * A.ntz;
+    const int nt = 2 * A.ntx * A.nty * A.ntz;
     double e = 0.0;
     unsigned long long f = 0;
     for (int t = threadIdx.x; t < nt; t += 256) {
@@ -1401,11 +1371,11 @@ __global__ void __launch_bounds__(256) k_sweep_multi_final(const SweepArgs *sys,
 
 static size_t pad256z(size_t x) { return (x + 255) / 256 * 256; }
 
-size_t sweep_multi_scratch_bytes(int nsys)
+size_t sweep_multi_scratch_bytes(int nsys, long long tiles)
 {
     return pad256z((size_t)nsys * sizeof(SweepArgs)) + pad256z((size_t)(nsys + 1) * 8) +
-           pad256z(3 * kLine * sizeof(unsigned)) + pad256z(sizeof(int)) +
-           2 * pad256z((size_t)nsys * sizeof(int));
+           pad256z(kCtlWords * sizeof(unsigned)) + pad256z(sizeof(int)) +
+           2 * pad256z((size_t)nsys * sizeof(int)) + 4 * bitmap_bytes_max((size_t)tiles);
 }
 
 cudaError_t launch_sweep_multi(int nsys, const SweepSys *sys, const KernelW &kw, const int *k3,
@@ -1420,12 +1390,12 @@ cudaError_t launch_sweep_multi(int nsys, const SweepSys *sys, const KernelW &kw,
         const int nt = sweep_tiles(y.g);
         toff[q + 1] = toff[q] + nt;
         As[q] = sweep_setup(y.g, kw, k3, y.fc, y.chi, y.W, y.U, y.dE, y.state, y.ctl, y.err,
-                            max_rounds, spin_limit, y.st);
+                            max_rounds, blocks, spin_limit, y.st);
         As[q].rs = y.rs;
         As[q].tile_dE = y.tile_dE;
         As[q].tile_nf = y.tile_nf;
-        cudaMemsetAsync(y.tile_dE, 0, (size_t)nt * sizeof(double), y.st);
-        cudaMemsetAsync(y.tile_nf, 0, (size_t)nt * sizeof(unsigned), y.st);
+        cudaMemsetAsync(y.tile_dE, 0, (size_t)2 * nt * sizeof(double), y.st);
+        cudaMemsetAsync(y.tile_nf, 0, (size_t)2 * nt * sizeof(unsigned), y.st);
     }
     if (toff[nsys] > 0x7fffffffll ||
         (toff[nsys] + blocks - 1) / blocks > (long long)kOwnWords * 32)
@@ -1445,15 +1415,29 @@ cudaError_t launch_sweep_multi(int nsys, const SweepSys *sys, const KernelW &kw,
     long long *d_toff = reinterpret_cast<long long *>(b);
     b += pad256z((size_t)(nsys + 1) * 8);
     unsigned *d_ctl = reinterpret_cast<unsigned *>(b);
-    b += pad256z(3 * kLine * sizeof(unsigned));
+    b += pad256z(kCtlWords * sizeof(unsigned));
     int *d_err = reinterpret_cast<int *>(b);
     b += pad256z(sizeof(int));
     int *d_rounds = reinterpret_cast<int *>(b);
     b += pad256z((size_t)nsys * sizeof(int));
     int *d_capped = reinterpret_cast<int *>(b);
+    b += pad256z((size_t)nsys * sizeof(int));
+    // the tiles of all systems share the launch's two bitmaps
+    const size_t map_bytes = bitmap_bytes_max((size_t)toff[nsys]);
+    unsigned *d_upd = reinterpret_cast<unsigned *>(b);
+    unsigned *d_stamp = reinterpret_cast<unsigned *>(b + 2 * map_bytes);
+    const int bwords = bitmap_words((size_t)toff[nsys], blocks);
+    cudaMemsetAsync(d_upd, 0, 4 * map_bytes, st);
+    for (int q = 0; q < nsys; ++q) {
+        As[q].upd = d_upd;
+        As[q].stamp = d_stamp;
+        As[q].bwords = bwords;
+        As[q].mapw = (unsigned)(map_bytes / 4);
+        As[q].tile0 = (unsigned)toff[q];
+    }
     cudaMemcpyAsync(d_sys, As.data(), (size_t)nsys * sizeof(SweepArgs), cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(d_toff, toff.data(), (size_t)(nsys + 1) * 8, cudaMemcpyHostToDevice, st);
-    cudaMemsetAsync(d_ctl, 0, 3 * kLine * sizeof(unsigned), st);
+    cudaMemsetAsync(d_ctl, 0, kCtlWords * sizeof(unsigned), st);
     cudaMemsetAsync(d_err, 0, sizeof(int), st);
     MultiArgs P;
     P.sys = d_sys;
@@ -1465,6 +1449,10 @@ cudaError_t launch_sweep_multi(int nsys, const SweepSys *sys, const KernelW &kw,
     P.err = d_err;
     P.rounds = d_rounds;
     P.capped = d_capped;
+    P.upd = d_upd;
+    P.stamp = d_stamp;
+    P.bwords = bwords;
+    P.mapw = (unsigned)(map_bytes / 4);
     P.max_rounds = max_rounds;
     P.spin_limit = spin_limit;
     P.stamps = stamps;

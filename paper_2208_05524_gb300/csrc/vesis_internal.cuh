@@ -215,7 +215,7 @@ cudaError_t launch_sweep(const GridDesc &g, const KernelW &kw, const int *k3,
                          int *rounds, int *capped, int max_rounds, int blocks,
                          long long spin_limit, int stamps, RoundState *rs, cudaStream_t st);
 // Decide stamps of the sweep (which tiles a round's decide visits): -1
-// while the leader tiles outnumber the grid's warps, 0 never (every leader
+// while the leader half tiles outnumber the grid's warps, 0 never (every leader
 // tile is decided every round), 1 always.  The rounds and labels are the
 // same in every mode.
 // Default bound on a sweep block's polls of its grid barrier (several
@@ -224,9 +224,9 @@ constexpr long long kSweepSpinLimit = 1ll << 24;
 // Multi-system sweep: the rounds of up to kMaxSweepSys systems (same
 // surface kernel) in one cooperative launch.  Per system: its grid, flip
 // constants, labels, W, U, dE scratch, sweep state, control words and
-// error flag (as for launch_sweep), a per-tile FP64 dE sum and flip count
-// (sweep_tiles(g) entries each), its RoundState and the stream its
-// set-up is enqueued on.  scratch: sweep_multi_scratch_bytes(nsys) bytes
+// error flag (as for launch_sweep), FP64 dE sums and flip counts per half
+// tile (2 sweep_tiles(g) entries each), its RoundState and the stream its
+// set-up is enqueued on.  scratch: sweep_multi_scratch_bytes(nsys, tiles of all) bytes
 // of device memory; err_out (pinned host, may be NULL) receives the
 // launch's error flag.  Everything else is enqueued on st.
 constexpr int kMaxSweepSys = 64;
@@ -245,7 +245,7 @@ struct SweepSys {
     RoundState *rs;
     cudaStream_t st;
 };
-size_t sweep_multi_scratch_bytes(int nsys);
+size_t sweep_multi_scratch_bytes(int nsys, long long tiles);
 cudaError_t launch_sweep_multi(int nsys, const SweepSys *sys, const KernelW &kw, const int *k3,
                                int max_rounds, int blocks, long long spin_limit, int stamps,
                                void *scratch, int *err_out, cudaStream_t st);
