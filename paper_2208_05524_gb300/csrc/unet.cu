@@ -19,7 +19,6 @@
 // weights, gradients and Adam moments in one flat vector.  The convolutions
 // are implicit GEMMs on the tensor cores (mma.sync m16n8k16, BF16 in, FP32
 // accumulate); the rest are plain elementwise and reduction kernels.
-#include <cuda.h>
 #include <cuda_bf16.h>
 
 #include "vesis_internal.cuh"
@@ -354,7 +353,8 @@ __device__ __forceinline__ unsigned smem_u32(const void *p)
 
 // try_wait suspends the thread until the phase completes or a short
 // hardware time limit passes, so the loop polls without sleeping; the
-// global timer, read every 64 misses, bounds the whole wait.
+// global timer, read every 64 misses (a slow read: not before the 64th),
+// bounds the whole wait.
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity)
 {
     unsigned long long t0 = 0;
@@ -366,10 +366,10 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity)
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
         if (ok) return true;
-        if ((i & 63u) == 0) {
+        if ((i & 63u) == 63u) {
             unsigned long long now;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-            if (i == 0) t0 = now;
+            if (i == 63u) t0 = now;
             else if (now - t0 > kTcWaitNs) return false;
         }
     }
@@ -556,239 +556,327 @@ __global__ void __launch_bounds__(128, 1) k_conv_tc(ConvArgs P, int *err)
     }
 }
 
-// Weight-stationary blocks: each block takes nb consecutive bricks (up to
-// 512 / NT, chosen per launch) and keeps a stage's weights in shared memory
-// for all of them, with one FP32 accumulator per brick in tensor memory (nb
-// x NT columns).  The bricks' halos stream through NBUF buffers: the next
-// bricks' halos load while the tensor cores run the current brick's MMAs; a
-// buffer is refilled once the MMAs that read it have committed.  Stage
-// boundaries wait for the stage's last MMAs before the weights are
-// replaced.  The fixed cost of a block (tensor-memory allocation, barrier
-// set-up, the first copies, the epilogue's drain) is spread over its
-// bricks: 8 bricks per block instead of 4 took 6 % off the 384^3 forward.
-__host__ __device__ constexpr int tma_max_nb(int NT) { return 512 / NT; }
-
-// TMA form of the weight-stationary convolution, for inputs at the
-// output's resolution (a decoder's coarse input is doubled first).  The
-// stage's weights come pre-arranged in global memory (one contiguous block
-// per stage and tile of output channels) and arrive by bulk copies (only
-// the planes and taps the stage uses); a brick's halo arrives as
-// tensor-map box loads (8 channels x 10 z x 18 y x 3 x each, or 1 x for
-// x1, cells outside the grid zero-filled by the copy engine).  Copies and MMAs complete on mbarriers, so one
-// thread runs the whole producer/consumer loop: it keeps the copies of the
-// next NBUF - 1 bricks in flight while the tensor cores work, and the
-// other warps only join for the epilogue.  Halo layout: [8-channel plane]
-// [x][y][z][8 ch], planes 128-byte aligned.
-constexpr int TMA_PLANE = 8704;                         // 540 x 16 B padded to 128 B
-constexpr int TMA_HALO = 4 * TMA_PLANE;
-
-// The halo area holds tma_nbuf(NT) full buffers; a stage that loads fewer
-// planes (k16 = 1) or one x-plane (x1) cuts it into more, smaller buffers
-// (up to TMA_MAXBUF), so that more bricks' copies are in flight.
-__host__ __device__ constexpr int tma_nbuf(int NT) { return NT == 32 ? 4 : 3; }
-constexpr int TMA_MAXBUF = 16;
-constexpr int TMA_PLANE_X1 = 2944;                      // 180 x 16 B padded to 128 B
-__host__ __device__ constexpr int tma_smem_bytes(int NT)
+// One lane of a converged warp (the same one every time).
+__device__ __forceinline__ unsigned elect_lane()
 {
-    return tc_w_bytes(NT) + tma_nbuf(NT) * TMA_HALO + 16 * TMA_MAXBUF + 128 + 128;
+    unsigned e;
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 l;\n\telect.sync l|p, 0xffffffff;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(e) :: "memory");
+    return e;
+}
+
+// tc_mma by the elected lane (el) of a converged warp, for operands whose
+// descriptors differ in the low word only (start address and K offset): A's
+// stride is a halo column, B's eight rows.  The issue of a block's MMAs is one
+// chain of instructions: the operands of a converged warp stay in uniform
+// registers, which the instruction wants.
+template <bool ACC>
+__device__ __forceinline__ void tc_mma_lo(unsigned el, unsigned dcol, unsigned alo, unsigned blo,
+                                          unsigned idesc)
+{
+    constexpr unsigned ahi = (TC_HZ * 16 >> 4) | (1u << 14), bhi = (8 * 16 >> 4) | (1u << 14);
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 e, %7, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}"
+        :: "r"(dcol), "r"(alo), "n"(ahi), "r"(blo), "n"(bhi), "r"(idesc), "n"(ACC ? 1 : 0), "r"(el)
+        : "memory");
+}
+
+// Arrival on an mbarrier once every MMA the lane issued so far has completed.
+__device__ __forceinline__ void tc_commit(unsigned el, unsigned bar)
+{
+    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 :: "r"(bar), "r"(el) : "memory");
+}
+
+// Weight-stationary column form.  A block takes nb consecutive bricks of one
+// column along x, with one FP32 accumulator per brick in tensor memory (NT
+// columns each, brick j at column j NT), and streams the column's nb + 2 input
+// planes (18 y x 10 z cells) through NBUF buffers, once per stage of 32 input
+// channels.  An input plane serves the taps of three output planes, whose
+// accumulators adjoin, so one MMA per tap (b, c) and K step has N = 3 NT:
+// weights of x taps 2, 1, 0 for output planes q - 2, q - 1, q of input plane
+// q.  Bound by the MMAs: one of M = 128, N = 96, K = 16 takes 74 cycles
+// (reading its 4 KB of halo, and its issue), hardly more than one of N = 32,
+// so a 32-channel layer does three taps for the price of one.  Each output
+// still sums the same products in the same order (stages, x taps, b, c, K
+// steps).
+// Measured on the forward of 256^3 cells (whole network): 9.03 ms with one
+// brick, N = NT and its three input planes per MMA, halos by tensor-map boxes
+// and one thread issuing; 3.61 ms like this (its 64 -> 32 layer 1.54 ms, 1.21
+// PFLOP/s).  Of that the issue is the most: with one thread of a diverged
+// warp issuing, every MMA took 120 cycles whatever its N (6.40 ms), and with
+// 64-bit descriptors built in a loop 350 (11.98 ms).
+//
+// The stage's weights sit in nine slices, one per (b, c): [8-channel plane]
+// [x tap 2, 1, 0][co][8], contiguous in global memory, a bulk copy each.  In
+// a stage's last plane every slice is committed to its own mbarrier, and the
+// next stage's slice replaces it while the tensor cores work on the others.
+// Warp 4 issues the MMAs; warps 5-8 copy the input planes by 16-byte cp.async
+// (a decoder's coarse input straight from half the coordinates, cells outside
+// the grid zero-filled), TMA_LAG planes in flight; warps 0-3 drain the output
+// planes of the last stage as they complete, under the next planes' MMAs.  Halo plane layout: [8-channel plane][y][z][8 ch],
+// the planes of a cell in different banks.  (Tensor-map boxes of 8 channels
+// take 3.7 cycles per 16-byte row, 2,700 per plane against 1,100 for its
+// MMAs.)
+__host__ __device__ constexpr int tma_max_nb(int NT) { return 512 / NT; }
+constexpr int TMA_LOAD = 128;                           // loading threads
+constexpr int TMA_THREADS = 160 + TMA_LOAD;
+constexpr int TMA_PLANE = 2912;                         // 180 x 16 B and a quarter line
+constexpr int TMA_STAGE_OUT = 4 * 4096;                 // epilogue staging, 4 KB per warp
+constexpr int TMA_MAXBUF = 8;
+constexpr int TMA_LAG = 4, TMA_LAG_SMALL = 2;           // planes in flight (MAXBUF, 4 buffers)
+__host__ __device__ constexpr int tma_slice_bytes(int NT) { return 4 * 3 * NT * 16; }
+// barriers: MAXBUF loads, MAXBUF buffers free, 9 slices full, 9 free, 16 outputs
+constexpr int TMA_TAIL = 8 * (2 * TMA_MAXBUF + 9 + 9 + 16) + 16;
+__host__ __device__ constexpr int tma_smem_bytes(int NT, int nbuf, int k16)
+{
+    return 9 * tma_slice_bytes(NT) + nbuf * 2 * k16 * TMA_PLANE + TMA_STAGE_OUT + TMA_TAIL + 128;
 }
 
 template <int NT, bool RAW>
-__global__ void __launch_bounds__(128, 1)
-k_conv_tma(ConvArgs P, const __grid_constant__ CUtensorMap tmA,
-           const __grid_constant__ CUtensorMap tmB, const bf16 *__restrict__ Wtc, int nbricks,
-           int nb, int *err)
+__global__ void __launch_bounds__(TMA_THREADS, 1)
+k_conv_tma(ConvArgs P, const bf16 *__restrict__ Wtc, int nb, int cols, int NBUF, int *err)
 {
-    // plane stride, buffer size and buffer count of this launch
-    const int PLs = P.x1 ? TMA_PLANE_X1 : TMA_PLANE;
-    const int HB = 2 * P.k16 * PLs;
-    const int NBUF = min(TMA_MAXBUF, tma_nbuf(NT) * TMA_HALO / HB);
+    const int HB = 2 * P.k16 * TMA_PLANE;
+    constexpr int SL = tma_slice_bytes(NT);
     extern __shared__ __align__(1024) unsigned char smem_tma[];
     const unsigned raw0 = smem_u32(smem_tma);
-    const unsigned pad = ((raw0 + 127u) & ~127u) - raw0;
-    unsigned char *smem = smem_tma + pad;
-    unsigned char *tail = smem + tc_w_bytes(NT) + tma_nbuf(NT) * TMA_HALO;
-    unsigned *tslot = reinterpret_cast<unsigned *>(tail + 16 * TMA_MAXBUF);
-    int *sfail = reinterpret_cast<int *>(tail + 16 * TMA_MAXBUF + 4);
+    unsigned char *smem = smem_tma + (((raw0 + 127u) & ~127u) - raw0);
+    unsigned char *tail = smem + 9 * SL + NBUF * HB + TMA_STAGE_OUT;
+    unsigned *tslot = reinterpret_cast<unsigned *>(tail + TMA_TAIL - 16);
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const int nyb = P.ny / TCY, nzb = P.nz / TCZ;
-    const int b0 = blockIdx.x * nb;
-    const int nbv = min(nb, nbricks - b0);
+    const int col = blockIdx.x % (nyb * nzb), bz = col % nzb, by = col / nzb;
+    const int x0 = (blockIdx.x / (nyb * nzb)) * nb;
+    const int nbv = min(nb, P.nx - x0);
     const int nst = (P.Ca + P.Cb) / 32;     // stages of the first input, then of the second
-    const int U = nst * nbv;
+    const int np = P.x1 ? nbv : nbv + 2;    // input planes of the column
+    const int U = nst * np;
     const int nnt = P.Cout / NT;
     const int co0 = blockIdx.y * NT;
-    const unsigned swa = smem_u32(smem), sha0 = swa + (unsigned)tc_w_bytes(NT);
-    const unsigned ldb0 = smem_u32(tail), mmb0 = ldb0 + 8u * NBUF;   // NBUF load + NBUF MMA barriers
+    const unsigned swa = smem_u32(smem), sha0 = swa + 9u * SL;
+    const unsigned ldb0 = smem_u32(tail), mmb0 = ldb0 + 8u * TMA_MAXBUF;
+    const unsigned wfull0 = mmb0 + 8u * TMA_MAXBUF, wfree0 = wfull0 + 8u * 9u, out0 = wfree0 + 8u * 9u;
     if (t == 0) {
-        *sfail = 0;
-        for (int q = 0; q < 2 * NBUF; ++q)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(ldb0 + 8u * q) : "memory");
+        for (int q = 0; q < 2 * TMA_MAXBUF + 9 + 9 + 16; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;"
+                         :: "r"(ldb0 + 8u * q), "r"(q < TMA_MAXBUF ? TMA_LOAD / 32 : 1) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("prefetch.tensormap [%0];"
-                     :: "l"(reinterpret_cast<unsigned long long>(&tmA)) : "memory");
-        if (P.Cb > 0)
-            asm volatile("prefetch.tensormap [%0];"
-                         :: "l"(reinterpret_cast<unsigned long long>(&tmB)) : "memory");
     }
     if (w == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_u32(tslot)), "r"(512) : "memory");
+                     :: "r"(smem_u32(tslot)), "r"(cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *tslot;
-    constexpr int CH = 1;       // accumulator chains per brick (more did not help)
 
-    if (t == 0) {
-        const unsigned idesc = tc_idesc(NT);
-        // unit u: stage u / nbv, brick u % nbv, buffer u % NBUF (its k-th
-        // use, k = u / NBUF, completes phase k of that buffer's barriers)
-        int issued = 0;      // units whose copies have been issued (in order)
-        auto issue = [&](int u) {
-            issued = u + 1;
-            const int st = u / nbv, bb = b0 + u % nbv, c0 = st * 32;
-            const int bz = bb % nzb, by = (bb / nzb) % nyb, bx = bb / (nzb * nyb);
-            const unsigned buf = (unsigned)(u % NBUF);
-            const unsigned lb = ldb0 + 8u * buf;
-            const unsigned sha = sha0 + buf * (unsigned)HB;
-            const bool wload = (u % nbv) == 0;
-            // x1: the halo is the brick's own x-plane only (180 rows per box)
-            // the stage's weights [8-channel plane][tap][co][8 ch]: all of
-            // them, or for a half-filled stage (k16 = 1) the first two
-            // planes, and with x1 only the taps 9..17 of each
-            const bool wall = P.k16 == 2 && !P.x1;
-            const int ntap = P.x1 ? 9 : 27, tap0 = P.x1 ? 9 : 0;
-            const unsigned wrun = (unsigned)(ntap * NT * 16);
-            const unsigned wbytes = wall ? (unsigned)tc_w_bytes(NT) : 2u * (unsigned)P.k16 * wrun;
-            const unsigned tx = 2u * (unsigned)P.k16 * (P.x1 ? 180u : 540u) * 16u +
-                                (wload ? wbytes : 0u);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                         :: "r"(lb), "r"(tx) : "memory");
-            if (wload) {
-                const bf16 *src = Wtc + (size_t)(st * nnt + blockIdx.y) * (4 * 27 * NT * 8);
-                if (wall) {
-                    asm volatile(
-                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                        :: "r"(swa), "l"(src), "r"((unsigned)tc_w_bytes(NT)), "r"(lb) : "memory");
-                } else {
-                    for (int kc = 0; kc < 2 * P.k16; ++kc) {
-                        const unsigned off = (unsigned)((kc * 27 + tap0) * NT * 16);
-                        asm volatile(
-                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                            :: "r"(swa + off), "l"(reinterpret_cast<const unsigned char *>(src) + off),
-                               "r"(wrun), "r"(lb) : "memory");
-                    }
-                }
-            }
-            const bool first_input = c0 < P.Ca;
-            const unsigned long long map = reinterpret_cast<unsigned long long>(first_input ? &tmA : &tmB);
-            const int cc = first_input ? c0 : c0 - P.Ca;
-            for (int kc = 0; kc < 2 * P.k16; ++kc)
-                asm volatile(
-                    "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-                    " [%0], [%1, {%2, %3, %4, %5}], [%6];"
-                    :: "r"(sha + (unsigned)(kc * PLs)), "l"(map),
-                       "r"(cc + 8 * kc), "r"(bz * TCZ - 1), "r"(by * TCY - 1),
-                       "r"(P.x1 ? bx : bx - 1), "r"(lb)
-                    : "memory");
+    // Units are numbered through the stages and their input planes; unit u
+    // uses buffer u % NBUF, and its k-th use, k = u / NBUF, completes phase k
+    // of that buffer's barriers.  The quotients are kept as running counters:
+    // divisions cost the two loops 0.8 us a unit.
+    struct Slot {
+        int buf;
+        unsigned parity;
+    };
+    auto advance = [&](Slot &s) {
+        if (++s.buf == NBUF) {
+            s.buf = 0;
+            s.parity ^= 1u;
+        }
+    };
+    if (t >= 160) {
+        // pieces of 8 channels, channel plane fastest (64 bytes of a cell)
+        constexpr int MP = (180 * 4 + TMA_LOAD - 1) / TMA_LOAD;
+        const int nkc = 2 * P.k16, lt = t - 160;
+        int offA[MP], offB[MP];
+        unsigned dst[MP], in = 0u;
+#pragma unroll
+        for (int m = 0; m < MP; ++m) {
+            const int p = lt + TMA_LOAD * m, kc = p & (nkc - 1), c = p / nkc;
+            const int gy = by * TCY - 1 + c / TC_HZ, gz = bz * TCZ - 1 + c % TC_HZ;
+            if (gy >= 0 && gz >= 0 && gy < P.ny && gz < P.nz) in |= 1u << m;
+            offA[m] = (gy * P.nz + gz) * P.Ca + 8 * kc;
+            offB[m] = ((gy >> 1) * (P.nz >> 1) + (gz >> 1)) * P.Cb + 8 * kc;
+            dst[m] = sha0 + (unsigned)(kc * TMA_PLANE + c * 16);
+        }
+        Slot put{0, 1u}, done{0, 0u};      // (a fresh buffer's wait passes at once)
+        const int lag = NBUF == TMA_MAXBUF ? TMA_LAG : TMA_LAG_SMALL;
+        auto landed = [&] {      // this warp's part of the next unit is in shared memory
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];"
+                             :: "r"(ldb0 + 8u * (unsigned)done.buf) : "memory");
+            advance(done);
         };
-        auto wait_bar = [&](unsigned base, int u) -> bool {
-            return mbar_wait(base + 8u * (unsigned)(u % NBUF), (unsigned)((u / NBUF) & 1));
+        int u = 0, c0 = 0, q = 0;
+        for (; u < U; ++u) {
+            if (!mbar_wait(mmb0 + 8u * (unsigned)put.buf, put.parity)) {
+                atomicExch(err, 1);
+                break;
+            }
+            const int x = x0 + q - (P.x1 ? 0 : 1);
+            const bool fine = c0 < P.Ca;
+            const bf16 *src = fine ? P.A + (long long)x * P.ny * P.nz * P.Ca + c0
+                                   : P.B + (long long)(x >> 1) * (P.ny >> 1) * (P.nz >> 1) * P.Cb +
+                                         (c0 - P.Ca);
+            const unsigned buf = (unsigned)put.buf * (unsigned)HB;
+            const unsigned v = x >= 0 && x < P.nx ? in : 0u;
+#pragma unroll
+            for (int m = 0; m < MP; ++m)
+                if (lt + TMA_LOAD * m < 180 * nkc) {
+                    const bool ok = (v >> m) & 1u;
+                    cp_async16(dst[m] + buf, ok ? src + (fine ? offA[m] : offB[m]) : P.A, ok);
+                }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            if (u >= lag) {
+                if (NBUF == TMA_MAXBUF)
+                    asm volatile("cp.async.wait_group %0;" :: "n"(TMA_LAG) : "memory");
+                else
+                    asm volatile("cp.async.wait_group %0;" :: "n"(TMA_LAG_SMALL) : "memory");
+                landed();
+            }
+            advance(put);
+            if (++q == np) {
+                q = 0;
+                c0 += 32;
+            }
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        for (int k = max(0, u - lag); k < u; ++k) landed();
+    }
+
+    if (w == 4) {
+        const unsigned el = elect_lane();
+        // the whole warp waits, and goes on together
+        auto wait_all = [&](unsigned bar, unsigned parity) -> bool {
+            return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+        };
+        // slice i of a stage's weights: all of it, or the channel planes and
+        // the x tap in use
+        int sliced = 0;      // slices whose copies have been issued (in order)
+        auto load_slice = [&](int st, int i) {
+            ++sliced;
+            if (!el) return;
+            const unsigned lb = wfull0 + 8u * (unsigned)i;
+            const unsigned char *src = reinterpret_cast<const unsigned char *>(Wtc) +
+                                       ((size_t)(st * nnt + blockIdx.y) * 9 + i) * SL;
+            const bool all = P.k16 == 2 && !P.x1;
+            const unsigned run = (P.x1 ? 1u : 3u) * NT * 16u;
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                         :: "r"(lb), "r"(all ? (unsigned)SL : 2u * (unsigned)P.k16 * run) : "memory");
+            for (int kc = 0; kc < (all ? 1 : 2 * P.k16); ++kc) {
+                const unsigned off = (unsigned)(kc * 3 + (P.x1 ? 1 : 0)) * NT * 16u;
+                asm volatile(
+                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                    :: "r"(swa + (unsigned)i * SL + off), "l"(src + off), "r"(all ? (unsigned)SL : run),
+                       "r"(lb) : "memory");
+            }
         };
         bool ok = true;
-        // prologue: the first stage's first NBUF - 1 bricks
-        for (int v = 0; v < NBUF - 1 && v < nbv && v < U; ++v) issue(v);
+        for (int i = 0; i < 9; ++i) load_slice(0, i);
+        Slot at{0, 0u}, last{0, 0u};
+        int st = 0, q = 0;
         for (int u = 0; u < U && ok; ++u) {
-            const int st = u / nbv;
-            if (!wait_bar(ldb0, u)) { ok = false; break; }
+            // output planes jlo .. jhi see this input plane, through x taps q - j
+            const int jlo = P.x1 ? q : max(0, q - 2), jhi = min(nbv - 1, q);
+            const int g0 = P.x1 ? 1 : 2 - (q - jlo);          // first group of weight rows
+            const int n = jhi - jlo + 1;
+            const unsigned dcol = tmem + (unsigned)(jlo * NT);
+            const unsigned idesc = tc_idesc(NT * n);
+            const bool fresh = st == 0 && jhi == q;           // output plane q starts here
+            if (!wait_all(ldb0 + 8u * (unsigned)at.buf, at.parity)) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const unsigned hbase = sha0 + (unsigned)(u % NBUF) * (unsigned)HB;
-            const unsigned long long ad0 = tc_desc(hbase, (unsigned)PLs, TC_HZ * 16);
-            const unsigned long long bd0 = tc_desc(swa, 27 * NT * 16, 8 * 16);
-            const unsigned dbase = tmem + (unsigned)((u % nbv) * CH * NT);
-            const bool first = st == 0;
-            // with x1 only the taps 9..17 (x offset 0) run; the first CH of
-            // them start the accumulator chains
-            const int t0 = P.x1 ? 9 : 0;
-            if (P.k16 == 2) {
+            // low words of the descriptors (the high words are constants)
+            const unsigned ad0 = (unsigned)tc_desc(sha0 + (unsigned)at.buf * (unsigned)HB, TMA_PLANE, 0);
+            const unsigned bw = (unsigned)tc_desc(swa, 3 * NT * 16, 0) + (unsigned)(g0 * NT);
+            const bool leave = q == np - 1 && st + 1 < nst;   // the slices' last plane
+            auto slices = [&](auto k16c) {
 #pragma unroll
-                for (int tap = 0; tap < 27; ++tap) {
-                    const int da = tap / 9, db = (tap / 3) % 3, dc = tap % 3;
-                    if (P.x1 && da != 1) continue;
-                    const unsigned long long ao =
-                        (unsigned long long)(((P.x1 ? 0 : da) * TC_HY + db) * TC_HZ + dc);
+                for (int i = 0; i < 9; ++i) {
+                    if (q == 0) {
+                        if (!wait_all(wfull0 + 8u * (unsigned)i, (unsigned)(st & 1))) {
+                            ok = false;
+                            return;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    }
 #pragma unroll
-                    for (int s2 = 0; s2 < 2; ++s2)
-                        tc_mma(dbase + (unsigned)((tap % CH) * NT),
-                               ad0 + ao + (unsigned long long)(2 * s2 * (PLs / 16)),
-                               bd0 + (unsigned long long)((2 * s2 * 27 + tap) * NT), idesc,
-                               (!first || tap >= t0 + CH || s2 > 0) ? 1u : 0u);
+                    for (int s2 = 0; s2 < k16c(); ++s2) {
+                        const unsigned a2 = ad0 + (unsigned)((i / 3) * TC_HZ + i % 3 + 2 * s2 * (TMA_PLANE / 16));
+                        const unsigned b2 = bw + (unsigned)(i * (SL / 16) + 2 * s2 * 3 * NT);
+                        if (i == 0 && s2 == 0 && fresh) {
+                            if (n > 1) tc_mma_lo<true>(el, dcol, a2, b2, tc_idesc(NT * (n - 1)));
+                            tc_mma_lo<false>(el, dcol + (unsigned)((n - 1) * NT), a2,
+                                             b2 + (unsigned)((n - 1) * NT), tc_idesc(NT));
+                        } else {
+                            tc_mma_lo<true>(el, dcol, a2, b2, idesc);
+                        }
+                    }
+                    if (leave) tc_commit(el, wfree0 + 8u * (unsigned)i);
                 }
-            } else {
-#pragma unroll
-                for (int tap = 0; tap < 27; ++tap) {
-                    const int da = tap / 9, db = (tap / 3) % 3, dc = tap % 3;
-                    if (P.x1 && da != 1) continue;
-                    const unsigned long long ao =
-                        (unsigned long long)(((P.x1 ? 0 : da) * TC_HY + db) * TC_HZ + dc);
-                    tc_mma(dbase + (unsigned)((tap % CH) * NT), ad0 + ao,
-                           bd0 + (unsigned long long)(tap * NT), idesc,
-                           (!first || tap >= t0 + CH) ? 1u : 0u);
+            };
+            if (P.k16 == 2) slices([] { return 2; });
+            else slices([] { return 1; });
+            if (!ok) break;
+            tc_commit(el, mmb0 + 8u * (unsigned)at.buf);
+            // the last stage completes an output plane with its third input plane
+            if (st == nst - 1) {
+                const int j = P.x1 ? q : q - 2;
+                if (j >= 0) tc_commit(el, out0 + 8u * (unsigned)j);
+            }
+            // next stage's weights, slice by slice as the last plane leaves them
+            if (q == np - 1 && st + 1 < nst)
+                for (int i = 0; i < 9 && ok; ++i) {
+                    ok = wait_all(wfree0 + 8u * (unsigned)i, (unsigned)(st & 1));
+                    if (ok) load_slice(st + 1, i);
                 }
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(mmb0 + 8u * (unsigned)(u % NBUF)) : "memory");
-            // with this brick's MMAs queued, refill the buffer the previous
-            // brick read (unit u + NBUF - 1 of the same stage): the tensor
-            // cores never wait for the issuing thread
-            const int v = u + NBUF - 1;
-            if (v < U && v / nbv == st) {
-                if (v >= NBUF && !wait_bar(mmb0, v - NBUF)) { ok = false; break; }
-                issue(v);
-            }
-            // stage boundary: replace the weights once every MMA of the stage
-            // has completed, then refill the pipeline
-            if (u + 1 < U && (u + 1) % nbv == 0) {
-                if (!wait_bar(mmb0, u)) { ok = false; break; }
-                for (int q = u + 1; q < u + NBUF && q < U && q / nbv == (u + 1) / nbv; ++q)
-                    issue(q);
+            last = at;
+            advance(at);
+            if (++q == np) {
+                q = 0;
+                ++st;
             }
         }
-        if (ok && U > 0 && !wait_bar(mmb0, U - 1)) ok = false;
+        if (ok && !wait_all(mmb0 + 8u * (unsigned)last.buf, last.parity)) ok = false;
         if (!ok) {
-            *sfail = 1;
-            atomicExch(err, 1);
+            if (el) atomicExch(err, 1);
             // copies still in flight target this block's shared memory:
-            // wait (bounded) for the last one of each buffer
-            for (int q = max(0, issued - NBUF); q < issued; ++q) wait_bar(ldb0, q);
+            // wait (bounded) for the last one of each slice
+            for (int v = max(0, sliced - 9); v < sliced; ++v)
+                wait_all(wfull0 + 8u * (unsigned)(v % 9), (unsigned)((v / 9) & 1));
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!*sfail) {
+    if (w < 4) {
         // Each warp holds 32 cells of a brick: one y row of 8 z cells per 8
-        // lanes.  A cell's outputs pass through the (now idle) halo buffers
-        // so that each store instruction writes whole 64- or 128-byte cell
-        // rows instead of one 16-byte piece of 32 cells.  Chunk slots are
-        // XOR-swizzled so that neither side has bank conflicts.
+        // lanes.  A cell's outputs pass through the staging area so that each
+        // store instruction writes whole 64- or 128-byte cell rows instead of
+        // one 16-byte piece of 32 cells.  Chunk slots are XOR-swizzled so that
+        // neither side has bank conflicts.
         const long long nyz = (long long)P.ny * P.nz;
-        uint4 *stg = reinterpret_cast<uint4 *>(smem + tc_w_bytes(NT)) + w * 256;   // 4 KB per warp
+        uint4 *stg = reinterpret_cast<uint4 *>(smem + 9 * SL + NBUF * HB) + w * 256;
         for (int b = 0; b < nbv; ++b) {
-            const int bb = b0 + b;
-            const int bz = bb % nzb, by = (bb / nzb) % nyb, bx = bb / (nzb * nyb);
+            if (!mbar_wait(out0 + 8u * (unsigned)b, 0u)) {     // the issuing thread gave up
+                atomicExch(err, 1);
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // cell of warp-local index c: row c >> 3 (y), z = c & 7
-            const long long vrow = (long long)bx * nyz + (long long)(by * TCY + 4 * w) * P.nz +
+            const long long vrow = (long long)(x0 + b) * nyz + (long long)(by * TCY + 4 * w) * P.nz +
                                    bz * TCZ;
             const long long vo = vrow + (long long)(lane >> 3) * P.nz + (lane & 7);
 #pragma unroll
             for (int half = 0; half < NT / 32; ++half) {
                 unsigned r[32];
                 const unsigned ta = tmem + ((unsigned)(32 * w) << 16) +
-                                    (unsigned)(b * CH * NT + 32 * half);
+                                    (unsigned)(b * NT + 32 * half);
                 asm volatile(
                     "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
                     "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -857,28 +945,13 @@ k_conv_tma(ConvArgs P, const __grid_constant__ CUtensorMap tmA,
     if (w == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
-                     :: "r"(tmem), "r"(512) : "memory");
+                     :: "r"(tmem), "r"(cols) : "memory");
     }
 }
 
-// Nearest doubling: Y[v][c] = X[parent(v)][c] for a fine grid nx x ny x nz
-// (16-byte copies; C / 8 = 2^qs groups of 8 channels): fine row (i, j) on
-// blockIdx.x, (k, group) on blockIdx.y x blockDim.x.
-__global__ void k_upsample(const bf16 *__restrict__ X, int nx, int ny, int nz, int C, int qs,
-                           bf16 *__restrict__ Y)
-{
-    const int q = C >> 3;
-    const int row = blockIdx.x, i = row / ny, j = row - i * ny;
-    const int e = blockIdx.y * blockDim.x + threadIdx.x;
-    if (e >= nz * q) return;
-    const int k = e >> qs, part = e & (q - 1);
-    const long long u = ((long long)(i >> 1) * (ny >> 1) + (j >> 1)) * (nz >> 1) + (k >> 1);
-    reinterpret_cast<uint4 *>(Y + ((long long)row * nz + k) * C)[part] =
-        reinterpret_cast<const uint4 *>(X + u * C)[part];
-}
-
 // Weights [27][Cout][Cin] -> the TMA form's layout: per stage of 32 input
-// channels and tile of NT output channels, [8-channel plane][tap][co][8].
+// channels and tile of NT output channels, [tap (b, c)][8-channel plane]
+// [x tap 2, 1, 0][co][8].
 __global__ void k_pack_tc(const bf16 *__restrict__ W, int Cout, int Cin, int NT,
                           bf16 *__restrict__ out)
 {
@@ -890,7 +963,8 @@ __global__ void k_pack_tc(const bf16 *__restrict__ W, int Cout, int Cin, int NT,
     const int ci = (int)(e % Cin);
     const int st = ci / 32, kc = (ci % 32) / 8, j = ci % 8;
     const int nt = co / NT, col = co % NT, nnt = Cout / NT;
-    out[((((long long)(st * nnt + nt) * 4 + kc) * 27 + tap) * NT + col) * 8 + j] = W[e];
+    out[(((((long long)(st * nnt + nt) * 9 + tap % 9) * 4 + kc) * 3 + 2 - tap / 9) * NT + col) * 8 + j] =
+        W[e];
 }
 
 // Weight gradient of a conv3: dW[tap][co][ci] = sum over cells v of
@@ -1651,7 +1725,6 @@ __global__ void k_features(const float *__restrict__ U, const float *__restrict_
 }  // namespace vesis
 
 // ================================================================ host side
-#include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <cmath>
@@ -1674,40 +1747,6 @@ struct Layer {
 };
 
 int tc_tile(int c) { return c % 64 == 0 ? 64 : 32; }
-
-// cuTensorMapEncodeTiled through the runtime's driver entry point (no link
-// against the driver library).
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
-{
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                             &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    });
-    return fn;
-}
-
-// Tensor map of a channels-last activation [nx][ny][nz][C] bf16 with the
-// halo box {8 ch, 10 z, 18 y, hx x}; out-of-range cells read as zero.
-bool encode_halo_map(CUtensorMap *m, const bf16 *base, int C, int nx, int ny, int nz,
-                     int hx = TC_HX)
-{
-    PFN_cuTensorMapEncodeTiled_v12000 fn = tensor_map_encoder();
-    if (!fn) return false;
-    const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)nz, (cuuint64_t)ny, (cuuint64_t)nx};
-    const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)C * 2 * nz,
-                                   (cuuint64_t)C * 2 * nz * ny};
-    const cuuint32_t box[4] = {8, (cuuint32_t)TC_HZ, (cuuint32_t)TC_HY, (cuuint32_t)hx};
-    const cuuint32_t es[4] = {1, 1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16 *>(base), dims, strides, box,
-              es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 
 enum { L_E0, L_E1, L_E2, L_E3, L_D2, L_D1, L_D0, L_HEAD, L_N };
 
@@ -1739,8 +1778,6 @@ struct vesis_net_t {
     long long part_cap = 0;       // floats
     double *h_loss = nullptr;
     int conv_kind = 1;            // 0 mma.sync, 1 tcgen05 where the shape allows
-    bf16 *up = nullptr;           // a decoder's coarse input doubled to its resolution
-    long long up_cap = 0;
     int *d_err = nullptr;         // timeout flag of the tcgen05 convolution
     int *h_err = nullptr;
     std::vector<void *> act;      // activation allocations
@@ -1782,8 +1819,6 @@ void free_act(vesis_net n)
 {
     for (void *q : n->act) cudaFree(q);
     n->act.clear();
-    n->up = nullptr;
-    n->up_cap = 0;
     n->nx = n->ny = n->nz = 0;
 }
 
@@ -1808,8 +1843,6 @@ int ensure_act(vesis_net n, int nx, int ny, int nz, bool train)
     NTRY(nalloc(A, &n->d[1], V1 * 32));
     NTRY(nalloc(A, &n->d[2], V2 * 64));
     NTRY(nalloc(A, &n->z, V0));
-    NTRY(nalloc(A, &n->up, V0 * 32));    // the largest doubled coarse input (d0's)
-    n->up_cap = V0 * 32;
     NTRY(nalloc(A, &n->loss_part, (V0 + 255) / 256));
     if (train) {
         NTRY(nalloc(A, &n->dz, V0));
@@ -1883,30 +1916,33 @@ bool conv(vesis_net n, int nx, int ny, int nz, const bf16 *A, int Ca, const bf16
     if (n->conv_kind == 1 && ny % TCY == 0 && nz % TCZ == 0 && Ca % 32 == 0 && Cb % 32 == 0 &&
         Cout % 32 == 0) {
         const unsigned bricks = (unsigned)(nx * (ny / TCY) * (nz / TCZ));
-        CUtensorMap tm, tmb;
-        bool tma_ok = bricks >= 152u * 4u && Wtc &&
-                      encode_halo_map(&tm, A, Ca, nx, ny, nz, x1 ? 1 : TC_HX);
-        if (tma_ok && Cb > 0) {
-            // the coarse input doubled to the output's resolution, so that
-            // both inputs arrive by tensor-map boxes
-            tma_ok = n->up && (long long)nx * ny * nz * Cb <= n->up_cap &&
-                     encode_halo_map(&tmb, n->up, Cb, nx, ny, nz);
-            if (tma_ok) {
-                count_launch();
-                k_upsample<<<row_grid(nx, ny, (long long)nz * (Cb / 8)), 128, 0, n->st>>>(
-                    B, nx, ny, nz, Cb, log2_groups(Cb), n->up);
-            }
-        } else {
-            tmb = tm;
-        }
-        if (tma_ok) {
-            // enough bricks for weight-stationary blocks: TMA and bulk copies,
-            // nb bricks per block, halved from 512 / NT while that leaves
-            // fewer than two blocks per SM
+        if (bricks >= 152u * 4u && Wtc) {
+            // enough bricks for weight-stationary blocks of nb bricks along x.
+            // A block costs its nb + 2 planes (nb of the folded input layer)
+            // and a start and an end worth about three more (6,000 cycles
+            // beside 1,900 a plane); the nb with the fewest such units over the waves of
+            // blocks is taken.  The folded layer's planes are small and short
+            // to compute, so two of its blocks share an SM (half the tensor
+            // memory each) and overlap their ends.
             const int NTt = tc_tile(Cout);
-            int bpb = tma_max_nb(NTt);
-            while (bpb > 2 && (long long)((bricks + bpb - 1) / bpb) * (Cout / NTt) < 2 * 152) bpb /= 2;
-            const unsigned nb = (bricks + bpb - 1) / bpb;
+            const int per_sm = x1 && k16 == 1 && NTt == 32 ? 2 : 1;
+            const long long columns = (long long)(ny / TCY) * (nz / TCZ);
+            int bpb = 1;
+            long long nb = 0, least = 0;
+            for (int c = tma_max_nb(NTt) / per_sm; c >= 1; c /= 2) {
+                const long long blk = columns * ((nx + c - 1) / c);
+                const long long waves = (blk * (Cout / NTt) + 152 * per_sm - 1) / (152 * per_sm);
+                const long long cost = waves * (std::min(c, nx) + (x1 ? 3 : 5));
+                if (nb == 0 || cost < least) {
+                    least = cost;
+                    bpb = c;
+                    nb = blk;
+                }
+            }
+            int tcols = 32;                      // tensor memory: a power of two
+            while (tcols < bpb * NTt) tcols *= 2;
+            const int nbuf = per_sm == 2 ? 4 : TMA_MAXBUF;
+            const int tsm = tma_smem_bytes(NTt, nbuf, k16);
             const bool fuse = hz && !raw && Cout == 32;
             if (fuse) {
                 a.hw = hw;
@@ -1914,13 +1950,13 @@ bool conv(vesis_net n, int nx, int ny, int nz, const bf16 *A, int Ca, const bf16
                 a.hz = hz;
             }
             if (tc_tile(Cout) == 64) {
-                dim3 tg(nb, Cout / 64);
-                if (raw) k_conv_tma<64, true><<<tg, 128, tma_smem_bytes(64), n->st>>>(a, tm, tmb, Wtc, (int)bricks, bpb, n->d_err);
-                else k_conv_tma<64, false><<<tg, 128, tma_smem_bytes(64), n->st>>>(a, tm, tmb, Wtc, (int)bricks, bpb, n->d_err);
+                dim3 tg((unsigned)nb, Cout / 64);
+                if (raw) k_conv_tma<64, true><<<tg, TMA_THREADS, tsm, n->st>>>(a, Wtc, bpb, tcols, nbuf, n->d_err);
+                else k_conv_tma<64, false><<<tg, TMA_THREADS, tsm, n->st>>>(a, Wtc, bpb, tcols, nbuf, n->d_err);
             } else {
-                dim3 tg(nb, Cout / 32);
-                if (raw) k_conv_tma<32, true><<<tg, 128, tma_smem_bytes(32), n->st>>>(a, tm, tmb, Wtc, (int)bricks, bpb, n->d_err);
-                else k_conv_tma<32, false><<<tg, 128, tma_smem_bytes(32), n->st>>>(a, tm, tmb, Wtc, (int)bricks, bpb, n->d_err);
+                dim3 tg((unsigned)nb, Cout / 32);
+                if (raw) k_conv_tma<32, true><<<tg, TMA_THREADS, tsm, n->st>>>(a, Wtc, bpb, tcols, nbuf, n->d_err);
+                else k_conv_tma<32, false><<<tg, TMA_THREADS, tsm, n->st>>>(a, Wtc, bpb, tcols, nbuf, n->d_err);
             }
             return fuse;
         }
@@ -2146,13 +2182,13 @@ int vesis_net_create(int n_features, void *cuda_stream, vesis_net *out)
          cudaFuncSetAttribute(k_conv_tc<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               tc_smem_bytes(64)) != cudaSuccess ||
          cudaFuncSetAttribute(k_conv_tma<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              tma_smem_bytes(32)) != cudaSuccess ||
+                              tma_smem_bytes(32, TMA_MAXBUF, 2)) != cudaSuccess ||
          cudaFuncSetAttribute(k_conv_tma<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              tma_smem_bytes(32)) != cudaSuccess ||
+                              tma_smem_bytes(32, TMA_MAXBUF, 2)) != cudaSuccess ||
          cudaFuncSetAttribute(k_conv_tma<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              tma_smem_bytes(64)) != cudaSuccess ||
+                              tma_smem_bytes(64, TMA_MAXBUF, 2)) != cudaSuccess ||
          cudaFuncSetAttribute(k_conv_tma<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              tma_smem_bytes(64)) != cudaSuccess ||
+                              tma_smem_bytes(64, TMA_MAXBUF, 2)) != cudaSuccess ||
          cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               WT_SMEM) != cudaSuccess))
         rc = nfail(VESIS_E_CUDA, "shared memory attribute of the tensor-core conv kernel");
