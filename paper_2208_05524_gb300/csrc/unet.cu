@@ -312,9 +312,13 @@ __global__ void __launch_bounds__(128) k_conv_halo(ConvArgs P)
 // bytes), so every tap's A operand is the halo itself seen through a
 // descriptor: a core matrix is 8 cells along z (consecutive 16-byte rows),
 // the next 8 rows of M are the next y column (a fixed stride), the next 8
-// channels of K the next channel plane (another fixed stride).  One thread
-// issues the 54 MMAs of a stage (27 taps x 2 steps of K = 16) and commits
-// them to an mbarrier that guards the buffers of the next stage.
+// channels of K the next channel plane (another fixed stride).  The weights
+// of a stage arrive by one bulk copy; warp 0 issues its 54 MMAs (27 taps x 2
+// steps of K = 16) and commits them to an mbarrier that guards the buffers of
+// the next stage.  Bound by the latency of a stage (copies, MMAs, barriers) on
+// grids of few bricks: 256 -> 64 channels on 32 bricks took 63 us with 16-byte
+// copies of the weights and one thread of a diverged warp issuing, 38 us like
+// this.
 constexpr int TCY = 16, TCZ = 8;                           // brick (x extent 1)
 constexpr int TC_HX = 3, TC_HY = TCY + 2, TC_HZ = TCZ + 2;
 constexpr int TC_HALO_BYTES = TC_HX * TC_HY * 4 * TC_HZ * 16;   // 34,560
@@ -325,9 +329,12 @@ constexpr unsigned long long kTcWaitNs = 2000000000ull;   // 2 s bound on one wa
 constexpr int TC_CHAINS = 4;
 
 __host__ __device__ constexpr int tc_w_bytes(int NT) { return 27 * 4 * NT * 16; }
+// Halo areas: at NT = 64 one block fills an SM and loads the next stage's
+// halo under the MMAs; at NT = 32 two blocks share an SM instead.
+__host__ __device__ constexpr int tc_halos(int NT) { return NT == 64 ? 2 : 1; }
 __host__ __device__ constexpr int tc_smem_bytes(int NT)
 {
-    return tc_w_bytes(NT) + TC_HALO_BYTES + 64;
+    return tc_w_bytes(NT) + tc_halos(NT) * TC_HALO_BYTES + 64;
 }
 
 // Shared-memory matrix descriptor: start, leading (K) and stride (M/N) byte
@@ -384,37 +391,65 @@ __device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool v
                  :: "r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
 }
 
-__device__ __forceinline__ void tc_mma(unsigned dcol, unsigned long long ad, unsigned long long bd,
-                                       unsigned idesc, unsigned acc)
+// One lane of a converged warp (the same one every time).
+__device__ __forceinline__ unsigned elect_lane()
 {
+    unsigned e;
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 l;\n\telect.sync l|p, 0xffffffff;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(e) :: "memory");
+    return e;
+}
+
+// tc_mma by the elected lane (el) of a converged warp, for operands whose
+// descriptors differ in the low word only (start address and K offset); SA,
+// SB: their strides (bytes) along M and N.  The issue of a block's MMAs is one
+// chain of instructions: the operands of a converged warp stay in uniform
+// registers, which the instruction wants.
+template <int SA, int SB>
+__device__ __forceinline__ void tc_mma_lo(unsigned el, unsigned dcol, unsigned alo, unsigned blo,
+                                          unsigned idesc, unsigned acc)
+{
+    constexpr unsigned ahi = (SA >> 4) | (1u << 14), bhi = (SB >> 4) | (1u << 14);
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :: "r"(dcol), "l"(ad), "l"(bd), "r"(idesc), "r"(acc) : "memory");
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 a, b;\n\t"
+        "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 e, %7, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}"
+        :: "r"(dcol), "r"(alo), "n"(ahi), "r"(blo), "n"(bhi), "r"(idesc), "r"(acc), "r"(el)
+        : "memory");
+}
+
+// Arrival on an mbarrier once every MMA the lane issued so far has completed.
+__device__ __forceinline__ void tc_commit(unsigned el, unsigned bar)
+{
+    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 :: "r"(bar), "r"(el) : "memory");
 }
 
 template <int NT, bool RAW>
-__global__ void __launch_bounds__(128, 1) k_conv_tc(ConvArgs P, int *err)
+__global__ void __launch_bounds__(128, 1)
+k_conv_tc(ConvArgs P, const bf16 *__restrict__ Wtc, int *err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char *sw = smem;                                 // weights
-    unsigned char *sh = smem + tc_w_bytes(NT);                // halo
-    unsigned long long *mbar = reinterpret_cast<unsigned long long *>(sh + TC_HALO_BYTES);
-    unsigned *tslot = reinterpret_cast<unsigned *>(sh + TC_HALO_BYTES + 8);
-    int *sfail = reinterpret_cast<int *>(sh + TC_HALO_BYTES + 16);
+    constexpr int NH = tc_halos(NT);
+    unsigned char *sh = smem + tc_w_bytes(NT);                // halo areas
+    unsigned char *tail = sh + NH * TC_HALO_BYTES;
+    unsigned *tslot = reinterpret_cast<unsigned *>(tail + 16);
+    int *sfail = reinterpret_cast<int *>(tail + 24);
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const int nyb = P.ny / TCY, nzb = P.nz / TCZ;
     const int bz = blockIdx.x % nzb, by = (blockIdx.x / nzb) % nyb, bx = blockIdx.x / (nzb * nyb);
     const int i0 = bx, j0 = by * TCY, k0 = bz * TCZ;
     const int co0 = blockIdx.y * NT;
-    const int Cin = P.Ca + P.Cb;
     const long long nyz = (long long)P.ny * P.nz;
     const int hy = P.ny >> 1, hz = P.nz >> 1;
-    const unsigned bar = smem_u32(mbar);
+    const unsigned bar = smem_u32(tail), wbar = bar + 8u;      // MMAs, weights
+    const unsigned swa = smem_u32(smem), sha = smem_u32(sh);
     if (t == 0) {
         *sfail = 0;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar) : "memory");
+        for (int q = 0; q < 2; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bar + 8u * q) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (w == 0) {
@@ -427,26 +462,15 @@ __global__ void __launch_bounds__(128, 1) k_conv_tc(ConvArgs P, int *err)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *tslot;
     const unsigned idesc = tc_idesc(NT);
-    const int nstage = Cin / 32;
-    for (int st = 0; st < nstage; ++st) {
+    const int nstage = (P.Ca + P.Cb) / 32, nnt = P.Cout / NT;
+    // halo of a stage: [hx][hy][kc][hz][8 ci], zero outside the grid; 8-channel
+    // pieces, the four of a cell first
+    auto load_halo = [&](int st) {
         const int c0 = st * 32;
-        if (st > 0 && !mbar_wait(bar, (unsigned)((st - 1) & 1))) {
-            *sfail = 1;
-            atomicExch(err, 1);
-        }
-        __syncthreads();
-        if (*sfail) break;
-        // weights of the stage: [tap][kc][co][8 ci]
-        const unsigned swa = smem_u32(sw), sha = smem_u32(sh);
-        for (int e = t; e < 27 * 4 * NT; e += 128) {
-            const int co = e % NT, kc = (e / NT) % 4, tap = e / (4 * NT);
-            const bf16 *src = P.Wt + ((long long)tap * P.Cout + co0 + co) * Cin + c0 + kc * 8;
-            cp_async16(swa + (unsigned)e * 16u, src, true);
-        }
-        // halo of the stage: [hx][hy][kc][hz][8 ci], zero outside the grid
-        for (int e = t; e < TC_HX * TC_HY * 4 * TC_HZ; e += 128) {
-            const int hzz = e % TC_HZ, kc = (e / TC_HZ) % 4, hyy = (e / (4 * TC_HZ)) % TC_HY,
-                      hxx = e / (4 * TC_HZ * TC_HY);
+        const unsigned to = sha + (unsigned)((NH == 2 ? st & 1 : 0) * TC_HALO_BYTES);
+        for (int e = t; e < TC_HX * TC_HY * TC_HZ * 4; e += 128) {
+            const int kc = e & 3, row = (e >> 2) / TC_HZ, hzz = (e >> 2) - row * TC_HZ;
+            const int hxx = row / TC_HY, hyy = row - hxx * TC_HY;
             const int ii = i0 + hxx - 1, jj = j0 + hyy - 1, kk = k0 + hzz - 1;
             const bool in = ii >= 0 && ii < P.nx && jj >= 0 && jj < P.ny && kk >= 0 && kk < P.nz;
             const bf16 *src = P.A;     // any valid address when nothing is read
@@ -458,34 +482,61 @@ __global__ void __launch_bounds__(128, 1) k_conv_tc(ConvArgs P, int *err)
                     src = P.B + (((long long)(ii >> 1) * hy + (jj >> 1)) * hz + (kk >> 1)) * P.Cb +
                           (c0 - P.Ca) + kc * 8;
             }
-            cp_async16(sha + (unsigned)e * 16u, src, in);
+            cp_async16(to + (unsigned)(((row * 4 + kc) * TC_HZ + hzz) * 16), src, in);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (NH == 2) load_halo(0);
+    for (int st = 0; st < nstage; ++st) {
+        if (st > 0 && !mbar_wait(bar, (unsigned)((st - 1) & 1))) {
+            *sfail = 1;
+            atomicExch(err, 1);
+        }
+        __syncthreads();
+        if (*sfail) break;
+        // the stage's weights, one bulk copy: [tap (b, c)][kc][x tap 2, 1, 0][co][8 ci]
+        if (t == 0) {
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                         :: "r"(wbar), "r"((unsigned)tc_w_bytes(NT)) : "memory");
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                :: "r"(swa), "l"(Wtc + (size_t)(st * nnt + blockIdx.y) * (tc_w_bytes(NT) / 2)),
+                   "r"((unsigned)tc_w_bytes(NT)), "r"(wbar) : "memory");
+        }
+        if (NH == 1) load_halo(st);
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (t == 0) {
+        if (w == 0) {
+            const unsigned el = elect_lane();
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(wbar, (unsigned)(st & 1)));
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             // descriptors of tap 0, step 0; the others differ only in the
             // start address field (16-byte units), so they are one add away
-            const unsigned long long ad0 = tc_desc(smem_u32(sh), TC_HZ * 16, 4 * TC_HZ * 16);
-            const unsigned long long bd0 = tc_desc(smem_u32(sw), NT * 16, 8 * 16);
+            const unsigned ad0 = (unsigned)tc_desc(
+                sha + (unsigned)((NH == 2 ? st & 1 : 0) * TC_HALO_BYTES), TC_HZ * 16, 0);
+            const unsigned bd0 = (unsigned)tc_desc(swa, 3 * NT * 16, 0);
+            const unsigned more = st > 0 ? 1u : 0u;
+            if (ok) {
 #pragma unroll
-            for (int tap = 0; tap < 27; ++tap) {
-                const int da = tap / 9, db = (tap / 3) % 3, dc = tap % 3;   // halo offsets 0..2
+                for (int tap = 0; tap < 27; ++tap) {
+                    const int da = tap / 9, db = (tap / 3) % 3, dc = tap % 3;   // halo offsets 0..2
 #pragma unroll
-                for (int s2 = 0; s2 < 2; ++s2) {
-                    const unsigned long long ad =
-                        ad0 + (unsigned long long)(((da * TC_HY + db) * 4 + 2 * s2) * TC_HZ + dc);
-                    const unsigned long long bd = bd0 + (unsigned long long)((tap * 4 + 2 * s2) * NT);
-                    const unsigned acc = (st > 0 || tap >= TC_CHAINS || s2 > 0) ? 1u : 0u;
-                    tc_mma(tmem + (unsigned)((tap % TC_CHAINS) * NT), ad, bd, idesc, acc);
+                    for (int s2 = 0; s2 < 2; ++s2)
+                        tc_mma_lo<4 * TC_HZ * 16, 8 * 16>(
+                            el, tmem + (unsigned)((tap % TC_CHAINS) * NT),
+                            ad0 + (unsigned)(((da * TC_HY + db) * 4 + 2 * s2) * TC_HZ + dc),
+                            bd0 + (unsigned)((((tap % 9) * 4 + 2 * s2) * 3 + 2 - da) * NT), idesc,
+                            tap >= TC_CHAINS || s2 > 0 ? 1u : more);
                 }
+                tc_commit(el, bar);
+            } else if (el) {      // nothing will be committed: the waits on the MMAs run out
+                atomicExch(err, 1);
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(bar) : "memory");
         }
+        if (NH == 2 && st + 1 < nstage) load_halo(st + 1);     // read by the next stage's MMAs
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
     const bool failed_before = *sfail != 0;
     __syncthreads();
     if (!failed_before && !mbar_wait(bar, (unsigned)((nstage - 1) & 1))) {
@@ -554,42 +605,6 @@ __global__ void __launch_bounds__(128, 1) k_conv_tc(ConvArgs P, int *err)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
                      :: "r"(tmem), "r"(TC_CHAINS * NT) : "memory");
     }
-}
-
-// One lane of a converged warp (the same one every time).
-__device__ __forceinline__ unsigned elect_lane()
-{
-    unsigned e;
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 l;\n\telect.sync l|p, 0xffffffff;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(e) :: "memory");
-    return e;
-}
-
-// tc_mma by the elected lane (el) of a converged warp, for operands whose
-// descriptors differ in the low word only (start address and K offset): A's
-// stride is a halo column, B's eight rows.  The issue of a block's MMAs is one
-// chain of instructions: the operands of a converged warp stay in uniform
-// registers, which the instruction wants.
-template <bool ACC>
-__device__ __forceinline__ void tc_mma_lo(unsigned el, unsigned dcol, unsigned alo, unsigned blo,
-                                          unsigned idesc)
-{
-    constexpr unsigned ahi = (TC_HZ * 16 >> 4) | (1u << 14), bhi = (8 * 16 >> 4) | (1u << 14);
-    asm volatile(
-        "{\n\t.reg .pred p, e;\n\t.reg .b64 a, b;\n\t"
-        "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
-        "setp.ne.b32 p, %6, 0;\n\tsetp.ne.b32 e, %7, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}"
-        :: "r"(dcol), "r"(alo), "n"(ahi), "r"(blo), "n"(bhi), "r"(idesc), "n"(ACC ? 1 : 0), "r"(el)
-        : "memory");
-}
-
-// Arrival on an mbarrier once every MMA the lane issued so far has completed.
-__device__ __forceinline__ void tc_commit(unsigned el, unsigned bar)
-{
-    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
-                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
-                 :: "r"(bar), "r"(el) : "memory");
 }
 
 // Weight-stationary column form.  A block takes nb consecutive bricks of one
@@ -759,6 +774,9 @@ k_conv_tma(ConvArgs P, const bf16 *__restrict__ Wtc, int nb, int cols, int NBUF,
         auto wait_all = [&](unsigned bar, unsigned parity) -> bool {
             return __all_sync(0xffffffffu, mbar_wait(bar, parity));
         };
+        auto mma = [&](unsigned d, unsigned a, unsigned b, unsigned id, unsigned acc) {
+            tc_mma_lo<TC_HZ * 16, 8 * 16>(el, d, a, b, id, acc);
+        };
         // slice i of a stage's weights: all of it, or the channel planes and
         // the x tap in use
         int sliced = 0;      // slices whose copies have been issued (in order)
@@ -813,11 +831,11 @@ k_conv_tma(ConvArgs P, const bf16 *__restrict__ Wtc, int nb, int cols, int NBUF,
                         const unsigned a2 = ad0 + (unsigned)((i / 3) * TC_HZ + i % 3 + 2 * s2 * (TMA_PLANE / 16));
                         const unsigned b2 = bw + (unsigned)(i * (SL / 16) + 2 * s2 * 3 * NT);
                         if (i == 0 && s2 == 0 && fresh) {
-                            if (n > 1) tc_mma_lo<true>(el, dcol, a2, b2, tc_idesc(NT * (n - 1)));
-                            tc_mma_lo<false>(el, dcol + (unsigned)((n - 1) * NT), a2,
-                                             b2 + (unsigned)((n - 1) * NT), tc_idesc(NT));
+                            if (n > 1) mma(dcol, a2, b2, tc_idesc(NT * (n - 1)), 1u);
+                            mma(dcol + (unsigned)((n - 1) * NT), a2, b2 + (unsigned)((n - 1) * NT),
+                                tc_idesc(NT), 0u);
                         } else {
-                            tc_mma_lo<true>(el, dcol, a2, b2, idesc);
+                            mma(dcol, a2, b2, idesc, 1u);
                         }
                     }
                     if (leave) tc_commit(el, wfree0 + 8u * (unsigned)i);
@@ -1095,27 +1113,35 @@ __global__ void __launch_bounds__(128) k_wgrad(WgradArgs P)
 // dW[tap][co][ci] = sum over cells v of dZ[v][co] X[v + tap][ci] on the
 // 5th-generation tensor cores, for levels that tile by bricks of 1 x 16 x 8
 // cells.  Per tap this is D[m][n] += sum over cells of P[cell][m] Q[cell][n]
-// (K = cells): one operand gives the 128 rows of D (M, zero channels pad it
-// to 128), the other its N columns.  Both operands sit in shared memory
-// MN-major without swizzle - a core matrix is 8 cells along z (16-byte
-// rows) by 8 channels - so the tiles keep the activations' channels-last
-// layout and nothing is transposed.  The dZ brick is [y][channel group][z][8]
-// and the input's halo [hx][hy][channel group][hz][8], as in the forward
-// kernel, so every tap's operand is the same halo seen from another start
-// address.  Rows are output channels when Cout >= Cin (encoder layers), else
-// a 128-channel tile of the input (decoder layers, whose input is the skip
-// and the doubled coarse tensor).  A block takes a chunk of consecutive
-// bricks and a group of taps whose accumulators fill the tensor memory (512
-// / N taps of N columns); one thread issues each brick's MMAs (8 per tap, K
-// = 16 cells = two z-columns of the brick) once its tiles are staged, and
-// the block writes its partial dW of those taps at the end, summed over the
-// chunks in order afterwards.
-constexpr int WT_KCM = 16;                                   // 128 M channels
-constexpr int WT_DZ_BYTES = TCY * WT_KCM * TCZ * 16;          // 32,768
-constexpr int WT_HALO_BYTES = TC_HX * TC_HY * WT_KCM * TC_HZ * 16;   // 138,240
-// buffer sets (one or two, as they fit) and the barriers in the last 64 bytes
+// (K = cells): one operand gives the 128 rows of D (M), the other its N
+// columns.  Both operands sit in shared memory MN-major without swizzle - a
+// core matrix is 8 cells along z (16-byte rows) by 8 channels - so the tiles
+// keep the activations' channels-last layout and nothing is transposed.  The
+// dZ brick is [y][channel group][z][8], the input's halo [hy][hx][channel
+// group][hz][8]: every tap's operand is the same halo seen from another start
+// address, and the channel groups of the three x taps of a tap pair (b, c)
+// follow one another.  So one MMA serves several x taps: where rows are output
+// channels (Cout >= Cin, encoder layers), its columns are the input channels
+// of all three; where rows are a tile of up to 128 input channels (decoder
+// layers, whose input is the skip and the coarse tensor), they are those of
+// 128 / tile x taps.  Rows past the last channel in use read whatever follows
+// in shared memory; they are never stored.  A block takes a chunk of
+// consecutive bricks and a group of tap pairs whose accumulators fit the
+// tensor memory; warp 8 issues each brick's MMAs (8 per pair and x group, K =
+// 16 cells = two z-columns of the brick), warps 0-7 copy the next bricks
+// meanwhile, and the block writes its partial dW of those taps at the end,
+// summed over the chunks in order afterwards.  Bound by the MMAs (about 74
+// cycles each).  Training step on 64^3 crops, full-resolution layers (32 -> 32
+// and 64 -> 32 channels): 186 and 260 us with one x tap per MMA, one thread of a
+// diverged warp issuing and rows padded with zeros; 61 and 114 us like this.
+constexpr int WT_LOAD = 256;                                 // copying threads
+constexpr int WT_THREADS = WT_LOAD + 32;
+constexpr int WT_OVER = 16 * TC_HZ * 16;                     // rows read past the halo's end
+// buffer sets (one or more, as they fit) and the barriers in the last 128 bytes
 constexpr int WT_SMEM = 227 * 1024;
-static_assert(WT_DZ_BYTES + WT_HALO_BYTES + 1024 <= WT_SMEM, "wgrad smem layout");
+constexpr int WT_MAXBUF = 4;
+static_assert(TCY * 16 * TCZ * 16 + TC_HX * TC_HY * 16 * TC_HZ * 16 + WT_OVER + 2048 <= WT_SMEM,
+              "wgrad smem layout");
 
 struct WgradTcArgs {
     int nx, ny, nz;
@@ -1126,9 +1152,10 @@ struct WgradTcArgs {
     const bf16 *dZ;      // [V][Cout]
     int Cout;
     float *part;         // [chunks][27][Cout][Cin]
-    int rows_co;         // 1: rows of D are output channels; 0: input channels
-    int N;               // columns of D per tap
-    int taps;            // taps per block (tap group)
+    int rows_co;         // 1: rows of D are output channels; 0: input channels (ROWS_CO)
+    int N;               // columns of D per MMA
+    int xper, xm;        // x taps per MMA, MMAs per tap pair
+    int pairs;           // tap pairs (b, c) per block
     int bricks_per_chunk;
     int nbricks;
 };
@@ -1146,7 +1173,8 @@ __device__ __forceinline__ int ilog2(int v)
     return 31 - __clz(v);
 }
 
-__global__ void __launch_bounds__(128, 1) k_wgrad_tc(WgradTcArgs P, int *err)
+template <bool ROWS_CO>
+__global__ void __launch_bounds__(WT_THREADS, 1) k_wgrad_tc(WgradTcArgs P, int *err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
@@ -1155,22 +1183,18 @@ __global__ void __launch_bounds__(128, 1) k_wgrad_tc(WgradTcArgs P, int *err)
     const long long nyz = (long long)P.ny * P.nz;
     const int hy = P.ny >> 1, hz = P.nz >> 1;
     const int chunk = blockIdx.x;
-    const int tap0 = blockIdx.y * P.taps;
-    const int ntap = min(P.taps, 27 - tap0);
-    const int ci0 = P.rows_co ? 0 : blockIdx.z * 128;   // first input channel of the rows
-    // channel groups (8 channels) in the layout and staged: the operand that
-    // gives the 128 rows of D is laid out with 16 groups, the ones past its
-    // channels zero (written once); the other has exactly its channels
-    const int kcz = P.rows_co ? WT_KCM : P.Cout / 8;
-    const int kch = P.rows_co ? Cin / 8 : WT_KCM;
+    const int pair0 = blockIdx.y * P.pairs;
+    const int npair = min(P.pairs, 9 - pair0);
+    const int ci0 = ROWS_CO ? 0 : blockIdx.z * 128;   // first input channel of the rows
+    // channel groups (8 channels) of the dZ brick and of the halo
     const int gz = P.Cout / 8;
-    const int gh = P.rows_co ? Cin / 8 : min(WT_KCM, (Cin - ci0) / 8);
+    const int gh = ROWS_CO ? Cin / 8 : min(16, (Cin - ci0) / 8);
     const int lgz = ilog2(gz), lgh = ilog2(gh);          // both powers of two
-    const int dz_bytes = TCY * kcz * TCZ * 16;
-    const int h_bytes = TC_HX * TC_HY * kch * TC_HZ * 16;
-    const int set_bytes = (dz_bytes + h_bytes + 1023) & ~1023;
-    const int nbuf = 2 * set_bytes + 1024 <= WT_SMEM ? 2 : 1;
-    unsigned long long *mbar = reinterpret_cast<unsigned long long *>(smem + WT_SMEM - 64);
+    const int dz_bytes = TCY * gz * TCZ * 16;
+    const int h_bytes = TC_HX * TC_HY * gh * TC_HZ * 16;
+    const int set_bytes = (dz_bytes + h_bytes + WT_OVER + 1023) & ~1023;
+    const int nbuf = min(WT_MAXBUF, (WT_SMEM - 128) / set_bytes);
+    const unsigned full0 = smem_u32(smem + WT_SMEM - 128), free0 = full0 + 8u * WT_MAXBUF;
     unsigned *tslot = reinterpret_cast<unsigned *>(smem + WT_SMEM - 32);
     int *sfail = reinterpret_cast<int *>(smem + WT_SMEM - 28);
     const int b0 = chunk * P.bricks_per_chunk;
@@ -1178,20 +1202,10 @@ __global__ void __launch_bounds__(128, 1) k_wgrad_tc(WgradTcArgs P, int *err)
     const int nb = b1 - b0;
     if (t == 0) {
         *sfail = 0;
-        for (int q = 0; q < 2; ++q)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(mbar + q)) : "memory");
+        for (int q = 0; q < 2 * WT_MAXBUF; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;"
+                         :: "r"(full0 + 8u * q), "r"(q < WT_MAXBUF ? WT_LOAD / 32 : 1) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    // zero the padding groups of every buffer set once
-    for (int q = 0; q < nbuf; ++q) {
-        uint4 *sz = reinterpret_cast<uint4 *>(smem + q * set_bytes);
-        uint4 *sh = reinterpret_cast<uint4 *>(smem + q * set_bytes + dz_bytes);
-        if (gz < kcz)
-            for (int e = t; e < TCY * kcz * TCZ; e += 128)
-                if (((e / TCZ) % kcz) >= gz) sz[e] = make_uint4(0u, 0u, 0u, 0u);
-        if (gh < kch)
-            for (int e = t; e < TC_HX * TC_HY * kch * TC_HZ; e += 128)
-                if (((e / TC_HZ) % kch) >= gh) sh[e] = make_uint4(0u, 0u, 0u, 0u);
     }
     if (w == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -1202,121 +1216,120 @@ __global__ void __launch_bounds__(128, 1) k_wgrad_tc(WgradTcArgs P, int *err)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned tmem = *tslot;
-    const unsigned idesc = wt_idesc(P.N);
 
-    // stages brick b into buffer set q (cp.async, one group committed)
-    auto stage = [&](int b, int q) {
-        const int bz = b % nzb, by = (b / nzb) % nyb, bx = b / (nzb * nyb);
-        const int i0 = bx, j0 = by * TCY, k0 = bz * TCZ;
-        const unsigned sza = smem_u32(smem + q * set_bytes), sha = sza + (unsigned)dz_bytes;
-        // dZ brick: [y][group][z][8 channels]; item e = ((y * gz) + g) * 8 + z
-        for (int e = t; e < TCY * gz * TCZ; e += 128) {
-            const int z = e & 7, g = (e >> 3) & (gz - 1), y = e >> (3 + lgz);
-            const bf16 *src = P.dZ + ((long long)i0 * nyz + (long long)(j0 + y) * P.nz + k0 + z) *
-                                         P.Cout + g * 8;
-            cp_async16(sza + (unsigned)(((y * kcz + g) * TCZ + z) * 16), src, true);
-        }
-        // halo: [hx][hy][group][hz][8 channels], zero outside the grid;
-        // item e = ((row * gh) + g) * 10 + hz with row = hx * 18 + hy
-        for (int e = t; e < TC_HX * TC_HY * gh * TC_HZ; e += 128) {
-            const int hzz = e % TC_HZ, rest = e / TC_HZ;
-            const int g = rest & (gh - 1), row = rest >> lgh;
-            const int hyy = row % TC_HY, hxx = row / TC_HY;
-            const int ii = i0 + hxx - 1, jj = j0 + hyy - 1, kk = k0 + hzz - 1;
-            const int c = ci0 + g * 8;
-            const bool in = ii >= 0 && ii < P.nx && jj >= 0 && jj < P.ny && kk >= 0 && kk < P.nz;
-            const bf16 *src = P.A;
-            if (in) {
-                if (c < P.Ca)
-                    src = P.A + ((long long)ii * nyz + (long long)jj * P.nz + kk) * P.Ca + c;
-                else
-                    src = P.B + (((long long)(ii >> 1) * hy + (jj >> 1)) * hz + (kk >> 1)) * P.Cb +
-                          (c - P.Ca);
-            }
-            cp_async16(sha + (unsigned)((((row * kch) + g) * TC_HZ + hzz) * 16), src, in);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    // brick j of the chunk uses buffer set j % nbuf; its MMAs commit to
-    // mbarrier j % 2 (the j / 2-th completion of that barrier)
-    auto wait_mma = [&](int j) -> bool {
-        return mbar_wait(smem_u32(mbar + (j & 1)), (unsigned)((j >> 1) & 1));
-    };
-    if (nb > 0) stage(b0, 0);
-    for (int j = 0; j < nb; ++j) {
-        const int q = j % nbuf;
-        if (nbuf == 2) {
-            // the other set is free once brick j - 1's MMAs have completed
-            if (j >= 1 && !wait_mma(j - 1)) {
-                *sfail = 1;
+    // Brick j of the chunk uses set j % nbuf; its MMAs free the set again
+    // (the j / nbuf-th completion of that barrier).
+    if (w < WT_LOAD / 32) {
+        int q = 0;
+        unsigned parity = 1u;          // (a fresh set's wait passes at once)
+        for (int j = 0; j < nb; ++j) {
+            if (!mbar_wait(free0 + 8u * (unsigned)q, parity)) {
                 atomicExch(err, 1);
+                *sfail = 1;
+                break;
             }
-            __syncthreads();
-            if (*sfail) break;
-            if (j + 1 < nb) {
-                stage(b0 + j + 1, (j + 1) % 2);
-                asm volatile("cp.async.wait_group 1;" ::: "memory");
-            } else {
-                asm volatile("cp.async.wait_group 0;" ::: "memory");
-            }
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (t == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int b = b0 + j;
+            const int bz = b % nzb, by = (b / nzb) % nyb, i0 = b / (nzb * nyb);
+            const int j0 = by * TCY, k0 = bz * TCZ;
             const unsigned sza = smem_u32(smem + q * set_bytes), sha = sza + (unsigned)dz_bytes;
-            // MN stride (SBO) between channel groups, K stride (LBO) between
-            // the two z-columns of a K step
-            const unsigned long long dz0 = tc_desc(sza, kcz * TCZ * 16, TCZ * 16);
-            const unsigned long long dh0 = tc_desc(sha, kch * TC_HZ * 16, TC_HZ * 16);
-            for (int jt = 0; jt < ntap; ++jt) {
-                const int tap = tap0 + jt;
-                const int da = tap / 9, db = (tap / 3) % 3, dc = tap % 3;
+            // dZ brick, channel groups fastest (whole cell rows)
+            for (int e = t; e < TCY * TCZ * gz; e += WT_LOAD) {
+                const int g = e & (gz - 1), c = e >> lgz, z = c & 7, y = c >> 3;
+                const bf16 *src = P.dZ + ((long long)i0 * nyz + (long long)(j0 + y) * P.nz + k0 + z) *
+                                             P.Cout + g * 8;
+                cp_async16(sza + (unsigned)(((y * gz + g) * TCZ + z) * 16), src, true);
+            }
+            // halo, channel groups fastest, zero outside the grid; cell c =
+            // (hx * 18 + hy) * 10 + hz
+            for (int e = t; e < TC_HX * TC_HY * TC_HZ * gh; e += WT_LOAD) {
+                const int g = e & (gh - 1), cell = e >> lgh;
+                const int row = cell / TC_HZ, hzz = cell - row * TC_HZ;
+                const int hxx = row / TC_HY, hyy = row - hxx * TC_HY;
+                const int ii = i0 + hxx - 1, jj = j0 + hyy - 1, kk = k0 + hzz - 1;
+                const int c = ci0 + g * 8;
+                const bool in = ii >= 0 && ii < P.nx && jj >= 0 && jj < P.ny && kk >= 0 && kk < P.nz;
+                const bf16 *src = P.A;     // any valid address when nothing is read
+                if (in) {
+                    if (c < P.Ca)
+                        src = P.A + ((long long)ii * nyz + (long long)jj * P.nz + kk) * P.Ca + c;
+                    else
+                        src = P.B + (((long long)(ii >> 1) * hy + (jj >> 1)) * hz + (kk >> 1)) * P.Cb +
+                              (c - P.Ca);
+                }
+                cp_async16(sha + (unsigned)((((hyy * TC_HX + hxx) * gh + g) * TC_HZ + hzz) * 16), src, in);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];"
+                             :: "r"(full0 + 8u * (unsigned)q) : "memory");
+            if (++q == nbuf) {
+                q = 0;
+                parity ^= 1u;
+            }
+        }
+    } else {
+        const unsigned el = elect_lane();
+        const unsigned idesc = wt_idesc(P.N);
+        // MN stride (SBO) between channel groups, K stride (LBO) between the
+        // two z-columns of a K step, in 16-byte units
+        const unsigned zlo = (unsigned)tc_desc(0, gz * TCZ * 16, 0),
+                       hlo = (unsigned)tc_desc(0, TC_HX * gh * TC_HZ * 16, 0);
+        const unsigned zstep = 2u * (unsigned)(gz * TCZ), hstep = 2u * (unsigned)(TC_HX * gh * TC_HZ);
+        const unsigned xstep = (unsigned)(P.xper * gh * TC_HZ);
+        int q = 0;
+        unsigned parity = 0u;
+        bool ok = true;
+        for (int j = 0; j < nb; ++j) {
+            ok = __all_sync(0xffffffffu, mbar_wait(full0 + 8u * (unsigned)q, parity));
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const unsigned sza = smem_u32(smem) + (unsigned)(q * set_bytes);
+            const unsigned zd = zlo + (sza >> 4), hd = hlo + ((sza + (unsigned)dz_bytes) >> 4);
+            unsigned dcol = tmem;
+            const unsigned more = j > 0 ? 1u : 0u;
+            for (int k = 0; k < npair; ++k) {
+                const int pr = pair0 + k, db = pr / 3, dc = pr - 3 * db;
+                for (int x = 0; x < P.xm; ++x) {
+                    const unsigned h0 = hd + (unsigned)(db * TC_HX * gh * TC_HZ + dc) + (unsigned)x * xstep;
 #pragma unroll
-                for (int s2 = 0; s2 < TCY / 2; ++s2) {
-                    // start addresses in 16-byte units
-                    const unsigned long long oz = (unsigned long long)(2 * s2 * kcz * TCZ);
-                    const unsigned long long oh =
-                        (unsigned long long)(((da * TC_HY + 2 * s2 + db) * kch) * TC_HZ + dc);
-                    const unsigned long long ad = P.rows_co ? dz0 + oz : dh0 + oh;
-                    const unsigned long long bd = P.rows_co ? dh0 + oh : dz0 + oz;
-                    const unsigned acc = (j > 0 || s2 > 0) ? 1u : 0u;
-                    tc_mma(tmem + (unsigned)(jt * P.N), ad, bd, idesc, acc);
+                    for (int s2 = 0; s2 < TCY / 2; ++s2) {
+                        const unsigned za = zd + (unsigned)s2 * zstep, ha = h0 + (unsigned)s2 * hstep;
+                        if (ROWS_CO) tc_mma_lo<TCZ * 16, TC_HZ * 16>(el, dcol, za, ha, idesc, s2 > 0 ? 1u : more);
+                        else tc_mma_lo<TC_HZ * 16, TCZ * 16>(el, dcol, ha, za, idesc, s2 > 0 ? 1u : more);
+                    }
+                    dcol += (unsigned)P.N;
                 }
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(smem_u32(mbar + (j & 1))) : "memory");
-        }
-        if (nbuf == 1) {
-            // one buffer set: the next brick's copies wait for these MMAs
-            if (!wait_mma(j)) {
-                *sfail = 1;
-                atomicExch(err, 1);
+            tc_commit(el, free0 + 8u * (unsigned)q);
+            // the last brick's MMAs end the chunk
+            if (j + 1 == nb) {
+                ok = __all_sync(0xffffffffu, mbar_wait(free0 + 8u * (unsigned)q, parity));
+                break;
             }
-            __syncthreads();
-            if (*sfail) break;
-            if (j + 1 < nb) stage(b0 + j + 1, 0);
+            if (++q == nbuf) {
+                q = 0;
+                parity ^= 1u;
+            }
+        }
+        if (!ok && el) {
+            atomicExch(err, 1);
+            *sfail = 1;
         }
     }
-    const bool failed_before = *sfail != 0;
-    __syncthreads();
-    if (!failed_before && nb > 0 && nbuf == 2 && !wait_mma(nb - 1)) {
-        *sfail = 1;
-        atomicExch(err, 1);
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!*sfail && nb > 0) {
+    if (!*sfail && nb > 0 && w < 4) {
         const int m = 32 * w + lane;                    // row of D
-        for (int jt = 0; jt < ntap; ++jt) {
-            const int tap = tap0 + jt;
+        const int rows = 8 * gh, xr = ROWS_CO ? 0 : m / rows;   // input rows of an x tap
+        for (int a = 0; a < npair * P.xm; ++a) {
+            const int pr = pair0 + a / P.xm, x = a % P.xm;
             for (int n0 = 0; n0 < P.N; n0 += 32) {
                 unsigned r[32];
-                const unsigned ta = tmem + ((unsigned)(32 * w) << 16) + (unsigned)(jt * P.N + n0);
+                const unsigned ta = tmem + ((unsigned)(32 * w) << 16) + (unsigned)(a * P.N + n0);
                 asm volatile(
                     "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
                     "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
@@ -1329,20 +1342,26 @@ __global__ void __launch_bounds__(128, 1) k_wgrad_tc(WgradTcArgs P, int *err)
                       "=r"(r[30]), "=r"(r[31])
                     : "r"(ta));
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                float *base = P.part + ((long long)chunk * 27 + tap) * P.Cout * Cin;
-                if (P.rows_co) {
+                if (ROWS_CO) {       // columns: x tap, input channel
+                    const int dx = n0 / Cin, da = x * P.xper + dx, c = n0 - dx * Cin;
                     if (m < P.Cout) {
-                        float4 *d = reinterpret_cast<float4 *>(base + (long long)m * Cin + n0);
+                        float4 *d = reinterpret_cast<float4 *>(
+                            P.part + (((long long)chunk * 27 + da * 9 + pr) * P.Cout + m) * Cin + c);
 #pragma unroll
                         for (int q = 0; q < 8; ++q)
                             d[q] = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
                                                __uint_as_float(r[4 * q + 2]),
                                                __uint_as_float(r[4 * q + 3]));
                     }
-                } else if (ci0 + m < Cin) {
+                } else {               // rows: x tap, input channel
+                    const int da = x * P.xper + xr;
+                    if (da < 3 && xr < P.xper) {
+                        float *base = P.part + ((long long)chunk * 27 + da * 9 + pr) * P.Cout * Cin +
+                                      ci0 + (m - xr * rows);
 #pragma unroll
-                    for (int q = 0; q < 32; ++q)
-                        base[(long long)(n0 + q) * Cin + ci0 + m] = __uint_as_float(r[q]);
+                        for (int q = 0; q < 32; ++q)
+                            base[(long long)(n0 + q) * Cin] = __uint_as_float(r[q]);
+                    }
                 }
             }
         }
@@ -1916,7 +1935,7 @@ bool conv(vesis_net n, int nx, int ny, int nz, const bf16 *A, int Ca, const bf16
     if (n->conv_kind == 1 && ny % TCY == 0 && nz % TCZ == 0 && Ca % 32 == 0 && Cb % 32 == 0 &&
         Cout % 32 == 0) {
         const unsigned bricks = (unsigned)(nx * (ny / TCY) * (nz / TCZ));
-        if (bricks >= 152u * 4u && Wtc) {
+        if (bricks >= 152u * 4u) {
             // enough bricks for weight-stationary blocks of nb bricks along x.
             // A block costs its nb + 2 planes (nb of the folded input layer)
             // and a start and an end worth about three more (6,000 cycles
@@ -1962,12 +1981,12 @@ bool conv(vesis_net n, int nx, int ny, int nz, const bf16 *A, int Ca, const bf16
         }
         if (Cout % 64 == 0) {
             dim3 tg(bricks, Cout / 64);
-            if (raw) k_conv_tc<64, true><<<tg, 128, tc_smem_bytes(64), n->st>>>(a, n->d_err);
-            else k_conv_tc<64, false><<<tg, 128, tc_smem_bytes(64), n->st>>>(a, n->d_err);
+            if (raw) k_conv_tc<64, true><<<tg, 128, tc_smem_bytes(64), n->st>>>(a, Wtc, n->d_err);
+            else k_conv_tc<64, false><<<tg, 128, tc_smem_bytes(64), n->st>>>(a, Wtc, n->d_err);
         } else {
             dim3 tg(bricks, Cout / 32);
-            if (raw) k_conv_tc<32, true><<<tg, 128, tc_smem_bytes(32), n->st>>>(a, n->d_err);
-            else k_conv_tc<32, false><<<tg, 128, tc_smem_bytes(32), n->st>>>(a, n->d_err);
+            if (raw) k_conv_tc<32, true><<<tg, 128, tc_smem_bytes(32), n->st>>>(a, Wtc, n->d_err);
+            else k_conv_tc<32, false><<<tg, 128, tc_smem_bytes(32), n->st>>>(a, Wtc, n->d_err);
         }
         return false;
     }
@@ -2011,19 +2030,29 @@ void wgrad(vesis_net n, int nx, int ny, int nz, const bf16 *A, int Ca, const bf1
         t.Cout = Cout;
         t.part = n->part;
         t.rows_co = Cout >= Cin_ ? 1 : 0;
-        t.N = t.rows_co ? Cin_ : Cout;
-        t.taps = std::min(27, 512 / t.N);
-        const int groups = (27 + t.taps - 1) / t.taps;
         const int mt = t.rows_co ? 1 : (Cin_ + 127) / 128;
+        // x taps per MMA: side by side in the columns (at most 256) or in
+        // the 128 rows
+        t.xper = t.rows_co ? (3 * Cin_ <= 256 ? 3 : 1) : 128 / std::min(128, Cin_);
+        t.N = t.rows_co ? t.xper * Cin_ : Cout;
+        t.xm = (3 + t.xper - 1) / t.xper;
+        const int fit = std::min(9, 512 / (t.N * t.xm));
+        const int groups = (9 + fit - 1) / fit;
+        t.pairs = (9 + groups - 1) / groups;
+        // chunks: one wave of blocks with a group per 512 columns of single
+        // taps (the sums over a chunk, and so the result, depend on its size)
+        const int taps = std::min(27, 512 / (t.rows_co ? Cin_ : Cout));
+        const int waves = (27 + taps - 1) / taps * mt;
         t.nbricks = nx * (ny / TCY) * (nz / TCZ);
-        long long chunks = std::max(1, 152 / (groups * mt));     // one wave
+        long long chunks = std::max(1, 152 / waves);
         chunks = std::min<long long>(chunks, t.nbricks);
         chunks = std::min<long long>(chunks, std::max(1ll, n->part_cap / nw_));
         t.bricks_per_chunk = (int)((t.nbricks + chunks - 1) / chunks);
         chunks = (t.nbricks + t.bricks_per_chunk - 1) / t.bricks_per_chunk;
         count_launch(2);
-        k_wgrad_tc<<<dim3((unsigned)chunks, (unsigned)groups, (unsigned)mt), 128, WT_SMEM,
-                     n->st>>>(t, n->d_err);
+        const dim3 tg((unsigned)chunks, (unsigned)groups, (unsigned)mt);
+        if (t.rows_co) k_wgrad_tc<true><<<tg, WT_THREADS, WT_SMEM, n->st>>>(t, n->d_err);
+        else k_wgrad_tc<false><<<tg, WT_THREADS, WT_SMEM, n->st>>>(t, n->d_err);
         k_sum_parts4<<<nblk(nw_ / 4), 256, 0, n->st>>>(reinterpret_cast<const float4 *>(n->part),
                                                         (int)chunks, nw_ / 4,
                                                         reinterpret_cast<float4 *>(dW));
@@ -2189,7 +2218,9 @@ int vesis_net_create(int n_features, void *cuda_stream, vesis_net *out)
                               tma_smem_bytes(64, TMA_MAXBUF, 2)) != cudaSuccess ||
          cudaFuncSetAttribute(k_conv_tma<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               tma_smem_bytes(64, TMA_MAXBUF, 2)) != cudaSuccess ||
-         cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+         cudaFuncSetAttribute(k_wgrad_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              WT_SMEM) != cudaSuccess ||
+         cudaFuncSetAttribute(k_wgrad_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               WT_SMEM) != cudaSuccess))
         rc = nfail(VESIS_E_CUDA, "shared memory attribute of the tensor-core conv kernel");
     if (rc == VESIS_OK) rc = nalloc(A, &n->d_err, 1);
