@@ -444,11 +444,16 @@ void enq_far(vesis_system s, double *bk)
     }
 }
 
-void enq_fields(vesis_system s, float *U, float *E, double *bk)
+void enq_grid_fields(vesis_system s, float *U, float *E)
 {
     const int sp = span_begin(s);
     enq_pair_energy(s, U, E, s->pe_pts);
     span_end(s, sp, 0, s->G * (long long)s->n, 0);
+}
+
+void enq_fields(vesis_system s, float *U, float *E, double *bk)
+{
+    enq_grid_fields(s, U, E);
     enq_far(s, bk);
 }
 
@@ -457,7 +462,9 @@ void enq_ss(vesis_system s, const double *d_pos, double *bk)
     launch_ss(s->ssplan, d_pos, s->d_sig_ss, s->d_sqeps_ss, s->d_q, s->d_excl,
               s->d_bond_ptr, s->d_bond_other, s->d_bond_k, s->d_bond_r0, s->n,
               s->coul, s->d_ss_part, s->d_ss_gpart, s->st);
-    launch_ss_final(s->d_ss_part, s->nb_ss, bk + S_SSB, s->st);
+    // (energies of bonded terms that do not exist are cleared on the way)
+    launch_ss_final(s->d_ss_part, s->nb_ss, bk + S_SSB, s->bonded.nang > 0 ? nullptr : bk + S_SSA,
+                    s->bonded.ntor > 0 ? nullptr : bk + S_SST, s->st);
     launch_force_reduce(s->d_ss_gpart, s->ssplan.nchunk, s->n, 1.0, s->d_grad_ss,
                         0, s->st);
     launch_bonded(s->bonded, d_pos, s->n, s->d_bonded_part, bk + S_SSA, bk + S_SST,
@@ -1123,8 +1130,9 @@ int vesis_energy_field(vesis_system s, const double *xyz, float *U_dev,
     else enq_pack(s, s->d_xyz);
     float *E = E_dev ? E_dev : s->d_E[0];
     double *bk = bank(s, 0);
-    enq_fields(s, U_dev, E, bk);
+    enq_grid_fields(s, U_dev, E);
     if (chi_dev && terms_out) {
+        enq_far(s, bk);
         enq_ss(s, s->d_xyz, bk);
         enq_terms(s, chi_dev, U_dev, E_dev, bk);
         VTRY(last_launch("energy_field"));

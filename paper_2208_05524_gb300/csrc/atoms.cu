@@ -295,8 +295,13 @@ void launch_ss(const SsPlan &sp, const double *xyz, const double *sig,
 // Sum of the blocks' partials, one warp per term: lane l adds blocks l,
 // l + 32, ... in order, then the lanes' sums are combined by a fixed tree,
 // so the result does not depend on timing.
-__global__ void k_ss_final(const double *__restrict__ e_part, int nb, double *out3)
+__global__ void k_ss_final(const double *__restrict__ e_part, int nb, double *out3, double *zero_a,
+                           double *zero_b)
 {
+    if (threadIdx.x == 0) {
+        if (zero_a) *zero_a = 0.0;
+        if (zero_b) *zero_b = 0.0;
+    }
     const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double t = 0.0;
     for (int b = lane; b < nb; b += 32) t += e_part[3 * b + c];
@@ -305,10 +310,11 @@ __global__ void k_ss_final(const double *__restrict__ e_part, int nb, double *ou
     if (lane == 0) out3[c] = t;
 }
 
-void launch_ss_final(const double *e_part, int nb, double *out3, cudaStream_t st)
+void launch_ss_final(const double *e_part, int nb, double *out3, double *zero_a, double *zero_b,
+                     cudaStream_t st)
 {
     count_launch();
-    k_ss_final<<<1, 96, 0, st>>>(e_part, nb, out3);
+    k_ss_final<<<1, 96, 0, st>>>(e_part, nb, out3, zero_a, zero_b);
 }
 
 // grad = a + b and max |grad component| (non-negative doubles order like
@@ -525,8 +531,8 @@ void launch_bonded(const BondedDev &b, const double *xyz, int n, double *part, d
         count_launch();
         k_bonded_energy<<<(nt + 127) / 128, 128, 0, st>>>(b, xyz, part);
     }
-    launch_sum_doubles(part, b.nang, e_bend, 0, st);
-    launch_sum_doubles(part + b.nang, b.ntor, e_tors, 0, st);
+    if (b.nang > 0) launch_sum_doubles(part, b.nang, e_bend, 0, st);
+    if (b.ntor > 0) launch_sum_doubles(part + b.nang, b.ntor, e_tors, 0, st);
     if (grad && nt > 0) {
         count_launch();
         k_bonded_grad<<<(n + 127) / 128, 128, 0, st>>>(b, xyz, n, grad);

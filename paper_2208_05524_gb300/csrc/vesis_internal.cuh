@@ -273,7 +273,8 @@ void launch_ss(const SsPlan &sp, const double *xyz, const double *sig,
                const int *bond_ptr, const int *bond_other, const double *bond_k,
                const double *bond_r0, int n, double coul, double *e_part,
                double *g_part, cudaStream_t st);
-void launch_ss_final(const double *e_part, int nb, double *out3,
+// Totals of the solute-solute blocks; zero_a, zero_b (may be NULL) are cleared.
+void launch_ss_final(const double *e_part, int nb, double *out3, double *zero_a, double *zero_b,
                      cudaStream_t st);
 // grad = a + b (+ c), and the max |component| into *gmax (FP64 bits).
 void launch_grad_combine(const double *a, const double *b, double *grad,
