@@ -465,7 +465,9 @@ k_pair_force_grid(GridDesc g, long long G, long long chunk_len,
 #pragma unroll
         for (int c = 0; c < 3; ++c) shi[pp][c] = slo[pp][c] = zero2;
 
-    const long long nyz = (long long)g.ny * g.nz;
+    // (cell indexes fit 32 bits: quotients in 64 took 7 % of a small
+    // solute's time, 445 us against 412 at 112^3 cells and 250 atoms)
+    const unsigned nyz = (unsigned)g.ny * (unsigned)g.nz, unz = (unsigned)g.nz;
     unsigned long long seen = 0;
     for (long long s = c0; s < c1; s += PF_STAGE) {
         // stage the solvent cells of [s, s + PF_STAGE) in index order
@@ -476,12 +478,10 @@ k_pair_force_grid(GridDesc g, long long G, long long chunk_len,
             long long idx = s + hlf * PF_THREADS + threadIdx.x;
             v[hlf] = (idx < c1) && chi[idx] == 0;
             if (idx >= c1) idx = s;          // position only feeds the box
-            const int i = (int)(idx / nyz);
-            const long long rem = idx - (long long)i * nyz;
-            const int j = (int)(rem / g.nz);
-            const int k = (int)(rem - (long long)j * g.nz);
-            P[hlf] = make_float4(cell_pos(i, g.cx, g.h), cell_pos(j, g.cy, g.h),
-                                 cell_pos(k, g.cz, g.h), 0.f);
+            const unsigned i = (unsigned)idx / nyz, rem = (unsigned)idx - i * nyz;
+            const unsigned j = rem / unz, k = rem - j * unz;
+            P[hlf] = make_float4(cell_pos((int)i, g.cx, g.h), cell_pos((int)j, g.cy, g.h),
+                                 cell_pos((int)k, g.cz, g.h), 0.f);
             if (v[hlf]) Ev[hlf] = make_float4(Ex[idx], Ey[idx], Ez[idx], 0.f);
         }
         // the stage needs the clamp only if its cells' box comes within r_min
@@ -534,14 +534,16 @@ k_pair_force_grid(GridDesc g, long long G, long long chunk_len,
         for (int pp = 0; pp < PAIRS; ++pp) fx[pp] = fy[pp] = fz[pp] = gx[pp] = gy[pp] = gz[pp] = zero2;
         // the stage's cells by z-pencil: the solvent cells of pencil pen sit
         // at positions [st, en) of the compacted list
-        const long long lim = min((long long)PF_STAGE, c1 - s);
-        const long long pen_end = (s + lim - 1) / g.nz;
-        for (long long pen = s / g.nz; pen <= pen_end; ++pen) {
-            const int st = stage_rank((int)max(pen * g.nz - s, 0LL), s_wc, s_bal);
-            const int en = stage_rank((int)min((pen + 1) * g.nz - s, lim), s_wc, s_bal);
+        const int lim = (int)min((long long)PF_STAGE, c1 - s);
+        unsigned pen = (unsigned)s / unz;
+        // z = 0 of the pencil and of the next one, relative to the stage
+        long long at = (long long)pen * unz - s;
+        for (; at < lim; ++pen, at += unz) {
+            const int st = stage_rank((int)max(at, 0LL), s_wc, s_bal);
+            const int en = stage_rank((int)min(at + unz, (long long)lim), s_wc, s_bal);
             if (st == en) continue;
-            const int i = (int)(pen / g.ny);
-            const int j = (int)(pen - (long long)i * g.ny);
+            const int i = (int)(pen / (unsigned)g.ny);
+            const int j = (int)(pen - (unsigned)i * (unsigned)g.ny);
             const float x = cell_pos(i, g.cx, g.h), y = cell_pos(j, g.cy, g.h);
             const f2 x2 = pk2(x, x), y2 = pk2(y, y);
             f2 dx[PAIRS], dy[PAIRS], dxy2[PAIRS], sc[PAIRS];
