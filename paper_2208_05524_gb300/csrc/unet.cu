@@ -31,6 +31,7 @@ typedef __nv_bfloat16 bf16;
 constexpr int kLevels = 4;
 constexpr int kCh[kLevels] = {32, 64, 128, 128};
 constexpr int kInPad = 32;       // input features padded to 32 channels
+constexpr int kConvLayers = 7;
 
 // ------------------------------------------------------------ mma helpers
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4],
@@ -967,24 +968,6 @@ k_conv_tma(ConvArgs P, const bf16 *__restrict__ Wtc, int nb, int cols, int NBUF,
     }
 }
 
-// Weights [27][Cout][Cin] -> the TMA form's layout: per stage of 32 input
-// channels and tile of NT output channels, [tap (b, c)][8-channel plane]
-// [x tap 2, 1, 0][co][8].
-__global__ void k_pack_tc(const bf16 *__restrict__ W, int Cout, int Cin, int NT,
-                          bf16 *__restrict__ out)
-{
-    const long long n = 27ll * Cout * Cin;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const int tap = (int)(e / ((long long)Cout * Cin));
-    const int co = (int)((e / Cin) % Cout);
-    const int ci = (int)(e % Cin);
-    const int st = ci / 32, kc = (ci % 32) / 8, j = ci % 8;
-    const int nt = co / NT, col = co % NT, nnt = Cout / NT;
-    out[(((((long long)(st * nnt + nt) * 9 + tap % 9) * 4 + kc) * 3 + 2 - tap / 9) * NT + col) * 8 + j] =
-        W[e];
-}
-
 // Weight gradient of a conv3: dW[tap][co][ci] = sum over cells v of
 // dZ[v][co] X[v + tap][ci] (X the concatenated input).  M = co (64 per
 // block), N = ci (32 per block), K = cells in stages of 32, split over
@@ -1552,6 +1535,7 @@ __global__ void __launch_bounds__(256) k_head(const bf16 *__restrict__ D0, long 
 // Head backward: g0[v][c] = Wh[c] dz[v] (FP32); the block's sums of
 // d0[v][c] dz[v] (c < 32) and of dz[v] (entry 32) go to part[block][33]
 // (summed over blocks in order afterwards into dWh and dbh).
+// 16-byte pieces of a cell's row per thread: 57 -> 20 us on 64^3 cells.
 __global__ void __launch_bounds__(256) k_head_bwd(const bf16 *__restrict__ D0, long long V,
                                                   const float *__restrict__ Wh,
                                                   const float *__restrict__ dz,
@@ -1564,10 +1548,23 @@ __global__ void __launch_bounds__(256) k_head_bwd(const bf16 *__restrict__ D0, l
     for (int c = 0; c < 33; ++c) pw[c] = 0.f;
     if (v < V) {
         const float d = dz[v];
+        const uint4 *src = reinterpret_cast<const uint4 *>(D0 + v * 32);
+        float4 *dst = reinterpret_cast<float4 *>(g0 + v * 32);
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-            g0[v * 32 + c] = Wh[c] * d;
-            pw[c] = __bfloat162float(D0[v * 32 + c]) * d;
+        for (int q = 0; q < 4; ++q) {       // eight channels
+            const uint4 r = src[q];
+            const unsigned b[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&b[h]));
+                pw[8 * q + 2 * h] = f.x * d;
+                pw[8 * q + 2 * h + 1] = f.y * d;
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float *wq = Wh + 8 * q + 4 * h;
+                dst[2 * q + h] = make_float4(wq[0] * d, wq[1] * d, wq[2] * d, wq[3] * d);
+            }
         }
         pw[32] = d;
     }
@@ -1589,7 +1586,8 @@ __global__ void __launch_bounds__(256) k_head_bwd(const bf16 *__restrict__ D0, l
 // dZ per channel go to part[block][C] (summed over blocks in order
 // afterwards into db).  C divides 256, so thread t only ever sees channel
 // t % C: it sums its elements in order, then the threads of a channel are
-// added in thread order.
+// added in thread order.  Eight elements' loads are in flight at a time
+// (latency: 75 -> 63 us over a training step on 64^3 cells).
 __global__ void __launch_bounds__(256) k_relu_bwd(const float *__restrict__ gsum,
                                                   const bf16 *__restrict__ y, long long V, int C,
                                                   bf16 *__restrict__ dZ, float *__restrict__ part)
@@ -1597,8 +1595,23 @@ __global__ void __launch_bounds__(256) k_relu_bwd(const float *__restrict__ gsum
     __shared__ float s_db[256];
     const long long n = V * C;
     float acc = 0.f;
-    for (long long e = (long long)blockIdx.x * 256 + threadIdx.x; e < n;
-         e += (long long)gridDim.x * 256) {
+    const long long step = (long long)gridDim.x * 256;
+    long long e = (long long)blockIdx.x * 256 + threadIdx.x;
+    for (; e + 7 * step < n; e += 8 * step) {       // eight elements' loads in flight
+        float yv[8], gv[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            yv[q] = __bfloat162float(y[e + q * step]);
+            gv[q] = gsum[e + q * step];
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const bf16 d = __float2bfloat16(yv[q] > 0.f ? gv[q] : 0.f);
+            dZ[e + q * step] = d;
+            acc += __bfloat162float(d);
+        }
+    }
+    for (; e < n; e += step) {
         const float yv = __bfloat162float(y[e]);
         const bf16 d = __float2bfloat16(yv > 0.f ? gsum[e] : 0.f);
         dZ[e] = d;
@@ -1616,92 +1629,139 @@ __global__ void __launch_bounds__(256) k_relu_bwd(const float *__restrict__ gsum
 // From the input gradient dX [v][Ca + Cb] (FP32) of a decoder conv: the
 // skip part is added into accA [v][Ca]; the coarse part, summed over the
 // 2x2x2 cells that read each coarse cell, is written to gB [u][Cb].
-__global__ void k_split_skip(const float *__restrict__ dX, long long V, int Ca, int Cb,
+__global__ void k_split_skip(const float *__restrict__ dX, int nz, int Ca, int Cb, int qs,
                              float *__restrict__ accA)
 {
-    const long long n = V * Ca;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const long long v = e / Ca;
-    const int c = (int)(e - v * Ca);
-    accA[e] += dX[v * (Ca + Cb) + c];
+    const int item = blockIdx.y * blockDim.x + threadIdx.x, k = item >> qs;
+    if (k >= nz) return;
+    const int c = 4 * (item & ((1 << qs) - 1));
+    const long long v = (long long)blockIdx.x * nz + k;
+    const float4 p = *reinterpret_cast<const float4 *>(dX + v * (Ca + Cb) + c);
+    float4 *d = reinterpret_cast<float4 *>(accA + v * Ca + c);
+    float4 a = *d;
+    a.x += p.x;
+    a.y += p.y;
+    a.z += p.z;
+    a.w += p.w;
+    *d = a;
 }
-
 __global__ void k_split_coarse(const float *__restrict__ dX, int nx, int ny, int nz, int Ca,
-                               int Cb, float *__restrict__ gB)
+                               int Cb, int qs, float *__restrict__ gB)
 {
-    const int hx = nx >> 1, hy = ny >> 1, hz = nz >> 1;
-    const long long n = (long long)hx * hy * hz * Cb;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const long long u = e / Cb;
-    const int c = (int)(e - u * Cb);
-    const int i = (int)(u / ((long long)hy * hz)), j = (int)((u / hz) % hy), k = (int)(u % hz);
-    float s = 0.f;
+    const int hy = ny >> 1, hz = nz >> 1;
+    const int item = blockIdx.y * blockDim.x + threadIdx.x, k = item >> qs;
+    if (k >= hz) return;
+    const int i = blockIdx.x / hy, j = blockIdx.x - i * hy, c = 4 * (item & ((1 << qs) - 1));
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int d = 0; d < 8; ++d) {
         const long long v = ((long long)(2 * i + (d >> 2)) * ny + 2 * j + ((d >> 1) & 1)) * nz +
                             2 * k + (d & 1);
-        s += dX[v * (Ca + Cb) + Ca + c];
+        const float4 p = *reinterpret_cast<const float4 *>(dX + v * (Ca + Cb) + Ca + c);
+        s.x += p.x;
+        s.y += p.y;
+        s.z += p.z;
+        s.w += p.w;
     }
-    gB[e] = s;
+    *reinterpret_cast<float4 *>(gB + (((long long)blockIdx.x) * hz + k) * Cb + c) = s;
 }
 
 // acc[v][c] += dP[parent(v)][c] / 8 (gradient through mean pooling).
-__global__ void k_pool_bwd(const float *__restrict__ dP, int nx, int ny, int nz, int C,
+// Row (i, j) on blockIdx.x, (k, group of 4 channels, C / 4 = 2^qs of them) on
+// blockIdx.y.  (Bound by HBM.  One channel per thread and 64-bit quotients
+// took 66 us over a training step on 64^3 cells, the skip split 42; 20 and 21
+// like this.)
+__global__ void k_pool_bwd(const float *__restrict__ dP, int nx, int ny, int nz, int C, int qs,
                            float *__restrict__ acc)
 {
-    const long long n = (long long)nx * ny * nz * C;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const long long v = e / C;
-    const int c = (int)(e - v * C);
-    const int i = (int)(v / ((long long)ny * nz)), j = (int)((v / nz) % ny), k = (int)(v % nz);
+    const int item = blockIdx.y * blockDim.x + threadIdx.x, k = item >> qs;
+    if (k >= nz) return;
+    const int i = blockIdx.x / ny, j = blockIdx.x - i * ny, c = 4 * (item & ((1 << qs) - 1));
     const long long u = ((long long)(i >> 1) * (ny >> 1) + (j >> 1)) * (nz >> 1) + (k >> 1);
-    acc[e] += 0.125f * dP[u * C + c];
+    const float4 p = *reinterpret_cast<const float4 *>(dP + u * C + c);
+    float4 *d = reinterpret_cast<float4 *>(acc + ((long long)blockIdx.x * nz + k) * C + c);
+    float4 a = *d;
+    a.x += 0.125f * p.x;
+    a.y += 0.125f * p.y;
+    a.z += 0.125f * p.z;
+    a.w += 0.125f * p.w;
+    *d = a;
 }
 
-// Flat FP32 parameters (per layer W[co][ci][3][3][3] then b) -> bf16
-// forward weights Wt[tap][co][cip] and flipped input-gradient weights
-// Wd[tap][ci][co] (cip: ci padded; padded entries zero).  fold: the input
-// carries each cell's x neighbours as channels dx ci_n + ci (dx = 0, 1, 2
-// for x offsets -1, 0, +1), so W[co][ci][dx][b][c] moves to the tap at x
-// offset 0, channel dx ci_n + ci, and the other taps are zero.
-__global__ void k_pack_weights(const float *__restrict__ W, int co_n, int ci_n, int cip,
-                               bool fold, bf16 *__restrict__ Wt, bf16 *__restrict__ Wd)
+// A layer's weights: flat FP32 W[co][ci][3][3][3] and gradient, bf16 forward
+// weights Wt[tap][co][cip] and flipped input-gradient weights Wd[tap][ci][co]
+// (cip: ci padded; padded entries zero), and both again as the tcgen05
+// convolutions read them (tc_weight_at).  fold: the input carries each cell's
+// x neighbours as channels dx ci_n + ci (dx = 0, 1, 2 for x offsets -1, 0,
+// +1), so W[co][ci][dx][b][c] moves to the tap at x offset 0, channel dx ci_n
+// + ci, and the other taps are zero.
+struct LayerWeights {
+    const float *W;
+    bf16 *Wt, *Wd, *Wtc, *Wdc;
+    const float *dW;       // [tap][co][cip]
+    float *g;              // flat gradient
+    int co_n, ci_n, cip, fold;
+};
+struct AllWeights {
+    LayerWeights l[kConvLayers];
+    unsigned first[kConvLayers + 1];     // of the launch's elements
+};
+
+// Place of weight (tap, co, ci) in the tcgen05 form: per stage of 32 input
+// channels and tile of NT output channels, [tap (b, c)][8-channel plane]
+// [x tap 2, 1, 0][co][8].
+__device__ __forceinline__ unsigned tc_weight_at(int tap, int co, int ci, int Cout, int NT)
 {
-    const long long n = 27ll * co_n * cip;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const int tap = (int)(e / ((long long)co_n * cip));
-    const int co = (int)((e / cip) % co_n);
-    const int ci = (int)(e % cip);
+    const int st = ci / 32, kc = (ci % 32) / 8, j = ci % 8;
+    const int nt = co / NT, col = co % NT, nnt = Cout / NT;
+    return (unsigned)((((((st * nnt + nt) * 9 + tap % 9) * 4 + kc) * 3 + 2 - tap / 9) * NT + col) * 8 + j);
+}
+
+__device__ __forceinline__ int layer_of(const AllWeights &A, unsigned e)
+{
+    int l = 0;
+    while (e >= A.first[l + 1]) ++l;
+    return l;
+}
+
+// All layers' weights in one launch (21 took 93 us a training step, this one
+// 21): thread (layer, tap, co, ci).
+__global__ void __launch_bounds__(256) k_pack_weights(const __grid_constant__ AllWeights A)
+{
+    const unsigned t = blockIdx.x * 256u + threadIdx.x;
+    if (t >= A.first[kConvLayers]) return;
+    const int l = layer_of(A, t);
+    const LayerWeights &y = A.l[l];
+    const unsigned e = t - A.first[l], cip = (unsigned)y.cip, con = (unsigned)y.co_n;
+    const int ci = (int)(e % cip), co = (int)((e / cip) % con), tap = (int)(e / (cip * con));
     float w;
-    if (fold) {
-        const int dx = ci / ci_n, f = ci - dx * ci_n;
-        w = tap / 9 == 1 && dx < 3 ? W[((long long)co * ci_n + f) * 27 + dx * 9 + tap % 9] : 0.f;
+    if (y.fold) {
+        const int dx = ci / y.ci_n, f = ci - dx * y.ci_n;
+        w = tap / 9 == 1 && dx < 3 ? y.W[(co * y.ci_n + f) * 27 + dx * 9 + tap % 9] : 0.f;
     } else {
-        w = ci < ci_n ? W[((long long)co * ci_n + ci) * 27 + tap] : 0.f;
+        w = ci < y.ci_n ? y.W[(co * y.ci_n + ci) * 27 + tap] : 0.f;
     }
     const bf16 b = __float2bfloat16(w);
-    Wt[e] = b;
-    if (Wd) Wd[((long long)(26 - tap) * cip + ci) * co_n + co] = b;
+    y.Wt[e] = b;
+    y.Wd[((unsigned)(26 - tap) * cip + (unsigned)ci) * con + (unsigned)co] = b;
+    y.Wtc[tc_weight_at(tap, co, ci, y.co_n, con % 64u == 0u ? 64 : 32)] = b;
+    y.Wdc[tc_weight_at(26 - tap, ci, co, y.cip, cip % 64u == 0u ? 64 : 32)] = b;
 }
 
-// dW[tap][co][cip] (FP32) -> flat gradient order W[co][ci][3][3][3]; with
-// fold (the packing above) W[co][ci][dx][b][c] is the x-offset-0 tap (b, c)
-// at channel dx ci_n + ci.
-__global__ void k_unpack_grad(const float *__restrict__ dW, int co_n, int ci_n, int cip,
-                              bool fold, float *__restrict__ g)
+// dW[tap][co][cip] (FP32) of all layers -> flat gradient order
+// W[co][ci][3][3][3]; with fold (the packing above) W[co][ci][dx][b][c] is the
+// x-offset-0 tap (b, c) at channel dx ci_n + ci.
+__global__ void __launch_bounds__(256) k_unpack_grad(const __grid_constant__ AllWeights A)
 {
-    const long long n = (long long)co_n * ci_n * 27;
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const int tap = (int)(e % 27);
-    const int ci = (int)((e / 27) % ci_n);
-    const int co = (int)(e / (27ll * ci_n));
-    g[e] = fold ? dW[((long long)(9 + tap % 9) * co_n + co) * cip + (tap / 9) * ci_n + ci]
-                : dW[((long long)tap * co_n + co) * cip + ci];
+    const unsigned t = blockIdx.x * 256u + threadIdx.x;
+    if (t >= A.first[kConvLayers]) return;
+    const int l = layer_of(A, t);
+    const LayerWeights &y = A.l[l];
+    const unsigned e = t - A.first[l];
+    const int tap = (int)(e % 27u), ci = (int)((e / 27u) % (unsigned)y.ci_n),
+              co = (int)(e / (27u * (unsigned)y.ci_n));
+    y.g[e] = y.fold ? y.dW[((9 + tap % 9) * y.co_n + co) * y.cip + (tap / 9) * y.ci_n + ci]
+                    : y.dW[(tap * y.co_n + co) * y.cip + ci];
 }
 
 __global__ void k_adam(float *__restrict__ th, const float *__restrict__ g, float *__restrict__ m,
@@ -1768,6 +1828,7 @@ struct Layer {
 int tc_tile(int c) { return c % 64 == 0 ? 64 : 32; }
 
 enum { L_E0, L_E1, L_E2, L_E3, L_D2, L_D1, L_D0, L_HEAD, L_N };
+static_assert(L_HEAD == kConvLayers, "layers before the head");
 
 }  // namespace unet
 }  // namespace vesis
@@ -2129,19 +2190,26 @@ void forward(vesis_net n, const float *x, int NX, int NY, int NZ, int ox, int oy
                                         chi ? n->dz : nullptr, chi ? n->loss_part : nullptr);
 }
 
+// The layers' weights for one launch over all of them; padded: elements count
+// the padded input channels.
+AllWeights all_weights(vesis_net n, bool padded)
+{
+    AllWeights A;
+    A.first[0] = 0;
+    for (int l = 0; l < L_HEAD; ++l) {
+        const Layer &y = n->L[l];
+        A.l[l] = {n->theta + y.w_off, y.Wt,   y.Wd,   y.Wtc, y.Wdc, y.dW, n->grad + y.w_off,
+                  y.co_n,             y.ci_n, y.cip,  l == L_E0 && n->fold};
+        A.first[l + 1] = A.first[l] + 27u * (unsigned)(y.co_n * (padded ? y.cip : y.ci_n));
+    }
+    return A;
+}
+
 int pack_weights(vesis_net n)
 {
-    for (int l = 0; l < L_HEAD; ++l) {
-        Layer &y = n->L[l];
-        count_launch();
-        k_pack_weights<<<nblk(27ll * y.co_n * y.cip), 256, 0, n->st>>>(
-            n->theta + y.w_off, y.co_n, y.ci_n, y.cip, l == L_E0 && n->fold, y.Wt, y.Wd);
-        count_launch(2);
-        k_pack_tc<<<nblk(27ll * y.co_n * y.cip), 256, 0, n->st>>>(y.Wt, y.co_n, y.cip,
-                                                                 tc_tile(y.co_n), y.Wtc);
-        k_pack_tc<<<nblk(27ll * y.co_n * y.cip), 256, 0, n->st>>>(y.Wd, y.cip, y.co_n,
-                                                                 tc_tile(y.cip), y.Wdc);
-    }
+    const AllWeights A = all_weights(n, true);
+    count_launch();
+    k_pack_weights<<<nblk(A.first[kConvLayers]), 256, 0, n->st>>>(A);
     n->packed = true;
     return VESIS_OK;
 }
@@ -2361,12 +2429,6 @@ int vesis_net_loss_grad(vesis_net n, const float *x_dev, const uint8_t *chi_dev,
         k_relu_bwd<<<(unsigned)nb, 256, 0, st>>>(g, y, Vl, C, n->dZ, n->part);
         k_sum_parts_tree<<<C, 256, 0, st>>>(n->part, (int)nb, C, db);
     };
-    auto unpack = [&](int l) {
-        Layer &y = L[l];
-        count_launch();
-        k_unpack_grad<<<nblk(27ll * y.co_n * y.ci_n), 256, 0, st>>>(
-            y.dW, y.co_n, y.ci_n, y.cip, l == L_E0 && n->fold, n->grad + y.w_off);
-    };
     // decoder: d0 (R0), d1 (R1), d2 (R2); skip inputs e0, e1, e2; coarse d1, d2, e3
     struct Dec {
         int l, lev, Ca, Cb, Cout;
@@ -2382,13 +2444,13 @@ int vesis_net_loss_grad(vesis_net n, const float *x_dev, const uint8_t *chi_dev,
         const long long Vl = V[D.lev];
         relu_bwd(D.gout, D.out, Vl, D.Cout, n->grad + L[D.l].b_off);
         wgrad(n, R[0], R[1], R[2], D.skip, D.Ca, D.coarse, D.Cb, n->dZ, D.Cout, L[D.l].dW);
-        unpack(D.l);
         conv(n, R[0], R[1], R[2], n->dZ, D.Cout, nullptr, 0, L[D.l].Wd, L[D.l].Wdc, nullptr,
              D.Ca + D.Cb, n->dX, true);
         count_launch(2);
-        k_split_skip<<<nblk(Vl * D.Ca), 256, 0, st>>>(n->dX, Vl, D.Ca, D.Cb, D.gskip);
-        k_split_coarse<<<nblk(V[D.lev + 1] * D.Cb), 256, 0, st>>>(n->dX, R[0], R[1], R[2], D.Ca,
-                                                                 D.Cb, D.gcoarse);
+        k_split_skip<<<row_grid(R[0], R[1], (long long)R[2] * (D.Ca / 4)), 128, 0, st>>>(
+            n->dX, R[2], D.Ca, D.Cb, log2_groups(2 * D.Ca), D.gskip);
+        k_split_coarse<<<row_grid(R[0] / 2, R[1] / 2, (long long)(R[2] / 2) * (D.Cb / 4)), 128, 0,
+                         st>>>(n->dX, R[0], R[1], R[2], D.Ca, D.Cb, log2_groups(2 * D.Cb), D.gcoarse);
     }
     // encoder: e3 (R3, input p2), e2 (R2, input p1), e1 (R1, input p0), e0 (R0, input X0)
     for (int l = 3; l >= 0; --l) {
@@ -2398,15 +2460,18 @@ int vesis_net_loss_grad(vesis_net n, const float *x_dev, const uint8_t *chi_dev,
         const int Cin = l == 0 ? kInPad : kCh[l - 1];
         relu_bwd(n->ge[l], n->e[l], Vl, kCh[l], n->grad + L[l].b_off);
         wgrad(n, R[0], R[1], R[2], in, Cin, nullptr, 0, n->dZ, kCh[l], L[l].dW);
-        unpack(l);
         if (l > 0) {
             conv(n, R[0], R[1], R[2], n->dZ, kCh[l], nullptr, 0, L[l].Wd, L[l].Wdc, nullptr, Cin,
                  n->dX, true);
             count_launch();
-            k_pool_bwd<<<nblk(V[l - 1] * Cin), 256, 0, st>>>(n->dX, r[l - 1][0], r[l - 1][1],
-                                                             r[l - 1][2], Cin, n->ge[l - 1]);
+            k_pool_bwd<<<row_grid(r[l - 1][0], r[l - 1][1], (long long)r[l - 1][2] * (Cin / 4)), 128,
+                         0, st>>>(n->dX, r[l - 1][0], r[l - 1][1], r[l - 1][2], Cin,
+                                  log2_groups(2 * Cin), n->ge[l - 1]);
         }
     }
+    const AllWeights all = all_weights(n, false);
+    count_launch();
+    k_unpack_grad<<<nblk(all.first[kConvLayers]), 256, 0, st>>>(all);
     launch_sum_doubles(n->loss_part, (int)nblk(V[0]), reinterpret_cast<double *>(n->dz), 0, st);
     NCK(cudaMemcpyAsync(n->h_loss, n->dz, sizeof(double), cudaMemcpyDeviceToHost, st));
     if (grad_host)
