@@ -363,6 +363,10 @@ def run_vesis(args, world, rank, local):
     avg_s = tm["pair_energy_ms"] * 1e-3 / max(1, tm["pair_energy_launches"])
     pairs_per_launch = tm["pair_energy_pairs"] / max(1, tm["pair_energy_launches"])
     achieved = pairs_per_launch * OPS_PER_PAIR / avg_s
+    # Large solutes' pair sums go through node values of tiles of cells (O(cells
+    # + atoms) pair terms): the operations per pair of the direct kernels do not
+    # describe what runs, and the rate of covered pairs passes the FP32 peak.
+    levels = achieved > peak_ops
     sweep = None
     if tm["sweep_ms"] > 0:
         # algorithmic bytes of the cells a round processes: 6 B per cell
@@ -410,6 +414,9 @@ def run_vesis(args, world, rank, local):
                  "traffic": pair_traffic(args.workload, "pair_force_grid"),
                  "ops_per_pair": FORCE_OPS_PER_PAIR,
                  "frac_at_28_ops_per_pair": fpairs * 28 / fs / peak_ops}
+        if fpairs * FORCE_OPS_PER_PAIR / fs > peak_ops:
+            force = by_levels("tree_force_rows + tree_force_nodes", force["ms_per_launch"],
+                              fpairs / fs, peak_ops)
 
     if rank == 0:
         cpu = None
@@ -437,7 +444,10 @@ def run_vesis(args, world, rank, local):
                        "l2": "working set (U, E fields %.0f MB) larger than L2"
                              % (16 * G / 1e6),
                        "parallelism": f"replicas x{world}"},
-            "roofline": {"bound": "alu", "kernel": "pair_energy_grid",
+            "roofline": by_levels("tree_nodes + tree_cells", avg_s * 1e3, pairs_per_launch / avg_s,
+                                  peak_ops, launches=tm["pair_energy_launches"])
+                        if levels else
+                        {"bound": "alu", "kernel": "pair_energy_grid",
                          "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
                          "unit": "Tops/s (FP32 lane-ops)",
                          "frac": achieved / peak_ops,
@@ -461,6 +471,15 @@ def run_vesis(args, world, rank, local):
         }
         print(json.dumps(out), flush=True)
     S.close()
+
+
+def by_levels(kernel, ms, pairs_per_s, peak_ops, **more):
+    """Figures of a pair sum through node values: covered pairs a second, and
+    the fraction of the FP32 lane peak is not stated (its pair terms are not
+    counted per launch)."""
+    return dict({"bound": "alu", "kernel": kernel, "ms_per_launch": ms,
+                 "covered_pairs_per_s": pairs_per_s, "achieved": None, "peak": peak_ops / 1e12,
+                 "unit": "Tops/s (FP32 lane-ops)", "frac": None, "traffic": None}, **more)
 
 
 def run_converge(args, world, rank, local):
