@@ -1145,19 +1145,26 @@ int vesis_energy_field(vesis_system s, const double *xyz, float *U_dev,
     return VESIS_OK;
 }
 
-int vesis_energy_terms(vesis_system s, const uint8_t *chi_dev, const float *U_dev,
-                       const float *E_dev, double *terms_out)
+// Energy terms at the system's positions; w_current: as enq_terms.
+static int energy_terms(vesis_system s, const uint8_t *chi_dev, const float *U_dev,
+                        const float *E_dev, double *terms_out, bool w_current)
 {
-    if (!s || !chi_dev || !U_dev || !terms_out) return fail(VESIS_E_ARG, "NULL argument");
     double *bk = bank(s, 0);
     enq_pack(s, s->d_xyz);
     enq_far(s, bk);
     enq_ss(s, s->d_xyz, bk);
-    enq_terms(s, chi_dev, U_dev, E_dev, bk);
+    enq_terms(s, chi_dev, U_dev, E_dev, bk, w_current);
     VTRY(last_launch("energy_terms"));
     VTRY(read_bank(s, bk));
     fill_terms(s->h_scal, E_dev != nullptr, terms_out);
     return VESIS_OK;
+}
+
+int vesis_energy_terms(vesis_system s, const uint8_t *chi_dev, const float *U_dev,
+                       const float *E_dev, double *terms_out)
+{
+    if (!s || !chi_dev || !U_dev || !terms_out) return fail(VESIS_E_ARG, "NULL argument");
+    return energy_terms(s, chi_dev, U_dev, E_dev, terms_out, false);
 }
 
 int vesis_surface_weights(vesis_system s, const uint8_t *chi_dev, uint32_t *W_dev)
@@ -1193,7 +1200,8 @@ int vesis_blsm_relax(vesis_system s, uint8_t *chi_dev, const float *U_dev,
     if (rounds_out) *rounds_out = rs.round;
     if (flips_out) *flips_out = (long long)rs.total_flips;
     if (dE_sum_out) *dE_sum_out = rs.total_dE;
-    if (terms_out) VTRY(vesis_energy_terms(s, chi_dev, U_dev, E_dev, terms_out));
+    // (the sweep has kept W the exact convolution of the labels)
+    if (terms_out) VTRY(energy_terms(s, chi_dev, U_dev, E_dev, terms_out, true));
     return rs.capped ? VESIS_W_MAX_ROUNDS : VESIS_OK;
 }
 
