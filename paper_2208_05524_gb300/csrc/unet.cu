@@ -17,7 +17,8 @@
 // bfloat16; weights bfloat16 [tap][cout][cin] for the forward pass and
 // [tap][cin][cout] with flipped taps for the input gradient; FP32 master
 // weights, gradients and Adam moments in one flat vector.  The convolutions
-// are implicit GEMMs on the tensor cores (mma.sync m16n8k16, BF16 in, FP32
+// are implicit GEMMs on the tensor cores (tcgen05 where the grid tiles by 16 x
+// 8 cells, mma.sync m16n8k16 elsewhere; BF16 in, FP32
 // accumulate); the rest are plain elementwise and reduction kernels.
 #include <cuda_bf16.h>
 
@@ -67,13 +68,13 @@ struct ConvArgs {
     void *Y;             // bf16 [V][Cout] (relu) or float [V][Cout]
     int k16 = 2;         // halves of each 32-channel stage that hold data (the
                          // input layer's 3 features fill only the first)
-    // 1x1 head fused into a 32-channel layer's epilogue (TMA kernel only):
+    // 1x1 head fused into a 32-channel layer's epilogue (k_conv_tma only):
     // hz[v] = hb + sum_c hw[c] y_c of the BF16-rounded outputs y, which are
     // then not stored
     const float *hw = nullptr, *hb = nullptr;
     float *hz = nullptr;
     // only the taps at x offset 0 hold weights (the input layer with its x
-    // neighbours folded into channels): the TMA kernel skips the others
+    // neighbours folded into channels): k_conv_tma skips the others
     bool x1 = false;
 };
 
@@ -1819,7 +1820,7 @@ struct Layer {
     int ci_n, cip, co_n, k;
     long long w_off, b_off;     // in the flat parameter vector
     bf16 *Wt = nullptr, *Wd = nullptr;
-    bf16 *Wtc = nullptr, *Wdc = nullptr;   // the same in the TMA kernel's layout
+    bf16 *Wtc = nullptr, *Wdc = nullptr;   // the same as the tcgen05 convolutions read them
     float *dW = nullptr;
 };
 
@@ -1969,7 +1970,7 @@ int log2_groups(int C)
 
 // Returns true when the 1x1 head (hw, hb -> hz, a 32-channel layer's
 // outputs) was fused into the convolution, whose outputs were then not
-// stored; only the TMA kernel fuses it.
+// stored; only k_conv_tma fuses it.
 bool conv(vesis_net n, int nx, int ny, int nz, const bf16 *A, int Ca, const bf16 *B, int Cb,
           const bf16 *Wt, const bf16 *Wtc, const float *bias, int Cout, void *Y, bool raw,
           int k16 = 2, const float *hw = nullptr, const float *hb = nullptr, float *hz = nullptr,
