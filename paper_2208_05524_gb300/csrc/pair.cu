@@ -672,6 +672,8 @@ ForcePlan plan_point_force(int np, int natoms, int nsm)
     return fp;
 }
 
+// APT atoms per thread; an atom's sums do not depend on it.
+template <int APT>
 __global__ void __launch_bounds__(PF_THREADS)
 k_point_force(const float4 *__restrict__ pts, const float *__restrict__ wf,
               int np, const float4 *__restrict__ UE, long long chunk_len,
@@ -683,11 +685,11 @@ k_point_force(const float4 *__restrict__ pts, const float *__restrict__ wf,
     const int tile = blockIdx.x;
     const long long c0 = (long long)chunk * chunk_len;
     const long long c1 = min((long long)np, c0 + chunk_len);
-    float ax[PF_APT], ay[PF_APT], az[PF_APT], k1[PF_APT], k2[PF_APT], kq[PF_APT];
-    int an[PF_APT];
+    float ax[APT], ay[APT], az[APT], k1[APT], k2[APT], kq[APT];
+    int an[APT];
 #pragma unroll
-    for (int u = 0; u < PF_APT; ++u) {
-        an[u] = tile * PF_ATOMS + u * PF_THREADS + threadIdx.x;
+    for (int u = 0; u < APT; ++u) {
+        an[u] = tile * PF_THREADS * APT + u * PF_THREADS + threadIdx.x;
         if (an[u] < a.n) {
             const float4 A = a.xyzq[an[u]];
             const float4 F = a.fcoef[an[u]];
@@ -698,9 +700,9 @@ k_point_force(const float4 *__restrict__ pts, const float *__restrict__ wf,
             k1[u] = k2[u] = kq[u] = 0.f;
         }
     }
-    double acc[PF_APT][3];
+    double acc[APT][3];
 #pragma unroll
-    for (int u = 0; u < PF_APT; ++u) acc[u][0] = acc[u][1] = acc[u][2] = 0.0;
+    for (int u = 0; u < APT; ++u) acc[u][0] = acc[u][1] = acc[u][2] = 0.0;
     for (long long s = c0; s < c1; s += PF_STAGE) {
         const int cnt = (int)min((long long)PF_STAGE, c1 - s);
         __syncthreads();
@@ -711,14 +713,15 @@ k_point_force(const float4 *__restrict__ pts, const float *__restrict__ wf,
             s_e[m] = UE[s + m];
         }
         __syncthreads();
-        float f[PF_APT][3];
+        float f[APT][3];
 #pragma unroll
-        for (int u = 0; u < PF_APT; ++u) f[u][0] = f[u][1] = f[u][2] = 0.f;
+        for (int u = 0; u < APT; ++u) f[u][0] = f[u][1] = f[u][2] = 0.f;
+#pragma unroll 4
         for (int p = 0; p < cnt; ++p) {
             const float4 Pp = s_p[p];
             const float4 Ep = s_e[p];
 #pragma unroll
-            for (int u = 0; u < PF_APT; ++u) {
+            for (int u = 0; u < APT; ++u) {
                 float gx = 0.f, gy = 0.f, gz = 0.f;
                 force_pair<true>(Pp.x, Pp.y, Pp.z, Ep, ax[u], ay[u], az[u], k1[u],
                                  k2[u], kq[u], 3.f * kq[u], rmin2, gx, gy, gz);
@@ -728,14 +731,14 @@ k_point_force(const float4 *__restrict__ pts, const float *__restrict__ wf,
             }
         }
 #pragma unroll
-        for (int u = 0; u < PF_APT; ++u) {
+        for (int u = 0; u < APT; ++u) {
             acc[u][0] += (double)f[u][0];
             acc[u][1] += (double)f[u][1];
             acc[u][2] += (double)f[u][2];
         }
     }
 #pragma unroll
-    for (int u = 0; u < PF_APT; ++u) {
+    for (int u = 0; u < APT; ++u) {
         if (an[u] < a.n) {
             double *o = part + ((long long)chunk * a.n + an[u]) * 3;
             o[0] = acc[u][0];
@@ -750,10 +753,17 @@ void launch_point_force(const float4 *pts, const float *wf, int np,
                         const AtomsDev &a, float rmin2, double *part,
                         cudaStream_t st)
 {
-    dim3 grid(fp.atom_tiles, fp.nchunk);
+    // Four atoms per thread amortise the staged points; with few blocks of 512
+    // atoms the chip idles and each thread's chain of 4 x 256 pairs is what
+    // the launch takes: one atom per thread then (12,288 points and 250 atoms:
+    // 47 us in 48 blocks, 16 in 96).
     count_launch();
-    k_point_force<<<grid, PF_THREADS, 0, st>>>(pts, wf, np, UE, fp.chunk_len,
-                                               a, rmin2, part);
+    if ((long long)fp.atom_tiles * fp.nchunk >= 2 * 152)
+        k_point_force<PF_APT><<<dim3(fp.atom_tiles, fp.nchunk), PF_THREADS, 0, st>>>(
+            pts, wf, np, UE, fp.chunk_len, a, rmin2, part);
+    else
+        k_point_force<1><<<dim3((a.n + PF_THREADS - 1) / PF_THREADS, fp.nchunk), PF_THREADS, 0, st>>>(
+            pts, wf, np, UE, fp.chunk_len, a, rmin2, part);
 }
 
 // ------------------------------------------------------ ordered reductions
