@@ -710,6 +710,8 @@ k_conv_tma(ConvArgs P, const bf16 *__restrict__ Wtc, int nb, int cols, int NBUF,
         // pieces of 8 channels, channel plane fastest (64 bytes of a cell)
         constexpr int MP = (180 * 4 + TMA_LOAD - 1) / TMA_LOAD;
         const int nkc = 2 * P.k16, lt = t - 160;
+        // offsets in a plane, in pieces of 8 channels: at most 2^28 cells x 4
+        // pieces fit 32 bits, where elements would not past 2^26 cells
         int offA[MP], offB[MP];
         unsigned dst[MP], in = 0u;
 #pragma unroll
@@ -717,8 +719,8 @@ k_conv_tma(ConvArgs P, const bf16 *__restrict__ Wtc, int nb, int cols, int NBUF,
             const int p = lt + TMA_LOAD * m, kc = p & (nkc - 1), c = p / nkc;
             const int gy = by * TCY - 1 + c / TC_HZ, gz = bz * TCZ - 1 + c % TC_HZ;
             if (gy >= 0 && gz >= 0 && gy < P.ny && gz < P.nz) in |= 1u << m;
-            offA[m] = (gy * P.nz + gz) * P.Ca + 8 * kc;
-            offB[m] = ((gy >> 1) * (P.nz >> 1) + (gz >> 1)) * P.Cb + 8 * kc;
+            offA[m] = (gy * P.nz + gz) * (P.Ca >> 3) + kc;
+            offB[m] = ((gy >> 1) * (P.nz >> 1) + (gz >> 1)) * (P.Cb >> 3) + kc;
             dst[m] = sha0 + (unsigned)(kc * TMA_PLANE + c * 16);
         }
         Slot put{0, 1u}, done{0, 0u};      // (a fresh buffer's wait passes at once)
@@ -748,7 +750,9 @@ k_conv_tma(ConvArgs P, const bf16 *__restrict__ Wtc, int nb, int cols, int NBUF,
             for (int m = 0; m < MP; ++m)
                 if (lt + TMA_LOAD * m < 180 * nkc) {
                     const bool ok = (v >> m) & 1u;
-                    cp_async16(dst[m] + buf, ok ? src + (fine ? offA[m] : offB[m]) : P.A, ok);
+                    cp_async16(dst[m] + buf,
+                               ok ? reinterpret_cast<const uint4 *>(src) + (fine ? offA[m] : offB[m])
+                                  : reinterpret_cast<const uint4 *>(P.A), ok);
                 }
             asm volatile("cp.async.commit_group;" ::: "memory");
             if (u >= lag) {
