@@ -1964,6 +1964,11 @@ dim3 row_grid(int nx, int ny, long long per_row, int t = 128)
     return dim3((unsigned)((long long)nx * ny), (unsigned)((per_row + t - 1) / t));
 }
 
+// Threads per block of the kernels with more items per row than the forward
+// pass's have: 128, or 1024 on rows that 65,535 blocks (the limit of y) of 128
+// would not cover.
+int row_threads(long long per_row) { return per_row > 65535ll * 128 ? 1024 : 128; }
+
 // log2 of the number of 8-channel groups of C channels (C / 8 a power of two).
 int log2_groups(int C)
 {
@@ -2459,9 +2464,10 @@ int vesis_net_loss_grad(vesis_net n, const float *x_dev, const uint8_t *chi_dev,
         conv(n, R[0], R[1], R[2], n->dZ, D.Cout, nullptr, 0, L[D.l].Wd, L[D.l].Wdc, nullptr,
              D.Ca + D.Cb, n->dX, true);
         count_launch(2);
-        k_split_skip<<<row_grid(R[0], R[1], (long long)R[2] * (D.Ca / 4)), 128, 0, st>>>(
+        const long long sk = (long long)R[2] * (D.Ca / 4), co = (long long)(R[2] / 2) * (D.Cb / 4);
+        k_split_skip<<<row_grid(R[0], R[1], sk, row_threads(sk)), row_threads(sk), 0, st>>>(
             n->dX, R[2], D.Ca, D.Cb, log2_groups(2 * D.Ca), D.gskip);
-        k_split_coarse<<<row_grid(R[0] / 2, R[1] / 2, (long long)(R[2] / 2) * (D.Cb / 4)), 128, 0,
+        k_split_coarse<<<row_grid(R[0] / 2, R[1] / 2, co, row_threads(co)), row_threads(co), 0,
                          st>>>(n->dX, R[0], R[1], R[2], D.Ca, D.Cb, log2_groups(2 * D.Cb), D.gcoarse);
     }
     // encoder: e3 (R3, input p2), e2 (R2, input p1), e1 (R1, input p0), e0 (R0, input X0)
@@ -2476,9 +2482,10 @@ int vesis_net_loss_grad(vesis_net n, const float *x_dev, const uint8_t *chi_dev,
             conv(n, R[0], R[1], R[2], n->dZ, kCh[l], nullptr, 0, L[l].Wd, L[l].Wdc, nullptr, Cin,
                  n->dX, true);
             count_launch();
-            k_pool_bwd<<<row_grid(r[l - 1][0], r[l - 1][1], (long long)r[l - 1][2] * (Cin / 4)), 128,
-                         0, st>>>(n->dX, r[l - 1][0], r[l - 1][1], r[l - 1][2], Cin,
-                                  log2_groups(2 * Cin), n->ge[l - 1]);
+            const long long it = (long long)r[l - 1][2] * (Cin / 4);
+            k_pool_bwd<<<row_grid(r[l - 1][0], r[l - 1][1], it, row_threads(it)), row_threads(it), 0,
+                         st>>>(n->dX, r[l - 1][0], r[l - 1][1], r[l - 1][2], Cin, log2_groups(2 * Cin),
+                               n->ge[l - 1]);
         }
     }
     const AllWeights all = all_weights(n, false);

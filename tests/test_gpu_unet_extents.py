@@ -1,5 +1,6 @@
-"""The network on grids with long planes: offsets past 32 bits in elements.
-The element-wise bounds are those of the other network tests."""
+"""The network on grids whose planes or rows are long: offsets past 32 bits in
+elements, and rows of more work items than one launch dimension holds.  The
+element-wise bounds are those of the other network tests."""
 import numpy as np
 import pytest
 
@@ -43,3 +44,26 @@ def test_planes_past_two_gigaelements():
     del x, whole
     torch.cuda.empty_cache()
     _elementwise(got, want, "far corner")
+
+
+def test_training_on_long_rows():
+    """Gradients on 8 x 8 rows of 1,048,640 cells made of two equal halves
+    against those of one half (the loss is a mean; the seam is 1e-4 of the
+    cells)."""
+    _need(80)
+    L = 524320
+    net = _net(1, 42)
+    g = torch.Generator(device="cuda").manual_seed(42)
+    x = torch.randn(8, 8, L, device="cuda", generator=g)
+    y = (x > 0.3).to(torch.uint8)
+    l1, g1 = net.loss_grad(x.reshape(-1), y.reshape(-1), (8, 8, L), grad=True)
+    x2, y2 = torch.cat([x, x], 2).reshape(-1), torch.cat([y, y], 2).reshape(-1)
+    l2, g2 = net.loss_grad(x2, y2, (8, 8, 2 * L), grad=True)
+    net.close()
+    del x, y, x2, y2
+    torch.cuda.empty_cache()
+    assert abs(l1 - l2) <= 1e-3 * abs(l1)
+    a, b = N.unpack(g1.astype(np.float64), 1), N.unpack(g2.astype(np.float64), 1)
+    for k in a:
+        for i in range(2):
+            _elementwise(b[k][i], a[k][i], "%s[%d]" % (k, i))
