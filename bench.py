@@ -360,13 +360,11 @@ def run_vesis(args, world, rank, local):
     f_max = float(pk.get("sm_max_mhz", 2070.0)) * 1e6
     nsm = torch.cuda.get_device_properties(dev).multi_processor_count
     peak_ops = nsm * FP32_LANES_PER_SM * f_max
-    avg_s = tm["pair_energy_ms"] * 1e-3 / max(1, tm["pair_energy_launches"])
-    pairs_per_launch = tm["pair_energy_pairs"] / max(1, tm["pair_energy_launches"])
-    achieved = pairs_per_launch * OPS_PER_PAIR / avg_s
-    # Large solutes' pair sums go through node values of tiles of cells (O(cells
-    # + atoms) pair terms): the operations per pair of the direct kernels do not
-    # describe what runs, and the rate of covered pairs passes the FP32 peak.
-    levels = achieved > peak_ops
+    sums = S.pair_sums()
+    roofline = fields_roofline(tm, sums["fields"], peak_ops,
+                               f"{nsm} SMs x {FP32_LANES_PER_SM} FP32 lanes x "
+                               f"{f_max/1e6:.0f} MHz ({pk_kind} max clock)",
+                               pair_traffic(args.workload))
     sweep = None
     if tm["sweep_ms"] > 0:
         # algorithmic bytes of the cells a round processes: 6 B per cell
@@ -402,21 +400,8 @@ def run_vesis(args, world, rank, local):
                     "peak": pk.get("hbm_gbs"), "unit": "GB/s",
                     "frac": gbs / pk.get("hbm_gbs", 6800.0), "bytes_per_cell": 17,
                     "launches": tm["conv_launches"]}
-    force = None
-    if tm["pair_force_launches"]:
-        fs = tm["pair_force_ms"] * 1e-3 / tm["pair_force_launches"]
-        fpairs = tm["pair_force_pairs"] / tm["pair_force_launches"]
-        force = {"bound": "alu", "kernel": "pair_force_grid",
-                 "ms_per_launch": fs * 1e3, "pairs_per_s": fpairs / fs,
-                 "achieved": fpairs * FORCE_OPS_PER_PAIR / fs / 1e12,
-                 "peak": peak_ops / 1e12, "unit": "Tops/s (FP32 lane-ops)",
-                 "frac": fpairs * FORCE_OPS_PER_PAIR / fs / peak_ops,
-                 "traffic": pair_traffic(args.workload, "pair_force_grid"),
-                 "ops_per_pair": FORCE_OPS_PER_PAIR,
-                 "frac_at_28_ops_per_pair": fpairs * 28 / fs / peak_ops}
-        if fpairs * FORCE_OPS_PER_PAIR / fs > peak_ops:
-            force = by_levels("tree_force_rows + tree_force_nodes", force["ms_per_launch"],
-                              fpairs / fs, peak_ops)
+    force = force_roofline(tm, sums["gradient"], peak_ops,
+                           pair_traffic(args.workload, "pair_force_grid"))
 
     if rank == 0:
         cpu = None
@@ -444,20 +429,7 @@ def run_vesis(args, world, rank, local):
                        "l2": "working set (U, E fields %.0f MB) larger than L2"
                              % (16 * G / 1e6),
                        "parallelism": f"replicas x{world}"},
-            "roofline": by_levels("tree_nodes + tree_cells", avg_s * 1e3, pairs_per_launch / avg_s,
-                                  peak_ops, launches=tm["pair_energy_launches"])
-                        if levels else
-                        {"bound": "alu", "kernel": "pair_energy_grid",
-                         "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
-                         "unit": "Tops/s (FP32 lane-ops)",
-                         "frac": achieved / peak_ops,
-                         "traffic": pair_traffic(args.workload),
-                         "ops_per_pair": OPS_PER_PAIR,
-                         "frac_at_18_ops_per_pair": pairs_per_launch * 18 / avg_s / peak_ops,
-                         "peak_basis": f"{nsm} SMs x {FP32_LANES_PER_SM} FP32 lanes x "
-                                       f"{f_max/1e6:.0f} MHz ({pk_kind} max clock)",
-                         "launches": tm["pair_energy_launches"],
-                         "ms_per_launch": avg_s * 1e3},
+            "roofline": roofline,
             "sweep": sweep, "force": force, "conv": conv,
             "clocks": clocks,
             "e2e": {"value": e2e_value, "unit": "pair-evals/s",
@@ -480,6 +452,39 @@ def by_levels(kernel, ms, pairs_per_s, peak_ops, **more):
     return dict({"bound": "alu", "kernel": kernel, "ms_per_launch": ms,
                  "covered_pairs_per_s": pairs_per_s, "achieved": None, "peak": peak_ops / 1e12,
                  "unit": "Tops/s (FP32 lane-ops)", "frac": None, "traffic": None}, **more)
+
+
+def fields_roofline(tm, sums, peak_ops, basis, traffic):
+    """Figures of the field sums from the timing tm; sums: which kernels ran,
+    as System.pair_sums reports it.  The hierarchical ones do not evaluate
+    every pair, so the direct kernel's operations per pair do not describe
+    them."""
+    launches = tm["pair_energy_launches"]
+    s = tm["pair_energy_ms"] * 1e-3 / max(1, launches)
+    rate = tm["pair_energy_pairs"] / max(1, launches) / s
+    if sums == "hierarchical":
+        return by_levels("tree_nodes + tree_cells", s * 1e3, rate, peak_ops, launches=launches)
+    return {"bound": "alu", "kernel": "pair_energy_grid",
+            "achieved": rate * OPS_PER_PAIR / 1e12, "peak": peak_ops / 1e12,
+            "unit": "Tops/s (FP32 lane-ops)", "frac": rate * OPS_PER_PAIR / peak_ops,
+            "traffic": traffic, "ops_per_pair": OPS_PER_PAIR,
+            "frac_at_18_ops_per_pair": rate * 18 / peak_ops, "peak_basis": basis,
+            "launches": launches, "ms_per_launch": s * 1e3}
+
+
+def force_roofline(tm, sums, peak_ops, traffic):
+    """The same for the grid-to-atom gradient; None if none was timed."""
+    if not tm["pair_force_launches"]:
+        return None
+    s = tm["pair_force_ms"] * 1e-3 / tm["pair_force_launches"]
+    rate = tm["pair_force_pairs"] / tm["pair_force_launches"] / s
+    if sums == "hierarchical":
+        return by_levels("tree_force_rows + tree_force_nodes", s * 1e3, rate, peak_ops)
+    return {"bound": "alu", "kernel": "pair_force_grid", "ms_per_launch": s * 1e3,
+            "pairs_per_s": rate, "achieved": rate * FORCE_OPS_PER_PAIR / 1e12,
+            "peak": peak_ops / 1e12, "unit": "Tops/s (FP32 lane-ops)",
+            "frac": rate * FORCE_OPS_PER_PAIR / peak_ops, "traffic": traffic,
+            "ops_per_pair": FORCE_OPS_PER_PAIR, "frac_at_28_ops_per_pair": rate * 28 / peak_ops}
 
 
 def run_converge(args, world, rank, local):

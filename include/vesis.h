@@ -363,6 +363,12 @@ int vesis_set_state(vesis_system s, const vesis_relax_state *st);
 int vesis_set_tiles(vesis_system s, int energy_pencil, int force_atoms);
 int vesis_get_tiles(vesis_system s, int *energy_pencil, int *force_atoms);
 
+/* Which kernels sum the system's atom-cell pairs, decided at set-up from its
+ * sizes, spacing and radii: *fields and *gradient (either may be NULL)
+ * receive 1 where far pairs are summed at interpolation nodes (hierarchical),
+ * 0 where every pair is summed directly. */
+int vesis_get_pair_sums(vesis_system s, int *fields, int *gradient);
+
 /* Autotuner: times each tile shape of the two pair kernels on the system's
  * current positions and labels chi_dev (one warm-up and `reps` launches
  * each, 1..1000, CUDA events on the system's stream) and keeps the fastest

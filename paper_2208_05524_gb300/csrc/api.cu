@@ -1706,6 +1706,14 @@ int vesis_get_tiles(vesis_system s, int *energy_pencil, int *force_atoms)
     return VESIS_OK;
 }
 
+int vesis_get_pair_sums(vesis_system s, int *fields, int *gradient)
+{
+    if (!s) return fail(VESIS_E_ARG, "NULL system");
+    if (fields) *fields = s->tree;
+    if (gradient) *gradient = s->tree_force;
+    return VESIS_OK;
+}
+
 int vesis_autotune(vesis_system s, const uint8_t *chi_dev, int reps, double *times_ms_out)
 {
     if (!s || !chi_dev) return fail(VESIS_E_ARG, "NULL argument");

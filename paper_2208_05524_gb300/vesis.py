@@ -127,6 +127,7 @@ def lib():
         L.vesis_net_set_conv_kernel.argtypes = [_p, _i]
         L.vesis_net_destroy.argtypes = [_p]
         L.vesis_get_tiles.argtypes = [_p, C.POINTER(_i), C.POINTER(_i)]
+        L.vesis_get_pair_sums.argtypes = [_p, C.POINTER(_i), C.POINTER(_i)]
         L.vesis_autotune.argtypes = [_p, _p, _i, _p]
         L.vesis_relax_batch.argtypes = [_i, _p, _p, _p, C.POINTER(RelaxOpts), _i, _i,
                                         _p, _p]
@@ -387,6 +388,14 @@ class System:
         pe, fa = _i(0), _i(0)
         _check(lib().vesis_get_tiles(self.h, C.byref(pe), C.byref(fa)))
         return pe.value, fa.value
+
+    def pair_sums(self):
+        """Which kernels sum the atom-cell pairs (vesis_get_pair_sums):
+        "hierarchical" or "direct" for the fields and for the gradient."""
+        f, g = _i(0), _i(0)
+        _check(lib().vesis_get_pair_sums(self.h, C.byref(f), C.byref(g)))
+        kind = ("direct", "hierarchical")
+        return dict(fields=kind[f.value], gradient=kind[g.value])
 
     def autotune(self, chi, reps=3):
         """Times the pair kernels' tile shapes on this system and keeps the
