@@ -185,10 +185,10 @@ int vesis_init_labels(vesis_system s, int kind, const double *d,
  *   C = (l_B / 8 pi)(1/eps_w - 1/eps_m),  d = x - r_i,  r = max(|d|, r_min).
  * xyz_or_null: new positions (host, n_atoms x 3) or NULL for the current.
  * U_dev: G floats; E_dev: 3 x G floats (Ex block, Ey block, Ez block) or
- * NULL.  FP32 pair sums; solutes of at least 256 atoms and 2e9 cell-atom pairs
+ * NULL.  FP32 pair sums; solutes of at least 400 atoms and 2e9 cell-atom pairs
  * (spacing permitting) sum near pairs directly and far ones at interpolation
- * nodes, to no larger error than direct sums.  If chi_dev is not NULL and terms_out is not NULL,
- * terms_out[0..5] = surface, vdW, CFA, far field, solute-solute, total
+ * nodes, to no larger rms error than direct sums (vesis_get_pair_sums tells
+ * which).  If chi_dev is not NULL and terms_out is not NULL, terms_out[0..5] = surface, vdW, CFA, far field, solute-solute, total
  * (FP64; vdW and CFA need E_dev). */
 int vesis_energy_field(vesis_system s, const double *xyz_or_null,
                        float *U_dev, float *E_dev, const uint8_t *chi_dev,

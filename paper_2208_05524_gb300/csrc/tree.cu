@@ -221,7 +221,7 @@ TreePlan plan_tree(const GridDesc &g, int n, int nsm)
 
 // Which systems take these kernels: a rule on sizes for each of the two
 // sums.  Measured on both sides of the lines, direct -> hierarchical in us:
-//   fields     N = 256, 200^3 (2.0e9 pairs)     860 ->  516
+//   fields     N = 400, 171^3 (2.0e9 pairs)     860 ->  450
 //              N = 1000, 128^3 (2.1e9)          910 ->  496
 //              N = 3000, 150^3 (1.0e10)        4030 -> 1026
 //   gradient   N = 256, 200^3 (2.0e9)          1876 -> 1992
@@ -229,14 +229,20 @@ TreePlan plan_tree(const GridDesc &g, int n, int nsm)
 //              N = 256, 256^3 (4.3e9)          3470 -> 2345
 //              N = 1000, 160^3 (4.1e9)         2786 -> 1920
 //              N = 3000, 150^3 (1.0e10)        5816 -> 3177
-// Below 256 atoms the direct sums round as little as these (2.6e-7 against
-// 2.8e-7 rms of E at 128 atoms), so those keep them.  Interpolation needs
-// every far pair beyond the clamp and the LJ core resolved (16 h >= 1.2
-// sigma keeps its error below FP32's).
+// Few atoms round little when summed directly: the rms error against 64 bits
+// of the hierarchical fields over the direct ones' (solvent cells, h = 0.3 to
+// 0.5, boxes of 2e9 pairs to 384^3, means of three solutes) is, for U and E,
+// 0.7-0.9 and 0.9-1.0 at 256 atoms but 1.1-1.4 on the half of the cells far from
+// the solute, still up to 1.07 there at 300 and 350, and from 400 atoms on at
+// most 0.87 (1.0 far away).  So solutes of fewer than 400 keep the direct sums.
+// Interpolation needs every far pair beyond the clamp and the LJ core
+// resolved (16 h >= 1.2 sigma keeps its error below FP32's).
+constexpr int kTreeAtoms = 400;
+
 bool tree_fields_pay(const GridDesc &g, int n, double h, double rmin, double max_sigma)
 {
     const double pairs = (double)g.nx * g.ny * g.nz * n;
-    return n >= 256 && pairs >= 2.0e9 && TC * h >= 1.2 * max_sigma && TC * h > rmin;
+    return n >= kTreeAtoms && pairs >= 2.0e9 && TC * h >= 1.2 * max_sigma && TC * h > rmin;
 }
 
 bool tree_force_pays(const GridDesc &g, int n, double h, double rmin, double max_sigma)
