@@ -962,7 +962,9 @@ static int init_impl(vesis_system s, const vesis_params *p, int n,
     long long nch = std::max(s->fplan.nchunk, s->fplan_far.nchunk);
     const double max_sigma = *std::max_element(sigma_sw, sigma_sw + n);
     s->tree = tree_fields_pay(s->g, n, p->h, p->r_min, max_sigma);
-    s->tree_force = tree_force_pays(s->g, n, p->h, p->r_min, max_sigma);
+    double sum_sigma3 = 0.0;
+    for (int i = 0; i < n; ++i) sum_sigma3 += sigma_sw[i] * sigma_sw[i] * sigma_sw[i];
+    s->tree_force = tree_force_pays(s->g, n, p->h, p->r_min, max_sigma, sum_sigma3);
     if (s->tree) {
         s->tplan = plan_tree(s->g, n, s->nsm);
         VTRY(dalloc(s, &s->d_tree, s->tplan.bytes));

@@ -219,16 +219,13 @@ TreePlan plan_tree(const GridDesc &g, int n, int nsm)
     return p;
 }
 
-// Which systems take these kernels: a rule on sizes for each of the two
-// sums.  Measured on both sides of the lines, direct -> hierarchical in us:
-//   fields     N = 400, 171^3 (2.0e9 pairs)     860 ->  450
-//              N = 1000, 128^3 (2.1e9)          910 ->  496
-//              N = 3000, 150^3 (1.0e10)        4030 -> 1026
-//   gradient   N = 256, 200^3 (2.0e9)          1876 -> 1992
-//              N = 700, 144^3 (2.1e9)          1768 -> 1794
-//              N = 256, 256^3 (4.3e9)          3470 -> 2345
-//              N = 1000, 160^3 (4.1e9)         2786 -> 1920
-//              N = 3000, 150^3 (1.0e10)        5816 -> 3177
+// Which systems take these kernels: a rule on sizes, spacing and radii for
+// each of the two sums.  Fields, direct -> hierarchical in us:
+//   N = 400, 171^3 (2.0e9 pairs)     860 ->  450
+//   N = 1000, 128^3 (2.1e9)          910 ->  496
+//   N = 3000, 150^3 (1.0e10)        4030 -> 1026
+// and faster on every shape of box tried at 2e9 pairs and more (1.1 times on 1 x
+// 1500 x 1500 cells, 4 to 7 times on long and flat boxes).
 // Few atoms round little when summed directly: the rms error against 64 bits
 // of the hierarchical fields over the direct ones' (solvent cells, h = 0.3 to
 // 0.5, boxes of 2e9 pairs to 384^3, means of three solutes) is, for U and E,
@@ -245,10 +242,48 @@ bool tree_fields_pay(const GridDesc &g, int n, double h, double rmin, double max
     return n >= kTreeAtoms && pairs >= 2.0e9 && TC * h >= 1.2 * max_sigma && TC * h > rmin;
 }
 
-bool tree_force_pays(const GridDesc &g, int n, double h, double rmin, double max_sigma)
+// The gradient depends on the shape as well: its near part is whole columns of
+// the box, so a long z makes every block's work long, and a box a few columns
+// wide has little else.  Both times are estimated (us; fitted to 80 boxes and
+// solutes, within 15 % on globules):
+//   direct        the pairs with the solvent fraction s of the cells, 1.5e6 a us;
+//   hierarchical  440 + 52 per tile of a column (the chains of blocks that do
+//                 not fill the chip) + 55 per 1e6 cells (gather and merge) + its
+//                 pair terms (rows of the near columns x s, nodes of the others)
+//                 at 1.6e6 a us;
+//   s             exp(-sum sigma^3 / volume): a packed atom and its share of the
+//                 surface take about sigma^3 (globules 0.63-0.99 against 0.50-0.99).
+// Measured, direct -> hierarchical in us (s of the tight start):
+//   N = 256, 200^3, s 0.98         1336 ->  1790     not taken (pairs)
+//   N = 1000, 166^3, 0.77          2392 ->  1994     taken
+//   N = 5000, 184^3, 0.69         14575 ->  4595     taken
+//   N = 2000, 70 x 70 x 925, 0.74  4383 ->  8316     not taken
+//   N = 2000, 925 x 70 x 70, 0.74  4687 ->  1501     taken
+//   N = 700, 65 x 65 x 1400, 0.73  2404 ->  8702     not taken
+//   N = 2000, 90 x 90 x 359, 0.67  2595 ->  3275     not taken
+//   N = 6000, 115 x 115 x 465, 0.59 14481 -> 9997    taken
+//   N = 1000, 17 x 600 x 600, 0.69 3028 ->  4056     not taken
+//   N = 1000, 600 x 600 x 17, 0.69 3522 ->  1346     taken
+// Taken where the estimate is a tenth shorter; never below 4e9 pairs.
+bool tree_force_pays(const GridDesc &g, int n, double h, double rmin, double max_sigma,
+                     double sum_sigma3)
 {
-    const double pairs = (double)g.nx * g.ny * g.nz * n;
-    return pairs >= 4.0e9 && tree_fields_pay(g, n, h, rmin, max_sigma);
+    const double G = (double)g.nx * g.ny * g.nz, pairs = G * n;
+    if (pairs < 4.0e9 || !tree_fields_pay(g, n, h, rmin, max_sigma)) return false;
+    const double s = std::exp(-sum_sigma3 / (G * h * h * h));
+    auto tiles = [](int cells, int lev) { return (cells + (TC << lev) - 1) / (TC << lev); };
+    // tile columns an atom meets at a level: those of the parents' 3 x 3 (level
+    // 2: all) but for its own 3 x 3
+    auto columns = [&](int lev) {
+        const int x = tiles(g.nx, lev), y = tiles(g.ny, lev), w = lev < 2 ? 6 : 1 << 30;
+        return (double)std::min(x, w) * std::min(y, w) - std::min(x, 3) * std::min(y, 3);
+    };
+    double terms = s * std::min(g.nx, 3 * TC) * std::min(g.ny, 3 * TC) * g.nz;
+    for (int lev = 0; lev < 3; ++lev)
+        terms += columns(lev) * tiles(g.nz, lev) * tp(lev) * tp(lev) * tp(lev);
+    const double direct = s * pairs / 1.5e6;
+    const double tree = 440.0 + 52.0 * tiles(g.nz, 0) + 55e-6 * G + n * terms / 1.6e6;
+    return direct > 1.1 * tree;
 }
 
 // ------------------------------------------------------------- sorting

@@ -33,9 +33,10 @@ struct TreePlan {
 
 // Whether a system's fields and its gradient take the hierarchical kernels (a
 // rule on the sizes, the spacing and the LJ radii alone; the gradient's
-// implies the fields').
+// implies the fields').  sum_sigma3: sum of the cubes of the LJ radii.
 bool tree_fields_pay(const GridDesc &g, int n, double h, double rmin, double max_sigma);
-bool tree_force_pays(const GridDesc &g, int n, double h, double rmin, double max_sigma);
+bool tree_force_pays(const GridDesc &g, int n, double h, double rmin, double max_sigma,
+                     double sum_sigma3);
 TreePlan plan_tree(const GridDesc &g, int n, int nsm);
 size_t tree_tab_bytes();
 void tree_fill_tab(void *host);

@@ -29,6 +29,13 @@ def globule(n_atoms, n, h, seed, smax=4.0):
                 h=h, origin=-0.5 * n * h)
 
 
+def spread(n_atoms, n, h, seed):
+    """The same atoms spread evenly over the box."""
+    s = globule(n_atoms, n, h, seed)
+    s["xyz"] = np.random.default_rng(seed).uniform(-0.98, 0.98, (n_atoms, 3)) * -s["origin"]
+    return s
+
+
 def _t(a):
     return torch.as_tensor(np.asarray(a, np.float64), device="cuda")
 
@@ -53,6 +60,28 @@ def fields64(s, idx):
         U.append((4 * p["rho_w"] * ep * (s6 * s6 - s6)).sum(1) +
                  O.cfa_prefactor(p) * e.square().sum(1))
     return torch.cat(U), torch.cat(E)
+
+
+def gradient64(s, chi, E, atoms):
+    """The grid gradient of some atoms in 64 bits, for the given field E [3][G]
+    (Eq. GradientG; clamped pairs keep the r^-3 E part)."""
+    p = O.params()
+    C = O.cfa_prefactor(p)
+    xyz, sg, ep, q = (_t(s[k])[atoms] for k in ("xyz", "sigma_sw", "eps_sw", "q"))
+    A, B = 4 * ep * sg ** 12, 4 * ep * sg ** 6
+    cells = torch.nonzero(chi == 0).flatten()
+    out = torch.zeros(len(atoms), 3, dtype=torch.float64, device="cuda")
+    for a in range(0, len(cells), 1 << 18):
+        c = cells[a:a + (1 << 18)]
+        d = _centres(s, c)[:, None] - xyz[None]
+        r = d.square().sum(-1).sqrt()
+        far = r >= p["rmin"]
+        r = r.clamp_min(p["rmin"])
+        e = E[:, c].double().T
+        cd = p["rho_w"] * (12 * A * r ** -14 - 6 * B * r ** -8) + \
+            6 * C * q * r ** -5 * (d * e[:, None]).sum(-1)
+        out += ((cd * far)[..., None] * d).sum(0) - 2 * C * ((q * r ** -3).T @ e)
+    return out * s["h"] ** 3
 
 
 def fields(s):
@@ -118,3 +147,56 @@ def test_few_atoms_are_summed_directly():
     """Below 400 atoms the direct sums round less far from the solute."""
     for n_atoms, kind in ((256, "direct"), (399, "direct"), (400, "hierarchical")):
         assert fields(globule(n_atoms, (256, 200, 200), 0.4, 1))[2] == kind
+
+
+# globules, and atoms spread over the box: cubes, boxes long in x (narrow
+# columns) and in z (rows of more than two stages of 256 cells), flat boxes
+GRADIENTS = [
+    (globule, 1000, (166, 166, 166), 0.3),
+    (globule, 1200, (700, 100, 110), 0.4),
+    (globule, 2000, (140, 141, 600), 0.4),
+    (spread, 1000, (600, 600, 17), 0.4),
+    (spread, 400, (2048, 2048, 4), 0.4),
+    (spread, 2000, (925, 70, 70), 0.4),
+]
+
+
+@pytest.mark.parametrize("make,n_atoms,n,h", GRADIENTS)
+def test_gradient_rounds_like_direct_sums(make, n_atoms, n, h):
+    """For the same labels and field, the rms error over 64 atoms is at most
+    1.25 times that of the direct kernel on the atoms in parts (both carry the
+    rounding of the FP32 coordinates and of the near rows)."""
+    s = make(n_atoms, n, h, 4)
+    chi, E = tight(s), fields(s)[1]
+    args = dict(far_field=0, eps_ss=1e30)
+    S = vesis.System(s, **args)
+    assert S.pair_sums()["gradient"] == "hierarchical"
+    g = S.atom_forces(chi, E=E.reshape(-1))
+    S.close()
+    gd = np.zeros_like(g)
+    m = -(-n_atoms // 350)
+    for k in range(m):
+        S = vesis.System(synth.subset(s, np.arange(k, n_atoms, m)), **args)
+        assert S.pair_sums()["gradient"] == "direct"
+        gd[k::m] = S.atom_forces(chi, E=E.reshape(-1))
+        S.close()
+    atoms = np.random.default_rng(6).choice(n_atoms, 64, replace=False)
+    ref = gradient64(s, chi, E, torch.as_tensor(atoms, device="cuda")).cpu().numpy()
+    err = np.sqrt(np.mean((g[atoms] - ref) ** 2))
+    assert err <= 1.25 * np.sqrt(np.mean((gd[atoms] - ref) ** 2))
+
+
+@pytest.mark.parametrize("make,n_atoms,n,kind", [
+    (spread, 2000, (70, 70, 925), "direct"),        # 4383 us direct, 8316 by nodes
+    (spread, 2000, (925, 70, 70), "hierarchical"),  # 4687, 1501
+    (spread, 700, (65, 65, 1400), "direct"),        # 2404, 8702
+    (spread, 1000, (17, 600, 600), "direct"),       # 3028, 4056
+    (spread, 1000, (600, 600, 17), "hierarchical"), # 3522, 1346
+    (globule, 1000, (166, 166, 167), "hierarchical"),
+])
+def test_gradient_rule_follows_the_shape(make, n_atoms, n, kind):
+    """Long z and boxes a few columns wide keep the direct gradient; the fields
+    are hierarchical in all of these."""
+    S = vesis.System(make(n_atoms, n, 0.4, 1))
+    assert S.pair_sums() == dict(fields="hierarchical", gradient=kind)
+    S.close()
