@@ -137,6 +137,20 @@ __device__ __forceinline__ void tree_coords(const TreeDims &d, int id, int &x, i
     }
 }
 
+// Tiles of level lev on an axis of n cells, and the place of tile (x, y, z)
+// among the tiles that hold cells (node values are kept for those alone: an id
+// also numbers the slots past the grid's end, up to three of four per axis).
+__host__ __device__ __forceinline__ int axis_tiles(int n, int lev)
+{
+    return (n + (TC << lev) - 1) / (TC << lev);
+}
+
+template <int LEV>
+__device__ __forceinline__ size_t tile_place(const GridDesc &g, int x, int y, int z)
+{
+    return ((size_t)x * axis_tiles(g.ny, LEV) + y) * axis_tiles(g.nz, LEV) + z;
+}
+
 // Cell index of an atom's coordinate on an axis of n cells, clamped into the
 // grid.  One function with fixed roundings: every kernel that asks for an
 // atom's tile has to get the tile it was sorted into.
@@ -176,10 +190,13 @@ TreePlan plan_tree(const GridDesc &g, int n, int nsm)
     p.d = tree_dims(g);
     const long long waves = 16ll * nsm;
     for (int l = 0; l < 3; ++l) {
-        const long long tiles = (long long)p.d.n2 << (3 * (2 - l));
-        const long long per_atom = l == 2 ? p.d.n2 : std::min<long long>(189, tiles);
+        const long long slots = (long long)p.d.n2 << (3 * (2 - l));
+        const long long per_atom = l == 2 ? p.d.n2 : std::min<long long>(189, slots);
+        // tiles that hold cells (slots past the grid's end have no items)
+        const long long tiles =
+            (long long)axis_tiles(g.nx, l) * axis_tiles(g.ny, l) * axis_tiles(g.nz, l);
         TreeList &f = p.list[l], &m = p.list[3 + l];
-        f.tiles = (int)tiles;
+        f.tiles = (int)slots;
         f.len = (int)std::max<long long>(256, (n * per_atom + waves - 1) / waves);
         f.max_items = (int)(tiles + n * per_atom / f.len);
         m.tiles = (p.d.nx * p.d.ny) << (2 * (2 - l));
@@ -211,9 +228,8 @@ TreePlan plan_tree(const GridDesc &g, int n, int nsm)
         l.o_first = take(((size_t)l.tiles + 1) * sizeof(int));
         l.o_item = take((size_t)l.max_items * sizeof(int));
     }
-    for (int l = 0; l < 3; ++l)     // per item (fields) or per tile (gradient)
-        p.o_v[l] = take((size_t)std::max(p.list[l].max_items, p.list[l].tiles) * tn4(l) *
-                        sizeof(float));
+    for (int l = 0; l < 3; ++l)     // per item (fields) or per tile with cells (gradient)
+        p.o_v[l] = take((size_t)p.list[l].max_items * tn4(l) * sizeof(float));
     p.bytes = o;
     p.part_slots = 9 * (kRowParts + kZParts0 + kZParts1) + p.sf;
     return p;
@@ -271,18 +287,17 @@ bool tree_force_pays(const GridDesc &g, int n, double h, double rmin, double max
     const double G = (double)g.nx * g.ny * g.nz, pairs = G * n;
     if (pairs < 4.0e9 || !tree_fields_pay(g, n, h, rmin, max_sigma)) return false;
     const double s = std::exp(-sum_sigma3 / (G * h * h * h));
-    auto tiles = [](int cells, int lev) { return (cells + (TC << lev) - 1) / (TC << lev); };
     // tile columns an atom meets at a level: those of the parents' 3 x 3 (level
     // 2: all) but for its own 3 x 3
     auto columns = [&](int lev) {
-        const int x = tiles(g.nx, lev), y = tiles(g.ny, lev), w = lev < 2 ? 6 : 1 << 30;
+        const int x = axis_tiles(g.nx, lev), y = axis_tiles(g.ny, lev), w = lev < 2 ? 6 : 1 << 30;
         return (double)std::min(x, w) * std::min(y, w) - std::min(x, 3) * std::min(y, 3);
     };
     double terms = s * std::min(g.nx, 3 * TC) * std::min(g.ny, 3 * TC) * g.nz;
     for (int lev = 0; lev < 3; ++lev)
-        terms += columns(lev) * tiles(g.nz, lev) * tp(lev) * tp(lev) * tp(lev);
+        terms += columns(lev) * axis_tiles(g.nz, lev) * tp(lev) * tp(lev) * tp(lev);
     const double direct = s * pairs / 1.5e6;
-    const double tree = 440.0 + 52.0 * tiles(g.nz, 0) + 55e-6 * G + n * terms / 1.6e6;
+    const double tree = 440.0 + 52.0 * axis_tiles(g.nz, 0) + 55e-6 * G + n * terms / 1.6e6;
     return direct > 1.1 * tree;
 }
 
@@ -377,7 +392,7 @@ constexpr int kMaxSeg = 216;            // 27 parents' neighbours x 8 children
 struct SegList {
     int first[kMaxSeg];
     int pre[kMaxSeg + 1];
-    int wsum[8];
+    int nseg;                            // ranges of a level-2 list
 };
 
 // Prefix sums of the ranges seg[0 .. nseg) (counts in pre[0 .. nseg) on
@@ -638,10 +653,10 @@ __device__ __forceinline__ int seg_far(SegList &L, const TreeDims &d, const int 
             }
             L.first[m] = at;
             L.pre[m++] = natoms - at;
-            L.wsum[0] = m;
+            L.nseg = m;
         }
         __syncthreads();
-        nseg = L.wsum[0];
+        nseg = L.nseg;
         return seg_scan(L, nseg);
     }
     constexpr int M = 2 - LEV;
@@ -1145,7 +1160,7 @@ k_tree_gather(GridDesc g, TreeDims d, const TreeTab *__restrict__ tab,
             }
         }
     }
-    float *W = V + (size_t)id * TN4;
+    float *W = V + tile_place<0>(g, x, y, z) * TN4;
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
         const int e = threadIdx.x + 128 * m;
@@ -1190,7 +1205,8 @@ k_tree_merge(GridDesc g, TreeDims d, const TreeTab *__restrict__ tab,
     };
     auto fetch = [&](int o) {
         const bool ok = o < 8 && inside(o);
-        const float *p = Vc + ((size_t)id * 8 + o) * 4 * C3 + (size_t)f * C3;
+        const float *p = Vc + tile_place<LEV - 1>(g, 2 * x + (o >> 2), 2 * y + ((o >> 1) & 1),
+                                                  2 * z + (o & 1)) * 4 * C3 + (size_t)f * C3;
 #pragma unroll
         for (int m = 0; m < NV; ++m) nx[m] = ok && t + 160 * m < C3 ? __ldg(p + t + 160 * m) : 0.f;
     };
@@ -1231,7 +1247,7 @@ k_tree_merge(GridDesc g, TreeDims d, const TreeTab *__restrict__ tab,
         __syncthreads();
     }
     if (t < P2) {
-        float *W = V + (size_t)id * 4 * P3 + (size_t)f * P3;
+        float *W = V + tile_place<LEV>(g, x, y, z) * 4 * P3 + (size_t)f * P3;
 #pragma unroll
         for (int k = 0; k < P; ++k) W[k * P2 + t] = acc[k];
     }
@@ -1710,16 +1726,14 @@ k_tree_force_nodes(GridDesc g, TreeDims d, const TreeTab *__restrict__ tab,
     const int o1 = LEV < 2 ? 4 * (ze - zb) : d.n2;
 #pragma unroll 1
     for (int o = o0; o < o1; o += step) {
-        int id, cx, cy, cz;
+        int cx, cy, cz;
         if (LEV < 2) {
             const int ch = o / nzp;
             cx = 2 * X + (ch >> 1);
             cy = 2 * Y + (ch & 1);
             cz = zb + o - ch * nzp;
-            id = tree_id<LEV>(d, cx, cy, cz);
         } else {
-            id = o;
-            tree_coords<LEV>(d, id, cx, cy, cz);
+            tree_coords<LEV>(d, o, cx, cy, cz);
         }
         if (cx * T >= g.nx || cy * T >= g.ny || cz * T >= g.nz) continue;
         // an atom near the column (or an idle slot) gets zero coefficients
@@ -1754,7 +1768,7 @@ k_tree_force_nodes(GridDesc g, TreeDims d, const TreeTab *__restrict__ tab,
             s_nz[threadIdx.x] = pk2(zz, zz);
         }
         __syncthreads();
-        tile_nodes<P, PAIRS>(V + (size_t)id * tn4(LEV), s_nx, s_ny, s_nz, s_n[w], A, az, c1, c2, kq, hi,
+        tile_nodes<P, PAIRS>(V + tile_place<LEV>(g, cx, cy, cz) * tn4(LEV), s_nx, s_ny, s_nz, s_n[w], A, az, c1, c2, kq, hi,
                       lo);
     }
     store_parts(A, hi, lo, s_acc, a.n, part, [&](int u) {
