@@ -424,8 +424,7 @@ void enq_pair_force(vesis_system s, const ForcePlan &fp, const uint8_t *chi, con
 {
     if (s->tree_force)
         launch_tree_force(s->g, s->tplan, s->d_tree, atoms_view(s), fp.cg, chi, E, E + s->G,
-                          E + 2 * s->G, s->rmin2, s->d_fpart, s->h3, s->d_grad_solv, s->d_fcount,
-                          s->st);
+                          E + 2 * s->G, s->rmin2, s->h3, s->d_grad_solv, s->d_fcount, s->st);
     else
         launch_pair_force_grid(s->g, fp, chi, E, E + s->G, E + 2 * s->G, atoms_view(s), s->rmin2,
                                s->d_fpart, s->d_fcount, s->st);
@@ -959,21 +958,12 @@ static int init_impl(vesis_system s, const vesis_params *p, int n,
     // gradient partials
     s->fplan = plan_pair_force(G, n, s->nsm, 4);
     s->fplan_far = plan_point_force(std::max(1, s->nfar), n, s->nsm);
-    long long nch = std::max(s->fplan.nchunk, s->fplan_far.nchunk);
+    const long long nch = std::max(s->fplan.nchunk, s->fplan_far.nchunk);
     const double max_sigma = *std::max_element(sigma_sw, sigma_sw + n);
     s->tree = tree_fields_pay(s->g, n, p->h, p->r_min, max_sigma);
     double sum_sigma3 = 0.0;
     for (int i = 0; i < n; ++i) sum_sigma3 += sigma_sw[i] * sigma_sw[i] * sigma_sw[i];
     s->tree_force = tree_force_pays(s->g, n, p->h, p->r_min, max_sigma, sum_sigma3);
-    if (s->tree) {
-        s->tplan = plan_tree(s->g, n, s->nsm);
-        VTRY(dalloc(s, &s->d_tree, s->tplan.bytes));
-        std::vector<uint8_t> tab(tree_tab_bytes());
-        tree_fill_tab(tab.data());
-        VCK(cudaMemcpy(s->d_tree + s->tplan.o_tab, tab.data(), tab.size(),
-                       cudaMemcpyHostToDevice));
-        if (s->tree_force) nch = std::max<long long>(nch, s->tplan.part_slots);
-    }
     VTRY(dalloc(s, &s->d_fpart, (size_t)nch * n * 3));
     VTRY(dalloc(s, &s->d_grad_solv, 3 * n));
     VTRY(dalloc(s, &s->d_grad_ss, 3 * n));
@@ -1008,6 +998,20 @@ static int init_impl(vesis_system s, const vesis_params *p, int n,
     VTRY(dalloc(s, &s->d_scal, 2 * S_BANK));
     VTRY(dalloc(s, &s->d_rs, 1));
     VTRY(dalloc(s, &s->d_gd, 1));
+    // last, so that what the direct sums need has its place: without room for
+    // the hierarchical workspace the system keeps the direct sums
+    if (s->tree) {
+        s->tplan = plan_tree(s->g, n, s->nsm, s->tree_force);
+        if (dalloc(s, &s->d_tree, s->tplan.bytes) == VESIS_OK) {
+            std::vector<uint8_t> tab(tree_tab_bytes());
+            tree_fill_tab(tab.data());
+            VCK(cudaMemcpy(s->d_tree + s->tplan.o_tab, tab.data(), tab.size(),
+                           cudaMemcpyHostToDevice));
+        } else {
+            cudaGetLastError();
+            s->tree = s->tree_force = false;
+        }
+    }
     VCK(cudaMemset(s->d_scal, 0, 2 * S_BANK * sizeof(double)));
     VCK(cudaMallocHost(&s->h_scal, S_BANK * sizeof(double)));
     VCK(cudaMallocHost(&s->h_scal2, S_BANK * sizeof(double)));

@@ -184,7 +184,7 @@ TreeDims tree_dims(const GridDesc &g)
 // (fields).  Lists 3-5: the atoms of the 3 x 3 columns around the tile columns
 // of levels 0, 1, 2 (gradient; long lists fill the warps also where a column
 // holds few atoms).
-TreePlan plan_tree(const GridDesc &g, int n, int nsm)
+TreePlan plan_tree(const GridDesc &g, int n, int nsm, bool force)
 {
     TreePlan p;
     p.d = tree_dims(g);
@@ -230,8 +230,10 @@ TreePlan plan_tree(const GridDesc &g, int n, int nsm)
     }
     for (int l = 0; l < 3; ++l)     // per item (fields) or per tile with cells (gradient)
         p.o_v[l] = take((size_t)p.list[l].max_items * tn4(l) * sizeof(float));
+    if (force)                      // FP64 partials per atom
+        p.o_part = take((size_t)(9 * (kRowParts + kZParts0 + kZParts1) + p.sf) * n * 3 *
+                        sizeof(double));
     p.bytes = o;
-    p.part_slots = 9 * (kRowParts + kZParts0 + kZParts1) + p.sf;
     return p;
 }
 
@@ -1812,7 +1814,7 @@ __global__ void k_tree_force_reduce(GridDesc g, const float4 *__restrict__ xyzq,
 
 void launch_tree_force(const GridDesc &g, const TreePlan &p, uint8_t *ws, const AtomsDev &a,
                        int cg, const uint8_t *chi, const float *Ex, const float *Ey,
-                       const float *Ez, float rmin2, double *part, double scale, double *out,
+                       const float *Ez, float rmin2, double scale, double *out,
                        unsigned long long *nsolvent, cudaStream_t st)
 {
     const TreeTab *tab = (const TreeTab *)(ws + p.o_tab);
@@ -1842,6 +1844,7 @@ void launch_tree_force(const GridDesc &g, const TreePlan &p, uint8_t *ws, const 
     k_tree_merge<2><<<dim3(n2, 4), 160, 0, st>>>(g, p.d, tab, V[1], V[2]);
     // pair terms
     const TreeList *l = p.list + 3;
+    double *part = (double *)(ws + p.o_part);
     const size_t block = (size_t)n * 3;
     k_tree_force_rows<<<dim3(l[0].max_items, kRowParts), TF_THREADS, 0, st>>>(
         g, p.d, coff, P.first[0], P.item[0], P.tiles[0], chi, Ex, Ey, Ez, ca, rmin2, cg, part);

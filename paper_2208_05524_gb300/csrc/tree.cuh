@@ -26,9 +26,8 @@ struct TreePlan {
     TreeDims d{};
     TreeList list[6];       // far atoms of levels 0, 1, 2; column atoms of levels 0, 1, 2
     int sf = 1;             // chunks of the level-2 gradient terms
-    int part_slots = 0;     // FP64 gradient partials per atom
     size_t o_tab = 0, o_cnt = 0, o_off = 0, o_cur = 0, o_coff = 0, o_id = 0, o_tmp = 0,
-           o_ord = 0, o_xyzq = 0, o_ab = 0, o_cxyz = 0, o_cfc = 0, o_v[3] = {0, 0, 0}, bytes = 0;
+           o_ord = 0, o_xyzq = 0, o_ab = 0, o_cxyz = 0, o_cfc = 0, o_part = 0, o_v[3] = {0, 0, 0}, bytes = 0;
 };
 
 // Whether a system's fields and its gradient take the hierarchical kernels (a
@@ -37,7 +36,8 @@ struct TreePlan {
 bool tree_fields_pay(const GridDesc &g, int n, double h, double rmin, double max_sigma);
 bool tree_force_pays(const GridDesc &g, int n, double h, double rmin, double max_sigma,
                      double sum_sigma3);
-TreePlan plan_tree(const GridDesc &g, int n, int nsm);
+// force: with the gradient's partials.
+TreePlan plan_tree(const GridDesc &g, int n, int nsm, bool force);
 size_t tree_tab_bytes();
 void tree_fill_tab(void *host);
 // U and E on every cell at the packed atoms.
@@ -45,11 +45,11 @@ void launch_tree_fields(const GridDesc &g, const TreePlan &p, uint8_t *ws, const
                         float rho, float cfa, float rmin2, float *U, float *Ex, float *Ey,
                         float *Ez, cudaStream_t st);
 // out[n][3] = scale x the grid gradient sums of the packed atoms a; cg: the
-// direct kernel's cell groups (plan_pair_force); part: part_slots x n x 3
-// doubles of scratch; the solvent cells are added to *nsolvent.
+// direct kernel's cell groups (plan_pair_force); the solvent cells are added
+// to *nsolvent.
 void launch_tree_force(const GridDesc &g, const TreePlan &p, uint8_t *ws, const AtomsDev &a,
                        int cg, const uint8_t *chi, const float *Ex, const float *Ey,
-                       const float *Ez, float rmin2, double *part, double scale, double *out,
+                       const float *Ez, float rmin2, double scale, double *out,
                        unsigned long long *nsolvent, cudaStream_t st);
 
 }  // namespace vesis

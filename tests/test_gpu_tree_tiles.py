@@ -70,3 +70,40 @@ def test_workspace_of_flat_boxes(n_atoms, n):
     thin = 16 / min(n)
     assert used <= (56 + 1.5 * 6.9 * thin + 32) * S.G + 300e6
     S.close()
+
+
+def test_without_room_for_the_workspace():
+    """A system whose grid fits but whose hierarchical workspace (80 MB here)
+    does not is created all the same and sums directly."""
+    s = spread(1500, (150, 141, 133), 0.4, 2)
+    chi = torch.ones(150 * 141 * 133, dtype=torch.uint8, device="cuda")
+    chi[::3] = 0
+
+    def sums():
+        S = vesis.System(s)
+        U = torch.empty(S.G, dtype=torch.float32, device="cuda")
+        S.energy_field(U)
+        kind = S.pair_sums()
+        g = S.atom_forces(chi)
+        S.close()
+        return kind, U, g
+
+    kind, U, g = sums()
+    assert kind == dict(fields="hierarchical", gradient="hierarchical")
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    a = torch.cuda.mem_get_info()[0]
+    S = vesis.System(s)
+    used = a - torch.cuda.mem_get_info()[0]
+    S.close()
+    # half the workspace is left once the rest (and U) has its place
+    full = torch.empty(a - used - U.nbytes + (40 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        kind, Ud, gd = sums()
+    finally:
+        del full
+        torch.cuda.empty_cache()
+    assert kind == dict(fields="direct", gradient="direct")
+    small = U.abs() < 1.0
+    assert torch.allclose(U[small], Ud[small], rtol=1e-3, atol=1e-5)
+    assert np.abs(g - gd).max() <= 1e-4 * np.abs(g).max()
