@@ -374,7 +374,9 @@ int vesis_get_pair_sums(vesis_system s, int *fields, int *gradient);
  * current positions and labels chi_dev (one warm-up and `reps` launches
  * each, 1..1000, CUDA events on the system's stream) and keeps the fastest
  * (vesis_set_tiles).  times_ms_out (may be NULL): 5 doubles, the mean
- * launch time of energy pencil 4, 8, 16 and gradient atoms 2, 4. */
+ * launch time of energy pencil 4, 8, 16 and gradient atoms 2, 4.  Sums that
+ * are hierarchical (vesis_get_pair_sums) have no shapes: they are timed once,
+ * their times are equal and their shape stays as it was. */
 int vesis_autotune(vesis_system s, const uint8_t *chi_dev, int reps,
                    double *times_ms_out);
 

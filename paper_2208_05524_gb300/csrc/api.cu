@@ -1754,13 +1754,22 @@ int vesis_autotune(vesis_system s, const uint8_t *chi_dev, int reps, double *tim
         *out = (double)t / reps;
         return VESIS_OK;
     };
+    // hierarchical sums have no shapes: timed once, and the shape set stays
     for (int v = 0; v < 3; ++v) {
+        if (s->tree && v > 0) {
+            ms[v] = ms[0];
+            continue;
+        }
         const int P = kPencil[v];
         VTRY(timed([&] {
             enq_pair_energy(s, U, E, P);
         }, &ms[v]));
     }
     for (int v = 0; v < 2; ++v) {
+        if (s->tree_force && v > 0) {
+            ms[3 + v] = ms[3];
+            continue;
+        }
         const ForcePlan fp = plan_pair_force(s->G, s->n, s->nsm, kAtoms[v]);
         VTRY(timed([&] {
             enq_pair_force(s, fp, chi_dev, E);
@@ -1774,7 +1783,8 @@ int vesis_autotune(vesis_system s, const uint8_t *chi_dev, int reps, double *tim
     int best = 1;
     for (int v = 0; v < 3; ++v)
         if (ms[v] < ms[best]) best = v;
-    return vesis_set_tiles(s, kPencil[best], ms[3] < ms[4] ? 2 : 4);
+    return vesis_set_tiles(s, s->tree ? s->pe_pts : kPencil[best],
+                           s->tree_force ? s->fplan.apt : ms[3] < ms[4] ? 2 : 4);
 }
 
 int vesis_relax_batch(int nsys, vesis_system *systems, uint8_t *const *chi_dev,

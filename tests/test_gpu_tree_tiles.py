@@ -107,3 +107,24 @@ def test_without_room_for_the_workspace():
     small = U.abs() < 1.0
     assert torch.allclose(U[small], Ud[small], rtol=1e-3, atol=1e-5)
     assert np.abs(g - gd).max() <= 1e-4 * np.abs(g).max()
+
+
+def test_autotune_leaves_hierarchical_sums_alone():
+    """Nothing to choose: one time for all shapes, and the shapes set before;
+    a gradient below its line is still tuned."""
+    s = spread(1500, (150, 141, 133), 0.4, 2)
+    chi = torch.zeros(150 * 141 * 133, dtype=torch.uint8, device="cuda")
+    S = vesis.System(s)
+    S.set_tiles(16, 2)
+    r = S.autotune(chi, reps=1)
+    ms = r["ms"]
+    assert ms["energy_pencil4"] == ms["energy_pencil8"] == ms["energy_pencil16"] > 0.0
+    assert ms["force_atoms2"] == ms["force_atoms4"] > 0.0
+    assert S.get_tiles() == (16, 2)
+    S.close()
+    S = vesis.System(spread(700, (150, 141, 140), 0.4, 2))
+    assert S.pair_sums() == dict(fields="hierarchical", gradient="direct")
+    ms = S.autotune(torch.zeros(S.G, dtype=torch.uint8, device="cuda"), reps=1)["ms"]
+    assert ms["energy_pencil4"] == ms["energy_pencil8"] == ms["energy_pencil16"] > 0.0
+    assert ms["force_atoms2"] > 0.0 and ms["force_atoms4"] > 0.0
+    S.close()
