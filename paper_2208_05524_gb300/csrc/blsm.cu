@@ -8,6 +8,7 @@
 //
 // This file holds the full-grid passes (convolution, flip energies, energy
 // sums, initial labels); the flip rounds themselves run in sweep.cu.
+#include "row_words.cuh"
 #include "vesis_internal.cuh"
 
 namespace vesis {
@@ -297,11 +298,8 @@ static void launch_walk(const Q17 &w, const TI *in, uint32_t *out, int n_axis, l
 // the chunk and its two neighbours as 8-byte words and applies that row's
 // 2R+1 weights (rows of all-zero weights are skipped, as are zero weights).
 // Bound by integer issue.  WHOLE: rows of whole 8-cell chunks, aligned: three
-// words.  Otherwise the chunk lies anywhere: the up to four aligned words that
-// hold cells of the row are shifted into place and the cells past its ends
-// cleared (a word with a cell of the row lies inside the allocation's last 8
-// bytes).  One thread per cell took 0.45 ms at 2.8 million cells of odd rows,
-// this 0.11 ms.
+// words.  Otherwise the chunk lies anywhere (row_words).  One thread per cell
+// took 0.45 ms at 2.8 million cells of odd rows, this 0.11 ms.
 constexpr int K3MAX = (2 * kMaxR + 1) * (2 * kMaxR + 1) * (2 * kMaxR + 1);
 
 template <bool WHOLE>
@@ -319,9 +317,6 @@ k_conv3_z8(int nx, int ny, int nz, int R, const int *__restrict__ k3,
     const int k0 = (int)(t - row * cpr) * 8;
     const int i = (int)(row / (unsigned)ny), j = (int)(row - (unsigned)i * (unsigned)ny);
     const int n = nz - k0;                 // cells of the row from here on
-    const auto upto = [](int c) {          // the first c bytes of a word
-        return c >= 8 ? ~0ull : c <= 0 ? 0ull : (1ull << (8 * c)) - 1ull;
-    };
     unsigned acc[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
     for (int a = -R; a <= R; ++a) {
         const int ii = i + a;
@@ -334,29 +329,17 @@ k_conv3_z8(int nx, int ny, int nz, int R, const int *__restrict__ k3,
             for (int c = -R; c <= R; ++c) any |= wr[c] != 0;
             if (!any) continue;
             const uint8_t *rp = chi + ((long long)ii * ny + jj) * nz;
-            unsigned long long lo, mid, hi;
+            uint64_t lo, mid, hi;
             if (WHOLE) {
                 lo = k0 >= 8 ? __ldg(reinterpret_cast<const unsigned long long *>(rp + k0 - 8)) : 0ull;
                 mid = __ldg(reinterpret_cast<const unsigned long long *>(rp + k0));
                 hi = n > 8 ? __ldg(reinterpret_cast<const unsigned long long *>(rp + k0 + 8)) : 0ull;
             } else {
-                const int m = (int)((uintptr_t)(rp + k0) & 7u);
-                unsigned long long v[4];     // aligned words from cell k0 - 8 - m on
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int z = k0 - m + 8 * (e - 1);
-                    v[e] = z + 8 > 0 && z < nz
-                               ? __ldg(reinterpret_cast<const unsigned long long *>(rp + z))
-                               : 0ull;
-                }
-                if (m) {
-#pragma unroll
-                    for (int e = 0; e < 3; ++e)
-                        v[e] = (v[e] >> (8 * m)) | (v[e + 1] << (64 - 8 * m));
-                }
-                lo = k0 >= 8 ? v[0] : 0ull;
-                mid = v[1] & upto(n);
-                hi = v[2] & upto(n - 8);
+                row_words(
+                    (uintptr_t)chi, ((unsigned)ii * (unsigned)ny + (unsigned)jj) * (unsigned)nz, k0, nz,
+                    (unsigned)nx * (unsigned)ny * (unsigned)nz,
+                    [](uintptr_t p) { return (uint64_t)__ldg(reinterpret_cast<const unsigned long long *>(p)); },
+                    [](uintptr_t p) { return __ldg(reinterpret_cast<const uint8_t *>(p)); }, lo, mid, hi);
             }
             unsigned by[24];
 #pragma unroll
