@@ -1665,8 +1665,8 @@ __device__ __forceinline__ void tile_nodes(const float *__restrict__ V, const fl
 // tiles of the group's four level-LEV columns (blockIdx.y: which of ZP cuts
 // of the z range, so that small solutes fill the chip); an atom whose own
 // column touches a tile's gets that tile's terms at a lower level (or
-// directly) and takes nothing here.  LEV = 2: block (chunk, y) takes the
-// level-2 tiles chunk, chunk + gridDim.x, ... against 128 atoms.
+// directly) and takes nothing here.  LEV = 2: block (x, chunk) takes the
+// level-2 tiles chunk, chunk + gridDim.y, ... against 128 atoms.
 template <int LEV>
 __global__ void __launch_bounds__(TF_THREADS, 3)
 k_tree_force_nodes(GridDesc g, TreeDims d, const TreeTab *__restrict__ tab,
@@ -1698,7 +1698,7 @@ k_tree_force_nodes(GridDesc g, TreeDims d, const TreeTab *__restrict__ tab,
             L.pre[0] = a.n;
         }
         const int total = seg_scan(L, 1);
-        load_atoms(A, L, 1, a, 128 * blockIdx.y, total);
+        load_atoms(A, L, 1, a, 128 * blockIdx.x, total);
     }
     const f2 zero = pk2(0.f, 0.f);
     const float rh = 1.f / g.h;
@@ -1724,7 +1724,7 @@ k_tree_force_nodes(GridDesc g, TreeDims d, const TreeTab *__restrict__ tab,
     // LEV < 2: the group's four columns, tiles zb .. ze of each
     const int zb = nzt * (int)blockIdx.y / ZP, ze = nzt * ((int)blockIdx.y + 1) / ZP;
     const int nzp = LEV < 2 ? max(1, ze - zb) : 1;
-    const int o0 = LEV < 2 ? 0 : blockIdx.x, step = LEV < 2 ? 1 : gridDim.x;
+    const int o0 = LEV < 2 ? 0 : blockIdx.y, step = LEV < 2 ? 1 : gridDim.y;
     const int o1 = LEV < 2 ? 4 * (ze - zb) : d.n2;
 #pragma unroll 1
     for (int o = o0; o < o1; o += step) {
@@ -1774,7 +1774,7 @@ k_tree_force_nodes(GridDesc g, TreeDims d, const TreeTab *__restrict__ tab,
                       lo);
     }
     store_parts(A, hi, lo, s_acc, a.n, part, [&](int u) {
-        return LEV < 2 ? 9 * (int)blockIdx.y + 8 - A.seg[u] : (int)blockIdx.x;
+        return LEV < 2 ? 9 * (int)blockIdx.y + 8 - A.seg[u] : (int)blockIdx.y;
     });
 }
 
@@ -1855,7 +1855,7 @@ void launch_tree_force(const GridDesc &g, const TreePlan &p, uint8_t *ws, const 
     k_tree_force_nodes<1><<<dim3(l[2].max_items, kZParts1), TF_THREADS, 0, st>>>(
         g, p.d, tab, coff, P.first[2], P.item[2], P.tiles[2], V[1], ca, pn);
     pn += 9 * kZParts1 * block;
-    k_tree_force_nodes<2><<<dim3((unsigned)p.sf, nb), TF_THREADS, 0, st>>>(
+    k_tree_force_nodes<2><<<dim3(nb, (unsigned)p.sf), TF_THREADS, 0, st>>>(
         g, p.d, tab, coff, nullptr, nullptr, 0, V[2], ca, pn);
     k_tree_force_reduce<<<(unsigned)((3 * n + 127) / 128), 128, 0, st>>>(g, ca.xyzq, ord, part, n,
                                                                          p.sf, scale, out);
