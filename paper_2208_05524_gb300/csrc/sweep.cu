@@ -41,7 +41,7 @@
 // The sweep stops when no tile holds a leader or after max_rounds rounds.
 // An opening pass computes every tile's leaders from the starting labels.
 //
-// A round is bound by latency: two grid barriers (1.6 us each) and, in each
+// A round is bound by latency: two grid barriers (1.2 us each alone) and, in each
 // phase, the chain from a tile's loads to its stores, which teams sharing an
 // SM stretch for one another through the instructions they issue.  A half
 // tile per warp keeps a tile's two warps apart but for one barrier: the
@@ -197,9 +197,12 @@ struct Barrier {
 // Barrier of all blocks: number e (1, 2, ...) completes when the counter
 // reaches e * gridDim.x.  Arrival is one release reduction (it orders the
 // block's earlier writes, which bar.sync has made visible to thread 0); the
-// wait polls with acquire loads, back to back (this block alone uses its SM,
-// so nothing is lost to the L1 they invalidate, and no closing acquire is
-// needed).  The poll is bounded (spin_limit polls; 0 gives up at the first
+// wait polls with acquire loads, back to back, and needs no closing acquire.
+// (Alone on its SM a block loses nothing to the L1 lines they invalidate; in a
+// batched relaxation other systems' kernels share the SM, and relaxed polls
+// with a closing acquire or a 32 ns sleep between polls changed batches of 8
+// and 24 systems on 1 to 16 slots by less than 1.5 %, the spread of their runs.)
+// The poll is bounded (spin_limit polls; 0 gives up at the first
 // poll that finds the barrier open) and watches the error flag every 256
 // polls; a timeout raises the flag and the caller returns.  (Spreading the
 // arrivals over 4 or 8 counters, polled by as many lanes, cost 0.1 us a

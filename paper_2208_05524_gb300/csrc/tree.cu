@@ -1,7 +1,6 @@
 // Hierarchical pair sums of the VESIS hot path (sm_103a, FP32 CUDA cores):
 // the fields U, E on the grid (Eq. Ur) and the grid-to-atom gradient (Eq.
-// GradientG) of large solutes, in O(cells + atoms) pair terms instead of
-// cells x atoms.
+// GradientG) of large solutes, in far fewer pair terms than cells x atoms.
 //
 // The grid is cut into cubic tiles of 16, 32 and 64 cells (levels 0, 1, 2).
 // Two tiles of a level are near if they touch (index distance at most 1 per
@@ -27,9 +26,12 @@
 // same for neighbouring cells; that, on the rows within 8 A, makes up nearly
 // all of the direct kernel's rounding error.  With near tiles in three
 // dimensions those small terms went through the nodes and the gradient was
-// nine times closer to 64 bits and 1.3 times faster to sum, but up to 1.2e-9
-// (2-norm) from what the direct kernel gives; with the rows kept whole the
-// two agree to the error of the fields.
+// nine times closer to 64 bits and 1.3 times faster to sum, but further from
+// what the direct kernel gives than the rows allow: with the rows kept whole
+// the two share their largest rounding.  The grid part of the gradient is 0.6
+// to 3.3e-8 (relative 2-norm; 2e-7 on 2048 x 2048 x 4 cells) from the direct
+// kernel's for the same field, and both are equally far from 64 bits (rms ratio
+// 0.97-1.04 over 16 boxes).
 //
 // Accuracy: at 16 cells >= 1.2 sigma the interpolation error (rms over
 // cells, relative to the sum of the terms' magnitudes) of 12 nodes per axis
@@ -41,10 +43,13 @@
 // (tree_fields_pay).  A node's rounding error is shared by all the cells it
 // is interpolated to, so node sums are blocked (128 atoms at a time).
 //
-// Work per atom, fields: 27 x 4096 direct cells and at most 189 x 1728 + 378
-// x 1000 nodes, 0.8e6 pair terms whatever the grid; gradient: 48 x 48 rows
-// and 27 columns of tiles per level, 6e3 pair terms per cell of a row's
-// length.  The direct kernels meet every cell.
+// Work per atom.  Fields: 27 x 4096 direct cells, at most 189 x 1728 nodes of
+// level 0 and 189 x 1000 of level 1 whatever the grid, and 1000 for each of the
+// level-2 tiles not near its own (0.6e6 pair terms and 1/262 of the grid's
+// cells; 0.8e6 at 384^3, 4.7e6 at 1024^3).  Gradient: rows of 48 x 48 cells and
+// 27 columns of level-0 and level-1 tiles, 2304 + 2916 + 844 pair terms per
+// cell of a row's length, and the level-2 tiles outside its 3 x 3 columns as
+// above.  The direct kernels meet every cell.
 #include <algorithm>
 #include <cmath>
 #include <vector>
