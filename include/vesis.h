@@ -367,7 +367,8 @@ int vesis_get_tiles(vesis_system s, int *energy_pencil, int *force_atoms);
  * sizes, spacing and radii: *fields and *gradient (either may be NULL)
  * receive 1 where far pairs are summed at interpolation nodes (hierarchical),
  * 0 where every pair is summed directly (also where the device had no room
- * left for the hierarchical workspace). */
+ * left for the hierarchical workspace; a relaxation resumed in another system
+ * repeats bit for bit where both answer alike). */
 int vesis_get_pair_sums(vesis_system s, int *fields, int *gradient);
 
 /* Autotuner: times each tile shape of the two pair kernels on the system's

@@ -399,7 +399,8 @@ class System:
 
     def autotune(self, chi, reps=3):
         """Times the pair kernels' tile shapes on this system and keeps the
-        fastest; returns the chosen shapes and the four mean times (ms)."""
+        fastest; returns the chosen shapes and the five mean times (ms).  Sums
+        that are hierarchical (pair_sums) keep theirs and report one time."""
         import torch
         t = (_d * 5)()
         _check(lib().vesis_autotune(self.h, _dp(chi, torch.uint8, self.G), int(reps),
